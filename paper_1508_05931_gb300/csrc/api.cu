@@ -54,7 +54,7 @@ struct Workspace {
   u32* fcur = nullptr;         // per bin: next position of the coarse-to-fine split
   u64* wkey = nullptr;         // per region and witness bin: the sample's best witness (follows bcnt)
   int2* sample = nullptr;      // every kSampleStride-th point (K1 or k0 copies them out)
-  PolyTab* poly = nullptr;     // the single-read front's sample polygon (follows wkey)
+  PolyTab* poly = nullptr;     // the single-read front's frame, polygon and candidates
   unsigned long long* key_or = nullptr;
 };
 
@@ -226,7 +226,7 @@ hull_status ensure_ws(hull_ctx* c, size_t n) {
   const size_t o_ctiles = take(((size_t)kCoarse + 1) * 4);
   const size_t o_bcnt = take(((size_t)kBins + kCoarse) * 4);
   const size_t o_wkey = take((size_t)2 * kWitnessBins * 8);   // right after bcnt: one memset clears both
-  const size_t o_poly = take(sizeof(PolyTab));                 // right after wkey: the same memset clears its head
+  const size_t o_poly = take(sizeof(PolyTab));
   const size_t o_sample = take((cap / kSampleStride + 1) * 8);
   const size_t o_bagg = take(((size_t)kBins + kBinPrefixBlocks) * 16);
   const size_t o_bpre = take((size_t)kBins * 16);
@@ -288,25 +288,31 @@ int grid_for(int occ, int num_sms, size_t work_tiles) {
   return (int)g;
 }
 
-// Copies the summary back, synchronises and maps device error bits.  With
-// `fallback`, a bucket sort that met a bin too large for it (ERR_FALLBACK,
-// no other error) sets *fallback and returns HULL_OK without recording
-// anything: the caller reruns the call on the radix passes.
-hull_status read_summary(hull_ctx* c, const Plan& p, bool* fallback);
+// What is left to do after an attempt: nothing, the bucket sort (the star
+// path did not decide: ERR_RETRY) or the radix passes (a bin too large for
+// the bucket sort: ERR_FALLBACK).
+enum Next { NEXT_NONE = 0, NEXT_BUCKET, NEXT_RADIX };
 
-hull_status finish(hull_ctx* c, cudaStream_t st, bool* fallback = nullptr) {
+// Copies the summary back, synchronises and maps device error bits.  With
+// `next`, an attempt that did not decide (and met no other error) sets *next
+// and returns HULL_OK without recording anything: the caller goes on.
+hull_status read_summary(hull_ctx* c, const Plan& p, Next* next);
+
+hull_status finish(hull_ctx* c, cudaStream_t st, Next* next = nullptr) {
   cudaError_t e = cudaMemcpyAsync(c->h_plan, c->plan, kSummaryBytes, cudaMemcpyDeviceToHost, st);
   if (e != cudaSuccess) return cuda_fail(e);
   e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_fail(e);
-  return read_summary(c, *c->h_plan, fallback);
+  return read_summary(c, *c->h_plan, next);
 }
 
 // The bookkeeping of finish() for one call's summary `p` (already on the host).
-hull_status read_summary(hull_ctx* c, const Plan& p, bool* fallback) {
-  if (fallback) {
-    *fallback = (p.error & ERR_FALLBACK) != 0 && (p.error & (ERR_RANGE | ERR_TIMEOUT)) == 0;
-    if (*fallback) return HULL_OK;
+hull_status read_summary(hull_ctx* c, const Plan& p, Next* next) {
+  if (next) {
+    *next = NEXT_NONE;
+    if ((p.error & (ERR_RANGE | ERR_TIMEOUT)) == 0)
+      *next = (p.error & ERR_RETRY) ? NEXT_BUCKET : (p.error & ERR_FALLBACK) ? NEXT_RADIX : NEXT_NONE;
+    if (*next != NEXT_NONE) return HULL_OK;
   }
   if (c->prof_pending) {
     c->prof_pending = false;
@@ -347,42 +353,66 @@ void mark(hull_ctx* c, int k, cudaStream_t st) {
   if (c->prof_pending) cudaEventRecord(c->ev[k], st);
 }
 
-// Inputs from this size up (16-byte aligned, no statistics asked for) take
-// the single-read front on the bucket-sort path.
-constexpr u32 kSingleReadMin = 1u << 16;
+// Inputs of more points than one block takes (kSmallMax) use the single-read front.
+bool single_read(u32 n) { return n >= kSmallMax; }
+
+// The star path decides the hulls only: no statistics of the paper's steps,
+// no mirrored round, no learned polygon on the small inputs that would have
+// met it.
+bool star_eligible(const hull_ctx* c, u32 n) {
+  return !c->cfg.collect_stats && !c->cfg.reverse_round &&
+         (single_read(n) || !(c->cfg.proposal == 1 && c->have_weights));
+}
+
+// The star path: the frame and the sample polygon, the pass over the input
+// that drops the points strictly inside it and writes the rest (raw
+// survivors, 0.3 % of a uniform 20M disk) to the chain buffers, and the hull
+// of those; a small input in one launch.  Ends with the summary in the Plan.
+// Profile slots: 0 sample polygon, 1 the pass, 11 the hull.
+hull_status run_star(hull_ctx* c, const int32_t* d_xy, u32 n, int32_t* d_out, int64_t cap, cudaStream_t st) {
+  Workspace& w = c->ws;
+  mark(c, 0, st);
+  cudaError_t e = cudaSuccess;
+  if (single_read(n)) {
+    u32* ridx = reinterpret_cast<u32*>(w.h_idx[0]);
+    e = cudaMemsetAsync(w.poly, 0, kPolyClearBytes, st);
+    if (e == cudaSuccess) e = launch_poly(d_xy, n, w.poly, c->num_sms, st);
+    mark(c, 1, st);
+    if (e == cudaSuccess) e = launch_k1_poly(d_xy, n, w.poly, w.h_xy[0], ridx, c->num_sms, st);
+    for (int p = 2; p <= 3 + kMaxPasses; ++p) mark(c, p, st);
+    if (e == cudaSuccess)
+      e = launch_star(d_xy, n, w.poly, w.h_xy[0], ridx, w.h_xy[1], reinterpret_cast<u32*>(w.h_idx[1]), c->plan, d_out,
+                      (long long)cap, c->num_sms, st);
+  } else {
+    for (int p = 1; p <= 3 + kMaxPasses; ++p) mark(c, p, st);
+    e = launch_small(d_xy, n, c->plan, d_out, (long long)cap, st);
+  }
+  mark(c, 4 + kMaxPasses, st);
+  return e == cudaSuccess ? HULL_OK : cuda_fail(e);
+}
 
 // K1 .. K4 of the pipeline on d_xy (n >= 1).  `bucket` selects the bucket
 // sort (K2 scatters the survivors into bins, one block sorts each group of
 // bins); otherwise K2 compacts them in index order for the radix passes.
-// `exact_lists`: the region lists must be exactly Figure 2's on every
-// first-round survivor (the two-read front; the single-read front's lists
-// are Figure 2's on a subset of them, which keeps every hull vertex).
+// `single`: the star path left its raw survivors in the chain buffers (free
+// until the group sort); the front goes on from those.  Its region lists are
+// Figure 2's on a subset of the first-round survivors, which keeps every
+// hull vertex; without it they are exactly Figure 2's on all of them (the
+// two-read front).
 hull_status run_front(hull_ctx* c, const int32_t* d_xy, u32 n, cudaStream_t st, bool bucket,
-                      bool exact_lists = false) {
+                      bool single = false) {
   Workspace& w = c->ws;
-  const bool single = bucket && !exact_lists && !c->cfg.collect_stats && n >= kSingleReadMin &&
-                      (reinterpret_cast<uintptr_t>(d_xy) & 15u) == 0;
   const size_t clear_bytes = (reinterpret_cast<char*>(w.wkey) - reinterpret_cast<char*>(w.bcnt)) +
-                             (size_t)2 * kWitnessBins * sizeof(u64) + kPolyClearBytes;
+                             (size_t)2 * kWitnessBins * sizeof(u64);
   mark(c, 0, st);
   cudaError_t e = cudaSuccess;
-  if (single) {
-    // The single-read front: the sample polygon (from every 1024th point),
-    // then one pass for the extremes that drops the points strictly inside
-    // that polygon and writes the rest (raw survivors, ~0.1-1 % of a uniform
-    // input) to the chain buffers, free until the group sort; the raw
-    // survivors are also the witnesses' candidates.
-    e = cudaMemsetAsync(w.bcnt, 0, clear_bytes, st);
-    if (e == cudaSuccess) e = launch_poly(d_xy, n, w.poly, c->num_sms, st);
-    mark(c, 1, st);
-    if (e == cudaSuccess)
-      e = launch_k1_poly(d_xy, n, c->cfg.spin_limit, c->plan, w.partials, w.poly, &w.poly->raw_count, w.h_xy[0],
-                         reinterpret_cast<u32*>(w.h_idx[0]), c->num_sms, st);
-  } else {
-    if (bucket) mark(c, 1, st);     // no sample polygon: an empty stage
+  if (bucket) mark(c, 1, st);       // the sample polygon's slot: an empty stage
+  if (single)
+    e = launch_k1_raw(w.h_xy[0], reinterpret_cast<const u32*>(w.h_idx[0]), n, c->cfg.spin_limit, c->plan, w.partials,
+                      w.poly, c->num_sms, st);
+  else
     e = launch_k1(d_xy, n, c->cfg.spin_limit, c->plan, w.partials, k1_grid(n, c->num_sms), st,
                   bucket ? w.sample : nullptr);
-  }
   if (e != cudaSuccess) return cuda_fail(e);
   if (c->cfg.proposal == 1 && c->have_weights && !single) {
     // Learned filter polygon: sampled features, MLP, exact hull of the
@@ -408,7 +438,7 @@ hull_status run_front(hull_ctx* c, const int32_t* d_xy, u32 n, cudaStream_t st, 
     // (the fused filter and its bin scan), 4 scatter (coarse bins), 5 split
     // (fine bins, their aggregates, group prefixes), 6 sort (+ second
     // round), 7..9 empty, 10 compaction.
-    if (!single) e = cudaMemsetAsync(w.bcnt, 0, clear_bytes, st);
+    e = cudaMemsetAsync(w.bcnt, 0, clear_bytes, st);
     // Witnesses: on the single-read front from every raw survivor (the
     // points nearest the hull, a small fraction of the input), else from
     // the every-32nd-point sample.
@@ -490,6 +520,37 @@ hull_status run_final(hull_ctx* c, const int2* lo_xy, const int* lo_idx, const i
   if (e != cudaSuccess) return cuda_fail(e);
   mark(c, 4 + kMaxPasses, st);
   return HULL_OK;
+}
+
+// One hull from a given step on: the star path, the bucket sort (on the raw
+// survivors that the star path left in this workspace, FROM_RAW), the radix
+// passes.  Each goes on to the next when it does not decide: the star path
+// on lists beyond one block and degenerate inputs, the bucket sort on a bin
+// it cannot sort in shared memory (heavily duplicated or extremely
+// clustered input); the radix passes take any input.
+enum From { FROM_STAR = 0, FROM_RAW, FROM_BUCKET, FROM_RADIX };
+
+hull_status compute_from(hull_ctx* c, const int32_t* d_xy, u32 n, int32_t* d_out, int64_t cap, int64_t* h_count,
+                         cudaStream_t st, From from) {
+  hull_status r = HULL_OK;
+  for (;;) {
+    Next next = NEXT_NONE;
+    c->prof_pending = c->prof;
+    if (from == FROM_STAR) {
+      r = run_star(c, d_xy, n, d_out, cap, st);
+    } else {
+      r = run_front(c, d_xy, n, st, from != FROM_RADIX, from == FROM_RAW);
+      if (r == HULL_OK)
+        r = run_final(c, c->ws.lo_xy, c->ws.lo_idx, c->ws.up_xy, c->ws.up_idx, (size_t)n, d_out, cap, st);
+    }
+    if (r != HULL_OK) { c->prof_pending = false; return r; }
+    r = finish(c, st, from == FROM_RADIX ? nullptr : &next);
+    if (next == NEXT_BUCKET) { from = single_read(n) ? FROM_RAW : FROM_BUCKET; continue; }
+    if (next == NEXT_RADIX) { c->fallbacks += 1; from = FROM_RADIX; continue; }
+    if (c->cfg.collect_stats) c->last.sort_fallback = from == FROM_RADIX ? 1 : 0;
+    if (r == HULL_OK || r == HULL_ECAPACITY) *h_count = c->h_plan->h;
+    return r;
+  }
 }
 
 hull_status new_call_patch(hull_ctx* c, cudaStream_t st, PlanPatch p) {
@@ -631,7 +692,7 @@ hull_status hull_create(hull_ctx** out, int device, const hull_config* cfg) {
   c->num_sms = prop.multiProcessorCount;
   if (k2_configure() != cudaSuccess || k3_configure() != cudaSuccess || bucket_configure() != cudaSuccess ||
       fused_configure() != cudaSuccess || fused_occupancy(&c->occ_kf) != cudaSuccess ||
-      k1_poly_configure() != cudaSuccess ||
+      k1_poly_configure() != cudaSuccess || star_configure() != cudaSuccess ||
       bucket_occupancy(&c->occ_kb) != cudaSuccess ||
       split_occupancy(&c->occ_sp) != cudaSuccess ||
       k5_configure(&c->occ_k5) != cudaSuccess ||
@@ -737,28 +798,7 @@ hull_status hull_compute(hull_ctx* c, const int32_t* d_xy, int64_t n, int32_t* d
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   hull_status r = ensure_ws(c, (size_t)n);
   if (r != HULL_OK) return r;
-  // The bucket sort first; a bin it cannot sort in shared memory (heavily
-  // duplicated or extremely clustered input) reruns the call on the radix
-  // passes, which take any input.
-  for (int attempt = 0; attempt < 2; ++attempt) {
-    const bool bucket = attempt == 0;
-    c->prof_pending = c->prof;
-    r = run_front(c, d_xy, (u32)n, st, bucket);
-    if (r != HULL_OK) { c->prof_pending = false; return r; }
-    r = run_final(c, c->ws.lo_xy, c->ws.lo_idx, c->ws.up_xy, c->ws.up_idx, (size_t)n, d_out, cap, st);
-    if (r != HULL_OK) c->prof_pending = false;
-    if (r != HULL_OK) return r;
-    bool fallback = false;
-    r = finish(c, st, bucket ? &fallback : nullptr);
-    if (fallback) {
-      c->fallbacks += 1;
-      continue;
-    }
-    if (c->cfg.collect_stats) c->last.sort_fallback = attempt;
-    if (r == HULL_OK || r == HULL_ECAPACITY) *h_count = c->h_plan->h;
-    return r;
-  }
-  return r;
+  return compute_from(c, d_xy, (u32)n, d_out, cap, h_count, st, star_eligible(c, (u32)n) ? FROM_STAR : FROM_BUCKET);
 }
 
 hull_status hull_compute_multi(hull_ctx* c, int32_t count, const int32_t* const* d_xy, const int64_t* n,
@@ -825,9 +865,13 @@ hull_status hull_compute_multi(hull_ctx* c, int32_t count, const int32_t* const*
     const cudaStream_t ls = lane1 ? c->aux : st;
     if (lane1) { std::swap(c->ws, c->ws2); std::swap(c->plan, c->plan2); }
     c->prof_pending = false;
-    r = run_front(c, d_xy[k], (u32)n[k], ls, true);
-    if (r == HULL_OK) r = run_final(c, c->ws.lo_xy, c->ws.lo_idx, c->ws.up_xy, c->ws.up_idx, (size_t)n[k], d_out[k],
-                                    cap[k], ls);
+    if (star_eligible(c, (u32)n[k])) {
+      r = run_star(c, d_xy[k], (u32)n[k], d_out[k], cap[k], ls);
+    } else {
+      r = run_front(c, d_xy[k], (u32)n[k], ls, true);
+      if (r == HULL_OK) r = run_final(c, c->ws.lo_xy, c->ws.lo_idx, c->ws.up_xy, c->ws.up_idx, (size_t)n[k], d_out[k],
+                                      cap[k], ls);
+    }
     cudaError_t e = cudaSuccess;
     if (r == HULL_OK)
       e = cudaMemcpyAsync(c->h_multi + (size_t)k * kSummaryBytes, c->plan, kSummaryBytes, cudaMemcpyDeviceToHost, ls);
@@ -851,13 +895,20 @@ hull_status hull_compute_multi(hull_ctx* c, int32_t count, const int32_t* const*
       if (c->cfg.collect_stats) c->last = hull_stats{};
       continue;
     }
-    bool fallback = false;
+    Next next = NEXT_NONE;
     const Plan& p = *reinterpret_cast<const Plan*>(c->h_multi + (size_t)k * kSummaryBytes);
-    r = read_summary(c, p, &fallback);
-    if (fallback) {
-      // A bin too large for the bucket sort: this input again, as
-      // hull_compute does (the radix passes after the bucket attempt).
-      r = hull_compute(c, d_xy[k], n[k], d_out[k], cap[k], &h_count[k], stream);
+    r = read_summary(c, p, &next);
+    if (next != NEXT_NONE) {
+      // Not decided: this input again, alone, from the next step on.  The
+      // last input of a lane still has its raw survivors in the lane's workspace.
+      const bool lane1 = two && (k & 1);
+      const bool last = two ? k + 2 >= count : k + 1 >= count;
+      if (lane1) { std::swap(c->ws, c->ws2); std::swap(c->plan, c->plan2); }
+      if (next == NEXT_RADIX) c->fallbacks += 1;
+      r = compute_from(c, d_xy[k], (u32)n[k], d_out[k], cap[k], &h_count[k], st,
+                       next == NEXT_RADIX ? FROM_RADIX
+                                          : single_read((u32)n[k]) && last ? FROM_RAW : FROM_BUCKET);
+      if (lane1) { std::swap(c->ws, c->ws2); std::swap(c->plan, c->plan2); }
     } else {
       if (c->cfg.collect_stats) c->last.sort_fallback = 0;
       if (r == HULL_OK || r == HULL_ECAPACITY) h_count[k] = p.h;
@@ -1107,11 +1158,11 @@ hull_status hull_stage_regions(hull_ctx* c, const int32_t* d_xy, int64_t n, int3
   for (int attempt = 0; attempt < 2; ++attempt) {
     const bool bucket = attempt == 0;
     c->prof_pending = false;
-    r = run_front(c, d_xy, (u32)n, st, bucket, true);   // Figure 2's lists on every first-round survivor
+    r = run_front(c, d_xy, (u32)n, st, bucket);   // Figure 2's lists on every first-round survivor
     if (r != HULL_OK) return r;
-    bool fallback = false;
-    r = finish(c, st, bucket ? &fallback : nullptr);
-    if (fallback) continue;
+    Next next = NEXT_NONE;
+    r = finish(c, st, bucket ? &next : nullptr);
+    if (next != NEXT_NONE) continue;
     if (r != HULL_OK) return r;
     if (h_fallback) *h_fallback = attempt;
     const int64_t rl = c->h_plan->r_lo, ru = c->h_plan->r_up;
@@ -1342,10 +1393,10 @@ hull_status hull_stage_bucket_sort(hull_ctx* c, uint64_t* d_keys, uint32_t* d_va
     e = launch_bucket_sort(w.keys[0], w.idx[0], w.keys[1], w.idx[1], c->plan, w.groups, w.bscratch,
                            c->occ_kb * c->num_sms, st);
   if (e != cudaSuccess) return cuda_fail(e);
-  bool fallback = false;
-  r = finish(c, st, &fallback);
+  Next next = NEXT_NONE;
+  r = finish(c, st, &next);
   if (r != HULL_OK) return r;
-  if (fallback) {
+  if (next != NEXT_NONE) {
     // The input is untouched: sort it on the radix passes instead.
     if (h_fallback) *h_fallback = 1;
     return hull_stage_sort(c, d_keys, d_vals, m, stream);

@@ -67,6 +67,7 @@ enum : u32 {
   ERR_CAPACITY = 4u,    // output capacity below the hull size
   ERR_INTERNAL = 8u,    // an index left its buffer (skipped, never written)
   ERR_FALLBACK = 16u,   // a bin too large for the bucket sort: the call reruns on the radix passes
+  ERR_RETRY = 32u,      // the star path did not decide: the call goes on with the bucket sort
 };
 
 // Each call consumes kEpochStride epochs; look-back status words carry the
@@ -97,27 +98,43 @@ struct ExtPartial {
   u32 idx[4];
 };
 
-// The single-read front's sample polygon (k0_poly.cu builds it, K1 filters
-// with it).  The first part is cleared before every call with the bins.
-constexpr int kPolyDirs = 32;          // directions of the sample's extreme points
-constexpr int kPolySlabs = 4096;       // most x slabs of the polygon's table
+// The single-read front's tables (k0_poly.cu builds the frame and the sample
+// polygon, k1_poly filters with them, k_star.cu finishes; star.cuh has the
+// device code).  The first part is cleared before every call.
+constexpr int kPolyDirs = 64;          // directions of the sample's extreme points
+constexpr int kPolySlabs = 8192;       // most x slabs of the polygon's table
+constexpr int kStarBins = 2048;        // angular bins of the candidates
+constexpr u32 kStarCap = 8192;         // most points that one block finishes
+// An interior input point c and the whitening map u = m00 dx, v = m10 dx +
+// m11 dy of d = p - c.
+struct StarFrame {
+  int cx, cy;
+  float m00, m10, m11;
+};
+// The sample polygon's table: column x (x1 <= x < x1 + xw) lies in slab
+// (x - x1) >> sh; height y is unit (y - y0) >> shy.
+struct PolyHead {
+  int ok, x1;
+  u32 xw, sh;
+  int y0;
+  u32 shy, nslab;
+};
 struct PolyTab {
   // cleared per call
   u64 best[kPolyDirs];   // per direction: (ordered projection << 32 | ~sample index), maximum
+  u64 key[kStarBins];    // per angular bin: the raw survivors' candidate (star::cand_key), maximum
   u32 raw_count;         // K1's survivors: points on or outside the polygon
   u32 done;              // last-block counter of k0
-  u32 pad[2];
-  // written by k0's last block
-  int ok;                // 1: at least 3 corners and an x range with an interior
-  int k;                 // corners (counter-clockwise from the lexicographic minimum)
-  int xl, xr;            // x of the leftmost and of the rightmost corner
-  u32 sh;                // slab s holds x in [xl + s 2^sh, xl + (s + 1) 2^sh)
-  u32 nslab;
-  u32 pad2[2];
-  int2 yb[kPolySlabs];    // per slab (ylo, yhi): a point of the slab with ylo < y < yhi is strictly
-                         // inside (ylo >= the lower chain, yhi <= the upper chain over the slab)
+  u32 list_count;        // points left by the candidates
+  u32 done2;             // last-block counter of k_star
+  u32 error;             // ERR_RANGE from K1
+  u32 pad[3];
+  // written by k0
+  StarFrame frame;
+  PolyHead head;
+  u32 tab[kPolySlabs];
 };
-constexpr size_t kPolyClearBytes = offsetof(PolyTab, ok);
+constexpr size_t kPolyClearBytes = offsetof(PolyTab, frame);
 
 struct Plan {
   // summary fields first: the host copies back everything before `ctr`

@@ -15,6 +15,7 @@
 // zeroed counters and histograms for the kernels that follow.
 #include "hull_internal.cuh"
 #include "kernels.h"
+#include "star.cuh"
 
 namespace gbh {
 
@@ -298,138 +299,64 @@ k1_extremes(const int* __restrict__ xy, u32 n, u32 spin_limit, Plan* plan,
   k1_reduce_finish<BLOCK>(b, n, spin_limit, plan, partials);
 }
 
-// ---- K1 of the single-read front: the extremes and the sample polygon's
-// filter in one pass.  A point strictly inside the sample polygon (PolyTab,
-// k0_poly.cu: xl < x < xr and strictly inside its slab's y interval) is
-// strictly inside the hull, so it is neither an extreme nor a vertex: it is
-// dropped.  Every other point is a candidate for the
-// extremes and is staged in its warp's slice of shared memory; a warp
-// flushes its slice with one atomic reservation into (rxy, ridx), in no
-// particular order (the later kernels order the survivors themselves).
-// Each warp streams one contiguous run of 8 x 32 pairs per round (16-byte
-// aligned input); the rest, and an odd last point, go one pair per lane.
+// ---- K1 of the single-read front: the sample polygon's filter, the only
+// pass over the input.  A point strictly inside the sample polygon (PolyTab)
+// is strictly inside the hull: it is dropped.  Every other point is staged
+// in its warp's slice of shared memory; a warp flushes its slice with one
+// atomic reservation into (rxy, ridx), in no particular order, and offers
+// each of its points as the candidate of its angular bin (star.cuh).
+//
+// Bound by the stream: a point costs about a dozen instructions and, inside
+// the polygon's columns, one 4-byte table word (8-byte words took two
+// shared-memory passes per warp).  Every warp streams one contiguous run of
+// 4 x 32 pairs per round, the next round's loads issued before this round is
+// tested.  The survivors (well below one in a hundred of ordinary inputs)
+// are pushed slot by slot under a warp-uniform branch, which costs a warp two
+// instructions for a slot without any.  An input that starts on an odd row
+// (8-byte aligned) gives its first point to one lane and streams the rest.
 constexpr int K1P_BLOCK = 512;
 constexpr int K1P_WARPS = K1P_BLOCK / 32;
-constexpr int K1P_SLICE = 256;                 // staged points per warp (a half round: 32 x 8)
+constexpr int K1P_SLICE = 256;                 // staged points per warp
+constexpr int K1P_V = 4;                       // pairs per lane and round
 
 struct K1PSmem {
   int2 sxy[K1P_WARPS][K1P_SLICE];
   u32 sidx[K1P_WARPS][K1P_SLICE];
-  int2 yb[kPolySlabs];
+  u32 tab[kPolySlabs];
 };
 
 __global__ void __launch_bounds__(K1P_BLOCK, 2)
-k1_poly(const int* __restrict__ xy, u32 n, u32 spin_limit, Plan* plan, ExtPartial* __restrict__ partials,
-        const PolyTab* __restrict__ T, u32* raw_count, int2* __restrict__ rxy, u32* __restrict__ ridx) {
+k1_poly(const int2* __restrict__ P, u32 n, PolyTab* __restrict__ T, int2* __restrict__ rxy, u32* __restrict__ ridx) {
   extern __shared__ __align__(16) unsigned char k1p_smem[];
   K1PSmem& S = *reinterpret_cast<K1PSmem*>(k1p_smem);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const u32 lt = (1u << lane) - 1u;
-  const int ok = T->ok;
-  const int xl = T->xl, xr = T->xr;
-  const u32 sh = T->sh;
+  const int wid = threadIdx.x >> 5;
+  const PolyHead H = T->head;
+  star::RawSink<kStarBins, K1P_SLICE> sink{S.sxy[wid], S.sidx[wid], 0u, &T->frame, &T->raw_count, &T->error, T->key,
+                                           rxy, ridx, n};
+  star::stream_points<K1P_V>(P, n, 0u, blockIdx.x * K1P_WARPS + wid, gridDim.x * K1P_WARPS, H, S.tab, sink, [&] {
+    for (u32 q = threadIdx.x; q < H.nslab; q += K1P_BLOCK) S.tab[q] = T->tab[q];
+    __syncthreads();
+  });
+  if (sink.fill) sink.flush();
+}
 
-  if (ok) {
-    const u32 nslab = T->nslab;
-    for (u32 q = threadIdx.x; q < nslab; q += K1P_BLOCK) S.yb[q] = T->yb[q];
-  }
-  __syncthreads();
-  // Branch-free: every lane looks its slab up (slab 0 when x is outside the
-  // range, whose answer is then ignored), so a warp never splits here.
-  auto inside = [&](int x, int y) -> bool {
-    const bool inx = ok && x > xl && x < xr;
-    const int2 q = S.yb[inx ? (u32)(x - xl) >> sh : 0u];
-    return inx & (y > q.x) & (y < q.y);
-  };
+// The extremes and the Plan from K1's raw survivors (every extreme is one),
+// when the call goes on with the bucket sort.
+__global__ void __launch_bounds__(512)
+k1_raw(const int2* __restrict__ rxy, const u32* __restrict__ ridx, u32 n, u32 spin_limit, Plan* plan,
+       ExtPartial* __restrict__ partials, const PolyTab* __restrict__ T) {
   Best b;
   best_init(b);
-  int2* sxy = S.sxy[wid];
-  u32* sidx = S.sidx[wid];
-  u32 fill = 0;                                   // uniform over the warp
-  auto flush = [&]() {
-    __syncwarp();
-    u32 base = 0;
-    if (lane == 0) base = atomicAdd(raw_count, fill);
-    base = __shfl_sync(0xFFFFFFFFu, base, 0);
-    for (u32 q = lane; q < fill; q += 32) {
-      if (base + q < n) { rxy[base + q] = sxy[q]; ridx[base + q] = sidx[q]; }
-      else flag_error(plan, ERR_INTERNAL);
-    }
-    __syncwarp();
-    fill = 0;
-  };
-  // Up to 8 points per lane (validity in `valid`): the survivors become
-  // extreme candidates and are staged (the whole warp calls it).
-  auto take = [&](const int* px, const int* py, const u32* pi, u32 valid, int cntpts) {
-    u32 keep = 0;
-    for (int e = 0; e < cntpts; ++e)
-      if (((valid >> e) & 1u) && !inside(px[e], py[e])) keep |= 1u << e;
-    if (!__any_sync(0xFFFFFFFFu, keep != 0)) return;
-    for (int e = 0; e < cntpts; ++e)
-      if ((keep >> e) & 1u) consider(b, px[e], py[e], pi[e]);
-    const u32 cnt = __popc(keep);
-    u32 inc = cnt;
-    #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const u32 t = __shfl_up_sync(0xFFFFFFFFu, inc, o);
-      if (lane >= o) inc += t;
-    }
-    const u32 tot = __shfl_sync(0xFFFFFFFFu, inc, 31);
-    if (fill + tot > (u32)K1P_SLICE) flush();
-    u32 pos = fill + inc - cnt;
-    for (int e = 0; e < cntpts; ++e)
-      if ((keep >> e) & 1u) { sxy[pos] = make_int2(px[e], py[e]); sidx[pos] = pi[e]; ++pos; }
-    fill += tot;
-  };
-  const int4* p4 = reinterpret_cast<const int4*>(xy);
-  const u32 npair = n >> 1;
-  const u32 nthreads = gridDim.x * K1P_BLOCK;
-  const u32 gw = (blockIdx.x * K1P_BLOCK + threadIdx.x) >> 5, nwarps = nthreads >> 5;
-  u32 R = 0;
-  for (; R + 8u * nthreads <= npair; R += 8u * nthreads) {
-    const u32 u0 = R + gw * 256u + lane;
-    int4 v[8];
-    #pragma unroll
-    for (int u = 0; u < 8; ++u) v[u] = p4[u0 + 32u * u];
-    #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      int px[8], py[8];
-      u32 pi[8];
-      #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int4 w = v[4 * h + q];
-        const u32 j = u0 + 32u * (4 * h + q);
-        px[2 * q] = w.x; py[2 * q] = w.y; pi[2 * q] = 2u * j;
-        px[2 * q + 1] = w.z; py[2 * q + 1] = w.w; pi[2 * q + 1] = 2u * j + 1u;
-      }
-      take(px, py, pi, 0xFFu, 8);
-    }
+  const u32 m = min(T->raw_count, n);
+  for (u32 i = blockIdx.x * 512u + threadIdx.x; i < m; i += gridDim.x * 512u) {
+    const int2 p = rxy[i];
+    const u32 id = ridx[i];
+    const u64 kxy = ((u64)ord(p.x) << 32) | ord(p.y), kyx = ((u64)ord(p.y) << 32) | ord(p.x);
+    const u64 k[4] = {kxy, ~kxy, kyx, ~kyx};
+    const u32 v[4] = {id, id, id, id};
+    merge_best(b, k, v);
   }
-  // The rest of the pairs, one per lane; then the odd last point.
-  for (u32 wb = R + gw * 32u; wb < npair; wb += nwarps * 32u) {
-    const u32 j = wb + lane;
-    int px[2] = {0, 0}, py[2] = {0, 0};
-    u32 pi[2] = {2u * j, 2u * j + 1u};
-    u32 valid = 0;
-    if (j < npair) {
-      const int4 w = p4[j];
-      px[0] = w.x; py[0] = w.y; px[1] = w.z; py[1] = w.w;
-      valid = 3u;
-    }
-    take(px, py, pi, valid, 2);
-  }
-  if ((n & 1u) && gw == 0) {
-    int px[1] = {0}, py[1] = {0};
-    u32 pi[1] = {n - 1};
-    u32 valid = 0;
-    if (lane == 0) {
-      px[0] = xy[2 * (n - 1)]; py[0] = xy[2 * (n - 1) + 1]; valid = 1u;
-    }
-    take(px, py, pi, valid, 1);
-  }
-  if (fill) flush();
-  __threadfence();
-  k1_reduce_finish<K1P_BLOCK>(b, n, spin_limit, plan, partials, raw_count);
+  k1_reduce_finish<512>(b, n, spin_limit, plan, partials, &T->raw_count);
 }
 
 }  // namespace
@@ -467,9 +394,17 @@ cudaError_t k1_poly_configure() {
   return cudaFuncSetAttribute(k1_poly, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(K1PSmem));
 }
 
-cudaError_t launch_k1_poly(const int* xy, u32 n, u32 spin_limit, Plan* plan, ExtPartial* partials, const PolyTab* T,
-                           u32* raw_count, int2* rxy, u32* ridx, int num_sms, cudaStream_t st) {
-  k1_poly<<<num_sms * 2, K1P_BLOCK, sizeof(K1PSmem), st>>>(xy, n, spin_limit, plan, partials, T, raw_count, rxy, ridx);
+cudaError_t launch_k1_poly(const int* xy, u32 n, PolyTab* T, int2* rxy, u32* ridx, int num_sms, cudaStream_t st) {
+  const u32 rounds = (n / 2 + K1P_BLOCK * K1P_V - 1) / (K1P_BLOCK * K1P_V);
+  const u32 cap = (u32)num_sms * 2u;
+  const u32 grid = rounds < 1u ? 1u : (rounds < cap ? rounds : cap);
+  k1_poly<<<grid, K1P_BLOCK, sizeof(K1PSmem), st>>>(reinterpret_cast<const int2*>(xy), n, T, rxy, ridx);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_k1_raw(const int2* rxy, const u32* ridx, u32 n, u32 spin_limit, Plan* plan, ExtPartial* partials,
+                          const PolyTab* T, int num_sms, cudaStream_t st) {
+  k1_raw<<<num_sms, 512, 0, st>>>(rxy, ridx, n, spin_limit, plan, partials, T);
   return cudaGetLastError();
 }
 

@@ -1,0 +1,225 @@
+// The star path's finishing kernels (star.cuh): the hull of the single-read
+// front's raw survivors, and the whole hull of a small input in one launch.
+//
+// k_star   all blocks test K1's raw survivors against the polygon of the
+//          angular candidates (about 129k of 20M uniform points come in,
+//          a few thousand at most go on) and append the rest to a list; the
+//          last block to finish sorts the list by angle and finds the hull
+//          in shared memory.
+// k_small  one block: frame, sample polygon, one pass over the points, then
+//          the same on the points left.
+//
+// Both are bound by latency (barriers and dependent loads), so the design
+// counts those: what the bucket sort and the chain merges did in eight
+// launches over the same few thousand points is one block's shared memory
+// here.  A list beyond kStarCap, a crowded bin or a degenerate input sets
+// ERR_RETRY and the call goes on with the bucket sort.
+#include "hull_internal.cuh"
+#include "kernels.h"
+#include "star.cuh"
+
+namespace gbh {
+
+namespace {
+
+constexpr int KS_BLOCK = 1024;
+constexpr int KS_CAP = (int)kStarCap;
+// More raw survivors than this and more than a quarter of the input: the
+// candidates cannot bring them below kStarCap (most points lie next to the
+// hull), so the blocks leave at once.
+constexpr u32 KS_RAW_MAX = 1u << 18;
+// Up to this many points k_small takes them all into its list: the sample
+// polygon would cost more than it saves.
+constexpr u32 KS_DIRECT = 4096;
+constexpr u32 KS_SLABS = 2048;
+constexpr int KS_SAMPLES = 4;         // samples per thread of k_small's polygon
+
+typedef star::ListSmem<KS_BLOCK, KS_CAP, kStarBins> List;
+typedef star::CandTab<kStarBins> Cands;
+
+struct StarSmem {
+  union {
+    List list;
+    Cands cands;
+  };
+  bool last;
+};
+
+struct SmallSmem {
+  List list;
+  union {
+    struct {
+      u64 key[kStarBins];
+      Cands cands;
+    };
+    u32 tab[KS_SLABS];
+  };
+  star::FrameSmem<KS_BLOCK> frame;
+  star::PolySmem poly;
+  u64 best[kPolyDirs];
+  u32 count, error;
+};
+
+// The call's summary (one thread).  h < 0: not decided.
+__device__ void write_summary(Plan* plan, u32 n, u32 raw, u32 s, int h, long long cap, u32 error) {
+  plan->n = n;
+  u32 e = error;
+  if (!(e & ERR_RANGE)) {
+    if (h < 0) e |= ERR_RETRY;
+    else if ((long long)h > cap) e |= ERR_CAPACITY;
+  }
+  plan->error = e;
+  plan->s = s; plan->s_quad = 0; plan->s_raw = raw; plan->r_lo = s; plan->r_up = 0;
+  plan->h = h > 0 ? (u32)h : 0u; plan->h_lo = 0; plan->h_up = 0;
+  plan->ncorner = 0; plan->learned_used = 0; plan->npasses = 0;
+  plan->sorted_in_b = 1; plan->ngroups = 1;
+}
+
+__global__ void __launch_bounds__(KS_BLOCK)
+k_star(const int2* __restrict__ P, u32 n, PolyTab* T, const int2* __restrict__ rxy, const u32* __restrict__ ridx,
+       int2* lxy, u32* lidx, Plan* plan, int* out, long long cap) {
+  extern __shared__ __align__(16) unsigned char ks_smem[];
+  StarSmem& S = *reinterpret_cast<StarSmem*>(ks_smem);
+  const int lane = threadIdx.x & 31, t = threadIdx.x;
+  const u32 q = min(T->raw_count, n);
+  const StarFrame F = T->frame;
+  if (q > KS_RAW_MAX && q > n / 4) {
+    if (blockIdx.x == 0 && t == 0) write_summary(plan, n, q, 0, -1, cap, T->error);
+    return;
+  }
+  if (blockIdx.x * (u32)KS_BLOCK < q) {
+    if (t < kStarBins / 32) S.cands.occ[t] = 0u;
+    __syncthreads();
+    constexpr int PER = kStarBins / KS_BLOCK;
+    u64 k[PER];
+    #pragma unroll
+    for (int j = 0; j < PER; ++j) k[j] = __ldcg(&T->key[t + j * KS_BLOCK]);
+    #pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      const int b = t + j * KS_BLOCK;
+      if (k[j]) {
+        const u32 id = min(~(u32)k[j], n - 1u);
+        S.cands.cand[b] = P[id];
+        S.cands.cid[b] = id;
+        atomicOr(&S.cands.occ[b >> 5], 1u << (b & 31));
+      }
+    }
+    __syncthreads();
+    for (u32 i0 = blockIdx.x * (u32)KS_BLOCK; i0 < q; i0 += gridDim.x * (u32)KS_BLOCK) {
+      const u32 i = i0 + t;
+      bool keep = false;
+      int2 p = make_int2(0, 0);
+      u32 id = 0;
+      if (i < q) {
+        p = rxy[i];
+        id = ridx[i];
+        float u, v;
+        star::to_uv(F, p.x - F.cx, p.y - F.cy, u, v);
+        keep = !star::dropped_by_cands<kStarBins>(S.cands, F, star::bin_of<kStarBins>(u, v), p.x, p.y, id);
+      }
+      const u32 bal = __ballot_sync(0xFFFFFFFFu, keep);
+      u32 base = 0;
+      if (lane == 0 && bal) base = atomicAdd(&T->list_count, (u32)__popc(bal));
+      base = __shfl_sync(0xFFFFFFFFu, base, 0) + __popc(bal & ((1u << lane) - 1u));
+      if (keep && base < kStarCap) { lxy[base] = p; lidx[base] = id; }
+    }
+  }
+  __threadfence();
+  __syncthreads();
+  if (t == 0) S.last = atomicAdd(&T->done2, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!S.last) return;
+  __threadfence();
+  const u32 m = *(volatile u32*)&T->list_count;
+  int h = -1;
+  const u32 err = T->error;
+  if (m <= kStarCap && !(err & ERR_RANGE)) {
+    for (u32 i = t; i < m; i += KS_BLOCK) {
+      S.list.p[i] = __ldcg(&lxy[i]);
+      S.list.id[i] = __ldcg(&lidx[i]);
+      S.list.ta[i] = (unsigned short)i;
+    }
+    __syncthreads();
+    h = star::list_hull<KS_BLOCK, KS_CAP, kStarBins>(S.list, m, F, out, cap);
+  }
+  if (t == 0) write_summary(plan, n, q, m, h, cap, err);
+}
+
+__global__ void __launch_bounds__(KS_BLOCK)
+k_small(const int2* __restrict__ P, u32 n, Plan* plan, int* out, long long cap) {
+  extern __shared__ __align__(16) unsigned char ks_smem[];
+  SmallSmem& S = *reinterpret_cast<SmallSmem*>(ks_smem);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, t = threadIdx.x;
+  if (t == 0) { S.count = 0u; S.error = 0u; }
+  if (t < kPolyDirs) S.best[t] = 0ull;
+  const StarFrame F = star::make_frame<KS_BLOCK>(P, n, S.frame);
+  u32 m0 = n;
+  bool bad = false;
+  if (n <= KS_DIRECT) {
+    for (u32 i = t; i < n; i += KS_BLOCK) {
+      const int2 p = P[i];
+      S.list.p[i] = p;
+      S.list.id[i] = i;
+      bad = bad || star::out_of_range(p.x, p.y);
+    }
+  } else {
+    constexpr u32 NS = KS_SAMPLES * KS_BLOCK;
+    static_assert(NS <= KS_DIRECT, "a stride of at least one point");
+    const u32 stride = n / NS;
+    int2 p[KS_SAMPLES];
+    #pragma unroll
+    for (int r = 0; r < KS_SAMPLES; ++r) p[r] = P[(r * KS_BLOCK + t) * stride];
+    #pragma unroll
+    for (int r = 0; r < KS_SAMPLES; ++r) star::offer_sample(F, p[r], r * KS_BLOCK + t, S.best);
+    __syncthreads();
+    if (t < kPolyDirs) {
+      const u32 i = ~(u32)S.best[t];
+      S.poly.p[t] = i < NS ? P[i * stride] : make_int2(0, 0);
+      const u32 h = __ballot_sync(0xFFFFFFFFu, i < NS);
+      if (lane == 0) S.poly.has[wid] = h;
+    }
+    __syncthreads();
+    const PolyHead H = star::build_poly<KS_BLOCK>(S.poly, F, S.tab, KS_SLABS);
+    __syncthreads();
+    star::ListSink<decltype(S.list)> sink{&S.list, &S.count, (u32)KS_CAP, false};
+    star::stream_points<4>(P, n, 0u, (u32)wid, (u32)(KS_BLOCK / 32), H, S.tab, sink, [] {});
+    bad = sink.bad;
+    __syncthreads();
+    m0 = S.count;
+  }
+  if (bad) S.error = ERR_RANGE;
+  __syncthreads();
+  const u32 err = S.error;
+  int h = -1;
+  u32 m = m0;
+  if (m0 <= (u32)KS_CAP && !err) {
+    m = star::filter_list<KS_BLOCK, KS_CAP, kStarBins>(S.list, m0, F, S.key, S.cands);
+    h = star::list_hull<KS_BLOCK, KS_CAP, kStarBins>(S.list, m, F, out, cap);
+  }
+  if (t == 0) write_summary(plan, n, m0, m, h, cap, err);
+}
+
+}  // namespace
+
+cudaError_t star_configure() {
+  cudaError_t e = cudaFuncSetAttribute(k_star, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(StarSmem));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmallSmem));
+  return e;
+}
+
+cudaError_t launch_star(const int* xy, u32 n, PolyTab* T, const int2* rxy, const u32* ridx, int2* lxy, u32* lidx,
+                        Plan* plan, int* out, long long cap, int num_sms, cudaStream_t st) {
+  const u32 want = n / (32u * KS_BLOCK) + 1u;      // a block per 32,768 input points
+  const u32 grid = want < (u32)num_sms ? want : (u32)num_sms;
+  k_star<<<grid, KS_BLOCK, sizeof(StarSmem), st>>>(reinterpret_cast<const int2*>(xy), n, T, rxy, ridx, lxy, lidx, plan,
+                                                   out, cap);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_small(const int* xy, u32 n, Plan* plan, int* out, long long cap, cudaStream_t st) {
+  k_small<<<1, KS_BLOCK, sizeof(SmallSmem), st>>>(reinterpret_cast<const int2*>(xy), n, plan, out, cap);
+  return cudaGetLastError();
+}
+
+}  // namespace gbh

@@ -58,14 +58,23 @@ cudaError_t launch_witness(const int2* sample, u32 n, Plan* plan, u64* wkey, int
 cudaError_t launch_k2_fused(const int* xy, u32 n, Plan* plan, const u64* wkey, const int2* sample, u64* okey,
                             u32* oidx, u32* btot, u32* bstart, uint2* groups, u32* fcur, bool count, int grid,
                             cudaStream_t st, const u32* ncount = nullptr, const u32* imap = nullptr);
-// The single-read front: the sample polygon (k0_poly.cu), then K1 with that
-// polygon as its filter, writing the points on or outside it to (rxy, ridx)
-// (count in T->raw_count, which must be zero before k0) and the witness
-// sample (every kSampleStride-th point) to `sample`.
+// The single-read front: the frame and the sample polygon (k0_poly.cu), then
+// K1 with that polygon as its filter, writing the points on or outside it to
+// (rxy, ridx) (count in T->raw_count) and their candidates to T->key; the
+// head of T (kPolyClearBytes) must be zero before k0.  launch_star finishes
+// the call from them (ERR_RETRY in the Plan: it did not decide), with (lxy,
+// lidx) of kStarCap entries as scratch; launch_k1_raw builds the Plan from
+// them for the bucket sort.  launch_small: a whole small input in one block.
+constexpr u32 kSmallMax = 1u << 16;
 cudaError_t launch_poly(const int* xy, u32 n, PolyTab* T, int num_sms, cudaStream_t st);
 cudaError_t k1_poly_configure();
-cudaError_t launch_k1_poly(const int* xy, u32 n, u32 spin_limit, Plan* plan, ExtPartial* partials, const PolyTab* T,
-                           u32* raw_count, int2* rxy, u32* ridx, int num_sms, cudaStream_t st);
+cudaError_t launch_k1_poly(const int* xy, u32 n, PolyTab* T, int2* rxy, u32* ridx, int num_sms, cudaStream_t st);
+cudaError_t launch_k1_raw(const int2* rxy, const u32* ridx, u32 n, u32 spin_limit, Plan* plan, ExtPartial* partials,
+                          const PolyTab* T, int num_sms, cudaStream_t st);
+cudaError_t star_configure();
+cudaError_t launch_star(const int* xy, u32 n, PolyTab* T, const int2* rxy, const u32* ridx, int2* lxy, u32* lidx,
+                        Plan* plan, int* out, long long cap, int num_sms, cudaStream_t st);
+cudaError_t launch_small(const int* xy, u32 n, Plan* plan, int* out, long long cap, cudaStream_t st);
 cudaError_t launch_place(const u64* ak, const u32* ai, u32 n, Plan* plan, const u32* bstart, u32* ccur, u64* ok,
                          u32* oi, int num_sms, cudaStream_t st);
 size_t bucket_smem();

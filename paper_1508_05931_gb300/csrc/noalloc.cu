@@ -125,7 +125,7 @@ hull_status noalloc_setup(int dev, NoAllocDevice** out) {
     cudaDeviceProp prop;
     if (cudaGetDeviceProperties(&prop, dev) != cudaSuccess) { cudaGetLastError(); return HULL_ECUDA; }
     if (carve(nullptr, prop.multiProcessorCount).total > kNoAllocBytes) return HULL_EINTERNAL;
-    if (k2_configure() != cudaSuccess || k3_configure() != cudaSuccess ||
+    if (star_configure() != cudaSuccess || k2_configure() != cudaSuccess || k3_configure() != cudaSuccess ||
         k5_configure(&d.occ_k5) != cudaSuccess ||
         k2_occupancy(&d.occ_k2c, &d.occ_k2) != cudaSuccess || k3_occupancy(&d.occ_k3) != cudaSuccess ||
         k4_occupancy(&d.occ_k4) != cudaSuccess || d.occ_k5 < 1) {
@@ -162,38 +162,45 @@ extern "C" hull_status hull_compute_noalloc(const int32_t* d_xy, int64_t n, int3
   Carve c = carve(d->base, d->num_sms);
   const u32 un = (u32)n;
 
-  cudaError_t e = cudaMemsetAsync(c.plan, 0, c.zero_bytes, st);
-  if (e == cudaSuccess)
-    e = launch_k1(d_xy, un, kDefaultSpinLimit, c.plan, c.partials, k1_grid(un, d->num_sms), st);
-  const size_t t2 = (un + k2_tile() - 1) / k2_tile();
-  if (e == cudaSuccess)
-    e = launch_k2(d_xy, c.plan, c.keys[0], c.idx[0], c.st_filter, c.mask, grid_for(d->occ_k2c, d->num_sms, t2),
-                   grid_for(d->occ_k2, d->num_sms, t2), st);
-  const size_t t3 = (un + k3_tile() - 1) / k3_tile();
-  for (u32 p = 0; p < (u32)kMaxPasses && e == cudaSuccess; ++p)
-    e = launch_k3(c.keys[p & 1], c.idx[p & 1], c.keys[(p + 1) & 1], c.idx[(p + 1) & 1], c.plan,
-                  c.st_sort, p, grid_for(d->occ_k3, d->num_sms, t3), st);
-  const size_t t4 = (un + k4_tile() - 1) / k4_tile();
-  if (e == cudaSuccess)
-    e = launch_k4(c.keys[0], c.idx[0], c.keys[1], c.idx[1], c.plan, c.st_region, t4, c.lo_xy, c.lo_idx,
-                  c.up_xy, c.up_idx, c.h_xy[0], c.h_idx[0], c.h_xy[1], c.h_idx[1],
-                  grid_for(d->occ_k4, d->num_sms, t4), st);
-  const size_t chunks = (un + 4) / (size_t)k5_chunk() + 2;
-  if (e == cudaSuccess)
-    e = launch_k5(c.lo_xy, c.lo_idx, c.up_xy, c.up_idx, c.plan, c.h_xy[0], c.h_idx[0], c.h_xy[1],
-                  c.h_idx[1], c.cnt[0], c.cnt[1], c.jobs, d_out, (long long)cap,
-                  grid_for(d->occ_k5 < 4 ? d->occ_k5 : 4, d->num_sms, chunks < 64 ? 64 : chunks), st);
-  // Read the summary back into host stack memory (a pageable copy: no
-  // pinned buffer is allocated) and wait for the stream.
+  // The summary comes back into host stack memory (a pageable copy: no
+  // pinned buffer is allocated) and the call waits for the stream.
   alignas(16) unsigned char summary[offsetof(Plan, ctr)];
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(summary, c.plan, sizeof(summary), cudaMemcpyDeviceToHost, st);
+  const Plan* p = reinterpret_cast<const Plan*>(summary);
+  // The star path first (one launch, no scratch but the Plan); what it does
+  // not decide takes the radix pipeline.
+  static_assert(HULL_NOALLOC_MAX_POINTS <= kSmallMax, "one block takes every call");
+  cudaError_t e = launch_small(d_xy, un, c.plan, d_out, (long long)cap, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(summary, c.plan, sizeof(summary), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e == cudaSuccess && (p->error & ERR_RETRY)) {
+    e = cudaMemsetAsync(c.plan, 0, c.zero_bytes, st);
+    if (e == cudaSuccess)
+      e = launch_k1(d_xy, un, kDefaultSpinLimit, c.plan, c.partials, k1_grid(un, d->num_sms), st);
+    const size_t t2 = (un + k2_tile() - 1) / k2_tile();
+    if (e == cudaSuccess)
+      e = launch_k2(d_xy, c.plan, c.keys[0], c.idx[0], c.st_filter, c.mask, grid_for(d->occ_k2c, d->num_sms, t2),
+                     grid_for(d->occ_k2, d->num_sms, t2), st);
+    const size_t t3 = (un + k3_tile() - 1) / k3_tile();
+    for (u32 p = 0; p < (u32)kMaxPasses && e == cudaSuccess; ++p)
+      e = launch_k3(c.keys[p & 1], c.idx[p & 1], c.keys[(p + 1) & 1], c.idx[(p + 1) & 1], c.plan,
+                    c.st_sort, p, grid_for(d->occ_k3, d->num_sms, t3), st);
+    const size_t t4 = (un + k4_tile() - 1) / k4_tile();
+    if (e == cudaSuccess)
+      e = launch_k4(c.keys[0], c.idx[0], c.keys[1], c.idx[1], c.plan, c.st_region, t4, c.lo_xy, c.lo_idx,
+                    c.up_xy, c.up_idx, c.h_xy[0], c.h_idx[0], c.h_xy[1], c.h_idx[1],
+                    grid_for(d->occ_k4, d->num_sms, t4), st);
+    const size_t chunks = (un + 4) / (size_t)k5_chunk() + 2;
+    if (e == cudaSuccess)
+      e = launch_k5(c.lo_xy, c.lo_idx, c.up_xy, c.up_idx, c.plan, c.h_xy[0], c.h_idx[0], c.h_xy[1],
+                    c.h_idx[1], c.cnt[0], c.cnt[1], c.jobs, d_out, (long long)cap,
+                    grid_for(d->occ_k5 < 4 ? d->occ_k5 : 4, d->num_sms, chunks < 64 ? 64 : chunks), st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(summary, c.plan, sizeof(summary), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     return HULL_ECUDA;
   }
-  const Plan* p = reinterpret_cast<const Plan*>(summary);
   if (p->error & ERR_RANGE) return HULL_ERANGE;
   if (p->error & ERR_TIMEOUT) return HULL_ETIMEOUT;
   if (p->error & ERR_INTERNAL) return HULL_EINTERNAL;

@@ -1,0 +1,741 @@
+// The star path: the hull of the points that survive a sample polygon,
+// found in angular order around an interior input point c (Section 2.1
+// steps 3-8 with the pivot moved inside: distance and angle about c, the
+// sort by angle, and the scan that pops non-left turns, run as rounds in
+// which every point looks at its neighbours).
+//
+// A frame holds c and a linear map that whitens the sample's covariance, so
+// that elongated sets spread evenly over the angular bins.  The map, the
+// bins and the choice of candidates are float and only steer; every
+// decision to drop a point is exact in 64-bit integers:
+//   a point q inside the closed triangle (c, a, b) of three input points
+//   with cross(a - c, b - c) > 0, not on the side a b, is no hull vertex
+//   (q = c aside); on the open segment a b neither; equal to a or b it is
+//   the duplicate with the larger index.
+// The drops of a round may use points that the same round drops: those are
+// input points too.  The rounds end with a polygon that is verified: every
+// consecutive cross product about c positive and every turn strictly left
+// means a convex polygon of input points with c strictly inside, in which
+// every other input point was shown to lie.  Anything else (a degenerate
+// set, a crowded bin, too many points or rounds) returns failure and the
+// caller takes the general path.
+#pragma once
+
+#include "hull_internal.cuh"
+
+namespace gbh {
+namespace star {
+
+__device__ __forceinline__ void to_uv(const StarFrame& F, int dx, int dy, float& u, float& v) {
+  const float fx = (float)dx, fy = (float)dy;
+  u = __fmul_rn(fx, F.m00);
+  v = __fmaf_rn(fy, F.m11, __fmul_rn(fx, F.m10));
+}
+
+// Angular bin of (u, v): the diamond angle t in [0, 4), monotone in the
+// polar angle (up to rounding, which the exact tests absorb).
+template <int NB>
+__device__ __forceinline__ u32 bin_of(float u, float v) {
+  const float t = __fdividef(v, fabsf(u) + fabsf(v));
+  const float a = u >= 0.0f ? (v >= 0.0f ? t : 4.0f + t) : 2.0f - t;
+  const int b = (int)(a * (float)(NB / 4));      // NaN (the point c itself) converts to 0
+  return (u32)min(max(b, 0), NB - 1);
+}
+
+// Candidate key of a point: the whitened radius, then the smaller index (all
+// duplicates of a point share its bin and radius).
+__device__ __forceinline__ u64 cand_key(float u, float v, u32 idx) {
+  return ((u64)__float_as_uint(__fmaf_rn(u, u, __fmul_rn(v, v))) << 32) | (u64)(~idx);
+}
+
+__device__ __forceinline__ bool out_of_range(int x, int y) {
+  return (u32)x + (u32)kCoordLimit > 2u * (u32)kCoordLimit || (u32)y + (u32)kCoordLimit > 2u * (u32)kCoordLimit;
+}
+
+// q dropped by the triangle (c, a, b); a, b, q relative to c.
+// orient(a, b, q) = cross(a, b) - cross(a, q) - cross(q, b): three products
+// (each below 2^61, the sum below 2^63).
+__device__ __forceinline__ bool dropped_by(int2 a, int2 b, int2 q) {
+  const long long ab = cross2(a.x, a.y, b.x, b.y);
+  const long long aq = cross2(a.x, a.y, q.x, q.y), qb = cross2(q.x, q.y, b.x, b.y);
+  const long long o = ab - aq - qb;
+  return ab > 0 && aq >= 0 && qb >= 0 && (o > 0 || (o == 0 && aq > 0 && qb > 0));
+}
+
+// Exclusive block scan; `ws` holds BLOCK / 32 words that no warp still reads
+// (callers alternate two areas, so one barrier per scan suffices).
+template <int BLOCK>
+__device__ __forceinline__ u32 block_scan(u32 v, u32* ws, u32& total) {
+  constexpr int W = BLOCK / 32;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  u32 inc = v;
+  #pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const u32 t = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+    if (lane >= o) inc += t;
+  }
+  if (lane == 31) ws[wid] = inc;
+  __syncthreads();
+  u32 x = lane < W ? ws[lane] : 0u;
+  #pragma unroll
+  for (int o = 1; o < W; o <<= 1) {
+    const u32 t = __shfl_up_sync(0xFFFFFFFFu, x, o);
+    if (lane >= o) x += t;
+  }
+  total = __shfl_sync(0xFFFFFFFFu, x, W - 1);
+  const u32 before = __shfl_sync(0xFFFFFFFFu, x, wid > 0 ? wid - 1 : 0);
+  return (wid > 0 ? before : 0u) + inc - v;
+}
+
+// ---------------------------------------------------------------- frame
+// From BLOCK strided points of P[0, n): their mean and covariance, the
+// whitening map (the inverse Cholesky factor, determinant > 0) and c, the
+// sampled point nearest the mean.  Every block that calls it with the same
+// P and n gets the same frame.
+template <int BLOCK>
+struct FrameSmem {
+  float sum[BLOCK / 32][5];
+  u64 best;
+  int2 c;
+};
+
+template <int BLOCK>
+__device__ __forceinline__ StarFrame make_frame(const int2* __restrict__ P, u32 n, FrameSmem<BLOCK>& S) {
+  constexpr int W = BLOCK / 32;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int2 o = P[0];
+  const int2 p = P[(u32)(((u64)threadIdx.x * n) / BLOCK)];
+  const float fx = (float)p.x - (float)o.x, fy = (float)p.y - (float)o.y;
+  float s[5] = {fx, fy, fx * fx, fx * fy, fy * fy};
+  #pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    #pragma unroll
+    for (int d = 16; d > 0; d >>= 1) s[k] += __shfl_xor_sync(0xFFFFFFFFu, s[k], d);
+    if (lane == 0) S.sum[wid][k] = s[k];
+  }
+  if (threadIdx.x == 0) S.best = ~0ull;
+  __syncthreads();
+  #pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    s[k] = lane < W ? S.sum[lane][k] : 0.0f;
+    #pragma unroll
+    for (int d = 16; d > 0; d >>= 1) s[k] += __shfl_xor_sync(0xFFFFFFFFu, s[k], d);
+    s[k] *= 1.0f / (float)BLOCK;
+  }
+  const float mx = s[0], my = s[1];
+  const float a = fmaxf(s[2] - mx * mx, 1.0f), d = fmaxf(s[4] - my * my, 1.0f), b = s[3] - mx * my;
+  const float l11 = sqrtf(a), l21 = b / l11, l22 = sqrtf(fmaxf(d - l21 * l21, 1.0e-8f * d));
+  StarFrame F;
+  F.m00 = 1.0f / l11;
+  F.m11 = 1.0f / l22;
+  F.m10 = -(l21 / l11) / l22;
+  const float u = (fx - mx) * F.m00, v = fmaf(fy - my, F.m11, (fx - mx) * F.m10);
+  const u32 r = __float_as_uint(fmaf(u, u, v * v)) & 0x7FFFFFFFu;
+  const u32 rm = __reduce_min_sync(0xFFFFFFFFu, r);
+  const u32 who = __ballot_sync(0xFFFFFFFFu, r == rm);
+  if (lane == __ffs(who) - 1) atomicMin(&S.best, ((u64)rm << 32) | (u64)threadIdx.x);
+  __syncthreads();
+  if ((u32)S.best == threadIdx.x) S.c = p;
+  __syncthreads();
+  F.cx = S.c.x;
+  F.cy = S.c.y;
+  return F;
+}
+
+// ---------------------------------------------------------------- sample polygon
+// The sample's candidates: per angular sector (kPolyDirs of them) the point
+// of the largest whitened radius (cand_key of the sample's position).  One
+// sector per sample: projecting every sample on every direction found the
+// same polygon at 30 times the instructions (8,500 cycles of a 1,024-thread
+// block for 2,048 samples).
+__device__ __forceinline__ void offer_sample(const StarFrame& F, int2 p, u32 pos, u64* best) {
+  float u, v;
+  to_uv(F, p.x - F.cx, p.y - F.cy, u, v);
+  const u64 k = cand_key(u, v, pos);
+  u64* slot = &best[bin_of<kPolyDirs>(u, v)];
+  if (k > *(volatile u64*)slot) atomicMax(slot, k);
+}
+
+struct PolySmem {
+  int2 p[kPolyDirs];                    // candidates by sector
+  u32 has[2];                           // sectors with one
+  int hx[kPolyDirs + 2], hy[kPolyDirs + 2];
+  float slope[kPolyDirs + 2];
+  int k, ir, ymin, ymax;
+};
+
+// The polygon of the candidates (in angular order about c) and the table of
+// its x slabs (see PolyHead).  Whole block; S.p and S.has are written and
+// visible; `tab` (shared or global) gets at most `slabs` words.
+//
+// Warp 0 reduces the candidates to a convex polygon by rounds (the rule of
+// list_hull, the alive sectors in one 64-bit mask) and verifies it; a set
+// that does not verify gets no polygon (nothing is dropped).
+//
+// Lower chain: corners 0 .. ir, x non-decreasing; upper chain: corners
+// ir .. k (corner k = corner 0), x non-increasing.  The lower chain is
+// convex and the upper one concave, so over a slab's columns their extreme
+// values lie at its ends; a slab of several columns takes the first column of
+// the next one as its end.  An edge's height over its start, p = slope (x -
+// x_e), carries at most 6 x 2^-24 of relative error (two conversions and the
+// division of the slope, one conversion, two roundings), so with e = |p|
+// 2^-21 the chain lies below y_e + floor(p + e) + 1 and above y_e + ceil(p -
+// e) - 1: integer heights strictly between floor(p + e) of the lower edge
+// and ceil(p - e) of the upper one are strictly inside.  For small
+// coordinates that is the exact test.  The heights are stored in 16 bits, in
+// units of 2^shy rounded inwards.
+template <int BLOCK>
+__device__ PolyHead build_poly(PolySmem& S, const StarFrame& F, u32* tab, u32 slabs) {
+  static_assert(kPolyDirs == 64, "two candidates per lane of a warp, one mask word");
+  const int lane = threadIdx.x & 31, t = threadIdx.x;
+  PolyHead H;
+  H.ok = 0; H.x1 = 0; H.xw = 0; H.sh = 0; H.y0 = 0; H.shy = 0; H.nslab = 0;
+  if (t < 32) {
+    u64 alive = ((u64)S.has[1] << 32) | S.has[0];
+    auto rel = [&](int j) { const int2 p = S.p[j]; return make_int2(p.x - F.cx, p.y - F.cy); };
+    bool ok = false;
+    for (int round = 0; round < 64 && __popcll(alive) >= 3; ++round) {
+      u32 drop[2], bad = 0;
+      #pragma unroll
+      for (int w = 0; w < 2; ++w) {
+        const int j = lane + 32 * w;
+        bool d = false;
+        if ((alive >> j) & 1ull) {
+          const u64 below = alive & ((1ull << j) - 1ull), above = j < 63 ? alive >> (j + 1) << (j + 1) : 0ull;
+          const int pj = 63 - __clzll((long long)(below ? below : above));
+          const int nj = __ffsll((long long)(above ? above : below)) - 1;
+          const int2 a = rel(pj), b = rel(nj), q = rel(j);
+          const long long ab = cross2(a.x, a.y, b.x, b.y);
+          const long long aq = cross2(a.x, a.y, q.x, q.y), qb = cross2(q.x, q.y, b.x, b.y);
+          const long long o = ab - aq - qb;
+          d = ab > 0 && aq >= 0 && qb >= 0 && (o > 0 || (o == 0 && aq > 0 && qb > 0));
+          bad |= !(aq > 0 && qb > 0 && o < 0) || out_of_range(S.p[j].x, S.p[j].y);
+        }
+        drop[w] = __ballot_sync(0xFFFFFFFFu, d);
+      }
+      if (!(drop[0] | drop[1])) {
+        ok = !__any_sync(0xFFFFFFFFu, bad != 0u);
+        break;
+      }
+      alive &= ~(((u64)drop[1] << 32) | drop[0]);
+    }
+    // Corners from the lexicographic minimum on.
+    const int k = ok ? __popcll(alive) : 0;
+    if (ok) {
+      auto lex = [&](int j) {
+        const int2 p = S.p[j];
+        return ((u64)((u32)p.x ^ 0x80000000u) << 32) | (u64)((u32)p.y ^ 0x80000000u);
+      };
+      u64 mn = ~0ull, mx = 0ull;
+      int ylo = 0x7FFFFFFF, yhi = (int)0x80000000;
+      #pragma unroll
+      for (int w = 0; w < 2; ++w) {
+        const int j = lane + 32 * w;
+        if ((alive >> j) & 1ull) {
+          const u64 v = lex(j);
+          mn = v < mn ? v : mn; mx = v > mx ? v : mx;
+          ylo = min(ylo, S.p[j].y); yhi = max(yhi, S.p[j].y);
+        }
+      }
+      #pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const u64 a = __shfl_xor_sync(0xFFFFFFFFu, mn, o), b = __shfl_xor_sync(0xFFFFFFFFu, mx, o);
+        mn = a < mn ? a : mn; mx = b > mx ? b : mx;
+      }
+      ylo = __reduce_min_sync(0xFFFFFFFFu, ylo);
+      yhi = __reduce_max_sync(0xFFFFFFFFu, yhi);
+      int r0 = -1, r1 = -1;
+      #pragma unroll
+      for (int w = 0; w < 2; ++w) {
+        const int j = lane + 32 * w;
+        if ((alive >> j) & 1ull) {
+          const int r = __popcll(alive & ((1ull << j) - 1ull));
+          if (lex(j) == mn) r0 = r;
+          if (lex(j) == mx) r1 = r;
+        }
+      }
+      r0 = __reduce_max_sync(0xFFFFFFFFu, r0);
+      r1 = __reduce_max_sync(0xFFFFFFFFu, r1);
+      #pragma unroll
+      for (int w = 0; w < 2; ++w) {
+        const int j = lane + 32 * w;
+        if ((alive >> j) & 1ull) {
+          const int r = __popcll(alive & ((1ull << j) - 1ull)) - r0, q = r < 0 ? r + k : r;
+          S.hx[q] = S.p[j].x; S.hy[q] = S.p[j].y;
+        }
+      }
+      __syncwarp();
+      for (int e = lane; e < k; e += 32) {
+        const int en = e + 1 < k ? e + 1 : 0;
+        const int dx = S.hx[en] - S.hx[e];
+        S.slope[e] = dx != 0 ? (float)(S.hy[en] - S.hy[e]) / (float)dx : 0.0f;    // vertical edges are never active
+      }
+      if (lane == 0) { S.ir = r1 >= r0 ? r1 - r0 : r1 - r0 + k; S.ymin = ylo; S.ymax = yhi; S.hx[k] = S.hx[0]; }
+    }
+    if (lane == 0) S.k = k;
+  }
+  __syncthreads();
+  const int k = S.k;
+  if (k < 3) return H;
+  const int ir = S.ir, xl = S.hx[0], xr = S.hx[ir], ymin = S.ymin, ymax = S.ymax;
+  if (xr - xl < 2 || ymax - ymin < 2) return H;
+  H.x1 = xl + 1;
+  H.xw = (u32)(xr - xl - 1);          // interior columns x1 .. x1 + xw - 1
+  while ((H.xw - 1u) >> H.sh >= slabs) ++H.sh;
+  H.nslab = ((H.xw - 1u) >> H.sh) + 1u;
+  H.y0 = ymin;
+  while ((u32)(ymax - ymin) >> H.shy > 65534u) ++H.shy;
+  H.ok = 1;
+  // A thread takes a run of slabs: along it the active lower edge le (x(le)
+  // < x <= x(le + 1)) only moves forward and the active upper edge ue (x(ue)
+  // > x >= x(ue + 1)) only backward.
+  const u32 per = (H.nslab + BLOCK - 1) / BLOCK;
+  const u32 s0 = t * per, s1 = min(H.nslab, s0 + per);
+  if (s0 >= s1) return H;
+  auto column = [&](u32 s) { return H.x1 + (int)min(H.xw - 1u, s << H.sh); };
+  int le = 0, ue = ir;
+  {
+    const int x = column(s0);
+    for (int hi = ir - 1; le < hi;) {
+      const int mid = (le + hi) >> 1;
+      if (S.hx[mid + 1] < x) le = mid + 1; else hi = mid;
+    }
+    for (int hi = k - 1; ue < hi;) {
+      const int mid = (ue + hi + 1) >> 1;
+      if (S.hx[mid] > x) ue = mid; else hi = mid - 1;
+    }
+  }
+  int lx = S.hx[le], lend = S.hx[le + 1], ly = S.hy[le];
+  int ux = S.hx[ue], uy = S.hy[ue];
+  float ls = S.slope[le], us = S.slope[ue];
+  auto heights = [&](int x, int& lo, int& hi) {
+    while (le < ir - 1 && lend < x) { ++le; lx = lend; lend = S.hx[le + 1]; ly = S.hy[le]; ls = S.slope[le]; }
+    while (ue > ir && ux <= x) { --ue; ux = S.hx[ue]; uy = S.hy[ue]; us = S.slope[ue]; }
+    const float p = __fmul_rn((float)(x - lx), ls), q = __fmul_rn((float)(x - ux), us);
+    lo = ly + (int)floorf(fmaf(fabsf(p), 4.76837158e-7f, p));
+    hi = uy + (int)ceilf(fmaf(fabsf(q), -4.76837158e-7f, q));
+  };
+  int lo0, hi0;
+  heights(column(s0), lo0, hi0);
+  for (u32 s = s0; s < s1; ++s) {
+    int lo1 = lo0, hi1 = hi0;
+    if (H.sh) heights(column(s + 1), lo1, hi1);      // past the last slab: its own last column
+    const int ylo = max(max(lo0, lo1), ymin), yhi = min(min(hi0, hi1), ymax);
+    u32 w = 0;
+    if (ylo < yhi) {
+      const u32 A = ((u32)(ylo - ymin) >> H.shy) + 1u, B = (u32)(yhi - ymin) >> H.shy;
+      if (B > A) w = A | ((B - A) << 16);
+    }
+    tab[s] = w;
+    if (!H.sh && s + 1 < s1) heights(column(s + 1), lo1, hi1);
+    lo0 = lo1; hi0 = hi1;
+  }
+  return H;
+}
+
+// Strictly inside the sample polygon (its table): word w holds the first
+// inside height unit (low half) and their number (high half).
+__device__ __forceinline__ bool inside_poly(const PolyHead& H, const u32* tab, int x, int y) {
+  const u32 xo = (u32)(x - H.x1);
+  u32 w = 0;
+  if (xo < H.xw) w = tab[xo >> H.sh];
+  return ((u32)(y - H.y0) >> H.shy) - (w & 0xFFFFu) < (w >> 16);
+}
+
+// ---------------------------------------------------------------- the stream
+// Where a warp puts the points on or outside the polygon: its slice of
+// SLICE staged points, flushed with one atomic reservation into (rxy, ridx),
+// in no particular order; every flushed point is offered as the candidate of
+// its angular bin.
+template <int NB, int SLICE>
+struct RawSink {
+  int2* sxy;
+  u32* sidx;
+  u32 fill;                 // uniform over the warp
+  const StarFrame* frame;
+  u32* raw_count;
+  u32* error;
+  u64* key;
+  int2* rxy;
+  u32* ridx;
+  u32 bound;                // capacity of (rxy, ridx)
+
+  __device__ __forceinline__ void flush() {
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    u32 base = 0;
+    if (lane == 0) base = atomicAdd(raw_count, fill);
+    base = __shfl_sync(0xFFFFFFFFu, base, 0);
+    const StarFrame F = *frame;
+    for (u32 q = lane; q < fill; q += 32) {
+      const int2 p = sxy[q];
+      const u32 id = sidx[q];
+      if (base + q < bound) { rxy[base + q] = p; ridx[base + q] = id; }
+      if (out_of_range(p.x, p.y)) atomicOr(error, ERR_RANGE);
+      float u, v;
+      to_uv(F, p.x - F.cx, p.y - F.cy, u, v);
+      const u64 k = cand_key(u, v, id);
+      u64* slot = &key[bin_of<NB>(u, v)];
+      if (k > __ldcg(slot)) atomicMax(slot, k);
+    }
+    __syncwarp();
+    fill = 0;
+  }
+  // One point per lane (the whole warp calls it; out: the point survives).
+  __device__ __forceinline__ void push(bool out, int x, int y, u32 id) {
+    const u32 bal = __ballot_sync(0xFFFFFFFFu, out);
+    if (bal) {
+      if (out) {
+        const u32 q = fill + __popc(bal & ((1u << (threadIdx.x & 31)) - 1u));
+        sxy[q] = make_int2(x, y);
+        sidx[q] = id;
+      }
+      fill += __popc(bal);
+      if (fill > (u32)SLICE - 32u) flush();
+    }
+  }
+};
+
+// The stream's sink of a block that finishes its points itself: its list.
+template <class L>
+struct ListSink {
+  L* list;
+  u32* count;
+  u32 cap;
+  bool bad;                 // a coordinate out of range
+  __device__ __forceinline__ void push(bool out, int x, int y, u32 id) {
+    const u32 bal = __ballot_sync(0xFFFFFFFFu, out);
+    if (bal) {
+      const int lane = threadIdx.x & 31;
+      u32 base = 0;
+      if (lane == 0) base = atomicAdd(count, (u32)__popc(bal));
+      base = __shfl_sync(0xFFFFFFFFu, base, 0) + __popc(bal & ((1u << lane) - 1u));
+      if (out) {
+        if (base < cap) { list->p[base] = make_int2(x, y); list->id[base] = id; }
+        bad = bad || out_of_range(x, y);
+      }
+    }
+  }
+};
+
+// Streams the points Q[0, cnt) (indices id0 ..) through the polygon's test:
+// this warp takes the rounds of 32 V pairs that start at pair 32 V (first +
+// k step).  The next round's loads go out before a round is tested; prep()
+// runs after the first loads are issued (it fills `tab` and has the block's
+// barrier).  Q starts on any row: the point before its 16-byte boundary and
+// the odd last one go to warp 0's lanes.
+template <int V, class Sink, class Prep>
+__device__ __forceinline__ void stream_points(const int2* __restrict__ Q, u32 cnt, u32 id0, u32 first, u32 step,
+                                              const PolyHead& H, const u32* tab, Sink& sink, Prep prep) {
+  const int lane = threadIdx.x & 31;
+  const u32 head = (reinterpret_cast<uintptr_t>(Q) & 15u) && cnt ? 1u : 0u;
+  const int4* p4 = reinterpret_cast<const int4*>(Q + head);
+  const u32 npair = (cnt - head) >> 1;
+  constexpr u32 R = 32u * V;
+  u32 w0 = first * R;                             // the warp's first pair of the round
+  int4 cur[V];
+  if (w0 + R <= npair) {
+    #pragma unroll
+    for (int u = 0; u < V; ++u) cur[u] = p4[w0 + lane + 32u * u];
+  }
+  prep();
+  while (w0 + R <= npair) {
+    const u32 w1 = w0 + step * R;
+    int4 nxt[V];
+    if (w1 + R <= npair) {
+      #pragma unroll
+      for (int u = 0; u < V; ++u) nxt[u] = p4[w1 + lane + 32u * u];
+    }
+    #pragma unroll
+    for (int u = 0; u < V; ++u) {
+      const u32 id = id0 + head + 2u * (w0 + lane + 32u * u);
+      sink.push(!inside_poly(H, tab, cur[u].x, cur[u].y), cur[u].x, cur[u].y, id);
+      sink.push(!inside_poly(H, tab, cur[u].z, cur[u].w), cur[u].z, cur[u].w, id + 1u);
+    }
+    #pragma unroll
+    for (int u = 0; u < V; ++u) cur[u] = nxt[u];
+    w0 = w1;
+  }
+  // The last, partial round (one warp has it).
+  for (u32 b = w0; b < min(npair, w0 + R); b += 32u) {
+    const u32 j = b + lane;
+    const bool in = j < npair;
+    const int4 w = in ? p4[j] : make_int4(0, 0, 0, 0);
+    const u32 id = id0 + head + 2u * j;
+    sink.push(in && !inside_poly(H, tab, w.x, w.y), w.x, w.y, id);
+    sink.push(in && !inside_poly(H, tab, w.z, w.w), w.z, w.w, id + 1u);
+  }
+  if (first == 0) {
+    const u32 rest = (cnt - head) & 1u;
+    const bool in = lane < 2 && (lane == 0 ? head : rest) != 0u;
+    const u32 j = lane == 0 ? 0u : cnt - 1u;
+    const int2 p = in ? Q[j] : make_int2(0, 0);
+    sink.push(in && !inside_poly(H, tab, p.x, p.y), p.x, p.y, id0 + j);
+  }
+}
+
+// ---------------------------------------------------------------- candidates
+// Candidate points of the angular bins: cand / cid with the occupancy bits.
+template <int NB>
+struct CandTab {
+  int2 cand[NB];
+  u32 cid[NB];
+  u32 occ[NB / 32];
+};
+// Nearest occupied bin after / before b, cyclically (b itself last); some
+// bin is occupied.
+template <int NB>
+__device__ __forceinline__ u32 next_bin(const u32* occ, u32 b) {
+  constexpr u32 NW = NB / 32;
+  u32 w = b >> 5;
+  u32 m = (b & 31u) == 31u ? 0u : occ[w] & (0xFFFFFFFFu << ((b & 31u) + 1u));
+  for (u32 it = 0; it < NW && m == 0u; ++it) { w = (w + 1u) & (NW - 1u); m = occ[w]; }
+  return m ? (w << 5) + (u32)__ffs(m) - 1u : b;
+}
+template <int NB>
+__device__ __forceinline__ u32 prev_bin(const u32* occ, u32 b) {
+  constexpr u32 NW = NB / 32;
+  u32 w = b >> 5;
+  u32 m = occ[w] & ((1u << (b & 31u)) - 1u);
+  for (u32 it = 0; it < NW && m == 0u; ++it) { w = (w + NW - 1u) & (NW - 1u); m = occ[w]; }
+  return m ? (w << 5) + 31u - (u32)__clz(m) : b;
+}
+
+// Point (x, y) with index id in bin b: dropped by its wedge of the candidate
+// polygon?
+template <int NB>
+__device__ __forceinline__ bool dropped_by_cands(const CandTab<NB>& C, const StarFrame& F, u32 b, int x, int y,
+                                                 u32 id) {
+  const int2 q = make_int2(x - F.cx, y - F.cy);
+  u32 ba, bb;
+  if ((C.occ[b >> 5] >> (b & 31u)) & 1u) {
+    const int2 p = C.cand[b];
+    const bool after = cross2(p.x - F.cx, p.y - F.cy, q.x, q.y) >= 0;
+    ba = after ? b : prev_bin<NB>(C.occ, b);
+    bb = after ? next_bin<NB>(C.occ, b) : b;
+  } else {
+    ba = prev_bin<NB>(C.occ, b);
+    bb = next_bin<NB>(C.occ, b);
+  }
+  const int2 A = C.cand[ba], B = C.cand[bb];
+  if ((x == A.x && y == A.y && id > C.cid[ba]) || (x == B.x && y == B.y && id > C.cid[bb])) return true;
+  return dropped_by(make_int2(A.x - F.cx, A.y - F.cy), make_int2(B.x - F.cx, B.y - F.cy), q);
+}
+
+// ---------------------------------------------------------------- hull of a list
+constexpr u32 kBinMax = 192;       // most points of one bin ordered by counting
+constexpr int kRounds = 48;        // most rounds
+
+// p, id: the points (any order) and their input indices, [0, CAP).  ta holds
+// the positions of the m points to start from.
+template <int BLOCK, int CAP, int NB>
+struct ListSmem {
+  int2 p[CAP];
+  u32 id[CAP];
+  unsigned short bn[CAP];
+  unsigned short ta[CAP], tb[CAP];
+  u32 cnt[NB], cur[NB];
+  u32 ws[2][BLOCK / 32];
+  u64 first;
+  u32 flag;
+};
+
+// The hull of the m points named by S.ta (the whole block; S.p, S.id, S.ta
+// written and visible).  Returns its number of vertices, written as input
+// indices counter-clockwise from the lexicographic minimum into out[0, cap)
+// (nothing when it exceeds cap), or -1: not decided here.
+template <int BLOCK, int CAP, int NB>
+__device__ int list_hull(ListSmem<BLOCK, CAP, NB>& S, u32 m, const StarFrame& F, int* out, long long cap) {
+  static_assert(NB % BLOCK == 0 || BLOCK % NB == 0, "whole bins per thread");
+  static_assert(CAP <= 32768, "a position and a flag in 16 bits");
+  constexpr int PER = NB / BLOCK > 0 ? NB / BLOCK : 1;
+  const int t = threadIdx.x;
+  if (m < 3 || m > (u32)CAP) return -1;
+  for (int b = t; b < NB; b += BLOCK) S.cnt[b] = 0u;
+  if (t == 0) { S.flag = 0u; S.first = ~0ull; }
+  __syncthreads();
+  for (u32 i = t; i < m; i += BLOCK) {
+    const u32 k = S.ta[i];
+    const int2 p = S.p[k];
+    float u, v;
+    to_uv(F, p.x - F.cx, p.y - F.cy, u, v);
+    const u32 b = bin_of<NB>(u, v);
+    S.bn[k] = (unsigned short)b;
+    if (atomicAdd(&S.cnt[b], 1u) >= kBinMax) S.flag = 1u;
+  }
+  __syncthreads();
+  if (S.flag) return -1;
+  {
+    u32 c[PER], sum = 0, tot;
+    #pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      const int b = t * PER + j;
+      c[j] = b < NB ? S.cnt[b] : 0u;
+      sum += c[j];
+    }
+    u32 ex = block_scan<BLOCK>(sum, S.ws[0], tot);
+    #pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      const int b = t * PER + j;
+      if (b < NB) S.cur[b] = ex;
+      ex += c[j];
+    }
+  }
+  __syncthreads();
+  for (u32 i = t; i < m; i += BLOCK) {
+    const unsigned short k = S.ta[i];
+    S.tb[atomicAdd(&S.cur[S.bn[k]], 1u)] = k;       // cur[b] ends at the bin's end
+  }
+  __syncthreads();
+  // Order inside the bins by counting: counter-clockwise about c, along a
+  // ray the farther first, equal points by index.  All but the first of a
+  // ray are marked (bit 15): nearer points of a ray are no vertices.
+  for (u32 i = t; i < m; i += BLOCK) {
+    const u32 k = S.tb[i], b = S.bn[k];
+    const u32 e = S.cur[b], s = e - S.cnt[b];
+    const int2 p = S.p[k];
+    const int2 q = make_int2(p.x - F.cx, p.y - F.cy);
+    const u32 qr = (u32)abs(q.x) + (u32)abs(q.y), qi = S.id[k];
+    u32 r = 0;
+    bool dead = q.x == 0 && q.y == 0;
+    for (u32 j = s; j < e; ++j) {
+      if (j == i) continue;
+      const u32 kj = S.tb[j];
+      const int2 w = S.p[kj];
+      const int2 d = make_int2(w.x - F.cx, w.y - F.cy);
+      const long long c = cross2(d.x, d.y, q.x, q.y);
+      if (c > 0) { ++r; continue; }
+      if (c < 0) continue;
+      const u32 dr = (u32)abs(d.x) + (u32)abs(d.y);
+      if (dr > qr || (dr == qr && S.id[kj] < qi)) { ++r; dead = true; }
+    }
+    S.ta[min(s + r, m - 1u)] = (unsigned short)(k | (dead ? 0x8000u : 0u));
+  }
+  __syncthreads();
+  // Rounds: thread t owns a run of consecutive entries.
+  unsigned short* cur = S.ta;
+  unsigned short* nxt = S.tb;
+  u32 par = 1;
+  bool done = false;
+  auto rel = [&](u32 k) { const int2 p = S.p[k]; return make_int2(p.x - F.cx, p.y - F.cy); };
+  for (int round = 0; round <= kRounds; ++round) {
+    const u32 per = (m + BLOCK - 1) / BLOCK;
+    const u32 i0 = min(m, t * per), i1 = min(m, i0 + per);
+    u32 kept = 0, mask = 0;       // per <= CAP / BLOCK <= 32
+    static_assert(CAP / BLOCK <= 32, "one mask bit per owned entry");
+    bool bad = false;
+    for (u32 i = i0; i < i1; ++i) {
+      const u32 k = cur[i];
+      bool keep;
+      if (round == 0) {
+        keep = !(k & 0x8000u);
+      } else {
+        const int2 q = rel(k);
+        const int2 a = rel(cur[i > 0 ? i - 1 : m - 1]), b = rel(cur[i + 1 < m ? i + 1 : 0]);
+        const long long ab = cross2(a.x, a.y, b.x, b.y);
+        const long long aq = cross2(a.x, a.y, q.x, q.y), qb = cross2(q.x, q.y, b.x, b.y);
+        const long long o = ab - aq - qb;
+        keep = !(ab > 0 && aq >= 0 && qb >= 0 && (o > 0 || (o == 0 && aq > 0 && qb > 0)));
+        // A vertex of the verified polygon: c strictly left of both its
+        // edges, a strict left turn (o < 0).
+        bad = bad || !(aq > 0 && qb > 0 && o < 0);
+        if (keep && round <= 3 && m > 8) {
+          // A wider wedge drops runs of points in fewer rounds.
+          const int2 a2 = rel(cur[i >= 2 ? i - 2 : i + m - 2]), b2 = rel(cur[i + 2 < m ? i + 2 : i + 2 - m]);
+          keep = !dropped_by(a2, b2, q);
+        }
+      }
+      if (keep) { mask |= 1u << (i - i0); ++kept; }
+    }
+    u32 tot;
+    u32 pos = block_scan<BLOCK>(kept, S.ws[par], tot);
+    par ^= 1u;
+    if (round > 0 && tot == m) {         // uniform: nothing dropped
+      done = !__syncthreads_or(bad);
+      break;
+    }
+    for (u32 i = i0; i < i1; ++i)
+      if ((mask >> (i - i0)) & 1u) nxt[pos++] = cur[i];
+    __syncthreads();
+    unsigned short* w = cur; cur = nxt; nxt = w;
+    m = tot;
+    if (m < 3) return -1;
+  }
+  if (!done) return -1;
+  // The lexicographic minimum starts the output.
+  auto lex = [&](u32 i) {
+    const int2 p = S.p[cur[i]];
+    return ((u64)((u32)p.x ^ 0x80000000u) << 32) | (u64)((u32)p.y ^ 0x80000000u);
+  };
+  u64 mn = ~0ull;
+  for (u32 i = t; i < m; i += BLOCK) { const u64 v = lex(i); mn = v < mn ? v : mn; }
+  {
+    const u32 hi = __reduce_min_sync(0xFFFFFFFFu, (u32)(mn >> 32));
+    const u32 lo = __reduce_min_sync(0xFFFFFFFFu, (u32)(mn >> 32) == hi ? (u32)mn : 0xFFFFFFFFu);
+    if ((t & 31) == 0 && (t & ~31) < (int)m) atomicMin(&S.first, ((u64)hi << 32) | lo);
+  }
+  __syncthreads();
+  const u64 f = S.first;
+  for (u32 i = t; i < m; i += BLOCK)
+    if (lex(i) == f) S.flag = i;              // one vertex: they are distinct
+  __syncthreads();
+  const u32 st = S.flag;
+  if ((long long)m <= cap)
+    for (u32 i = t; i < m; i += BLOCK) {
+      const u32 j = st + i;
+      out[i] = (int)S.id[cur[j < m ? j : j - m]];
+    }
+  return (int)m;
+}
+
+// The candidates of the list S.p[0, m0) and the points that they do not
+// drop: their positions to S.ta, their number returned (the whole block;
+// key: NB words of scratch).
+template <int BLOCK, int CAP, int NB>
+__device__ u32 filter_list(ListSmem<BLOCK, CAP, NB>& S, u32 m0, const StarFrame& F, u64* key, CandTab<NB>& C) {
+  const int t = threadIdx.x;
+  for (int b = t; b < NB; b += BLOCK) key[b] = 0ull;
+  for (int b = t; b < NB / 32; b += BLOCK) C.occ[b] = 0u;
+  if (t == 0) S.flag = 0u;
+  __syncthreads();
+  for (u32 i = t; i < m0; i += BLOCK) {
+    const int2 p = S.p[i];
+    float u, v;
+    to_uv(F, p.x - F.cx, p.y - F.cy, u, v);
+    const u32 b = bin_of<NB>(u, v);
+    const u64 k = cand_key(u, v, S.id[i]);
+    S.bn[i] = (unsigned short)b;
+    if (k > *(volatile u64*)&key[b]) atomicMax(&key[b], k);
+  }
+  __syncthreads();
+  for (u32 i = t; i < m0; i += BLOCK) {
+    const u32 b = S.bn[i], id = S.id[i];
+    if ((u32)key[b] == ~id) {
+      C.cand[b] = S.p[i];
+      C.cid[b] = id;
+      atomicOr(&C.occ[b >> 5], 1u << (b & 31u));
+    }
+  }
+  __syncthreads();
+  const int lane = t & 31;
+  for (u32 i0 = 0; i0 < m0; i0 += BLOCK) {
+    const u32 i = i0 + t;
+    bool keep = false;
+    if (i < m0) {
+      const int2 p = S.p[i];
+      keep = !dropped_by_cands<NB>(C, F, S.bn[i], p.x, p.y, S.id[i]);
+    }
+    const u32 bal = __ballot_sync(0xFFFFFFFFu, keep);
+    u32 base = 0;
+    if (lane == 0 && bal) base = atomicAdd(&S.flag, (u32)__popc(bal));
+    base = __shfl_sync(0xFFFFFFFFu, base, 0);
+    if (keep) S.ta[base + __popc(bal & ((1u << lane) - 1u))] = (unsigned short)i;
+  }
+  __syncthreads();
+  const u32 m = S.flag;
+  __syncthreads();
+  return m;
+}
+
+}  // namespace star
+}  // namespace gbh
