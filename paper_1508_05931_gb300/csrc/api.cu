@@ -77,7 +77,8 @@ struct BatchWs {
   long long* slot0 = nullptr;
   int* order = nullptr;
   u32* hcount = nullptr;
-  u32* ctl = nullptr;          // [0], [1]: queues; [2]: error bits
+  int* redo = nullptr;         // instances that the star path did not decide
+  u32* ctl = nullptr;          // [0], [1], [3], [4], [6]: queues; [2]: error bits; [5]: number of `redo`
   // pinned host staging
   size_t h_cap = 0;
   long long* h_off = nullptr;
@@ -96,6 +97,7 @@ struct BatchWs {
 };
 
 constexpr int64_t kSmallInstance = 16384;   // size bucket boundary
+constexpr int64_t kStarSmall = 16384;       // star path: instances up to this size take one block each
 // Instances of this many points or more take the segmented path (flat
 // streaming passes over all their tiles) unless the autotuner chose another
 // boundary among kSegCandidates (the last one: no instance takes it).
@@ -693,6 +695,7 @@ hull_status hull_create(hull_ctx** out, int device, const hull_config* cfg) {
   if (k2_configure() != cudaSuccess || k3_configure() != cudaSuccess || bucket_configure() != cudaSuccess ||
       fused_configure() != cudaSuccess || fused_occupancy(&c->occ_kf) != cudaSuccess ||
       k1_poly_configure() != cudaSuccess || star_configure() != cudaSuccess ||
+      batch_star_configure() != cudaSuccess ||
       bucket_occupancy(&c->occ_kb) != cudaSuccess ||
       split_occupancy(&c->occ_sp) != cudaSuccess ||
       k5_configure(&c->occ_k5) != cudaSuccess ||
@@ -1705,7 +1708,7 @@ hull_status hull_compute_batched(hull_ctx* c, const int32_t* d_xy, const int64_t
     const size_t bytes = cs * (8 + 8 + 4 + 4 + 8 + 4 + 8 + 4 + 4);
     const size_t cb = (size_t)B + 1024;
     if (cudaMalloc(&w.base, bytes) != cudaSuccess ||
-        cudaMalloc(&w.slot0, cb * 8 + cb * 4 + cb * 4 + 256) != cudaSuccess) {
+        cudaMalloc(&w.slot0, cb * 8 + cb * 4 + cb * 4 + cb * 4 + 256) != cudaSuccess) {
       cudaGetLastError();
       if (w.base) cudaFree(w.base);
       w.base = nullptr;
@@ -1724,7 +1727,8 @@ hull_status hull_compute_batched(hull_ctx* c, const int32_t* d_xy, const int64_t
     char* t = reinterpret_cast<char*>(w.slot0);
     w.order = reinterpret_cast<int*>(t + cb * 8);
     w.hcount = reinterpret_cast<u32*>(t + cb * 8 + cb * 4);
-    w.ctl = reinterpret_cast<u32*>(t + cb * 16);
+    w.redo = reinterpret_cast<int*>(t + cb * 16);
+    w.ctl = reinterpret_cast<u32*>(t + cb * 20);
     w.cap_slots = cs;
     w.cap_b = (size_t)B;
   }
@@ -1736,7 +1740,7 @@ hull_status hull_compute_batched(hull_ctx* c, const int32_t* d_xy, const int64_t
     w.seg = nullptr; w.cap_tiles = 0; w.cap_seg = 0;
     const size_t ct = (size_t)tiles_all + 1024, cb = (size_t)B + 1024;
     const size_t b_text = align_up(ct * seg_text_bytes(), 256), b_tcnt = align_up(ct * 4, 256);
-    const size_t b_rec = align_up(cb * seg_rec_bytes(), 256), b_tf = align_up((cb + 1) * 4, 256);
+    const size_t b_rec = align_up(cb * std::max(seg_rec_bytes(), batch_star_rec_bytes()), 256), b_tf = align_up((cb + 1) * 4, 256);
     if (cudaMalloc(&w.seg, b_text + b_tcnt + b_rec + b_tf) != cudaSuccess) {
       cudaGetLastError();
       w.seg = nullptr;
@@ -1753,16 +1757,19 @@ hull_status hull_compute_batched(hull_ctx* c, const int32_t* d_xy, const int64_t
   e = cudaMemcpyAsync(w.slot0, w.h_slot0, (size_t)B * 8, cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) return cuda_fail(e);
 
+  // The general path, for the instances of `todo` (every one on the first
+  // call that autotunes, then those that the star path does not decide).
   // Size buckets: the segmented path (seg_min points or more), large
   // (more than kSmallInstance) and small instances; `order` lists them in
   // that order, each bucket largest first.  The host arrays are rewritten
   // only after the stream has finished the copies of the previous layout.
   int nh = 0, nl = 0, ns = 0, ntiles = 0;
+  std::vector<int> todo;
   auto layout = [&](int64_t seg_min) -> cudaError_t {
     cudaError_t r = cudaStreamSynchronize(st);
     if (r != cudaSuccess) return r;
     std::vector<int> huge, large, small;
-    for (int i = 0; i < B; ++i) {
+    for (int i : todo) {
       const int64_t ni = w.h_off[i + 1] - w.h_off[i];
       (ni >= seg_min ? huge : ni <= kSmallInstance ? small : large).push_back(i);
     }
@@ -1783,7 +1790,7 @@ hull_status hull_compute_batched(hull_ctx* c, const int32_t* d_xy, const int64_t
       ntiles += (int)((w.h_off[huge[h] + 1] - w.h_off[huge[h]] + tile - 1) / tile);
     }
     w.h_tfirst[nh] = ntiles;
-    r = cudaMemcpyAsync(w.order, w.h_order, (size_t)B * 4, cudaMemcpyHostToDevice, st);
+    r = cudaMemcpyAsync(w.order, w.h_order, todo.size() * 4, cudaMemcpyHostToDevice, st);
     if (r == cudaSuccess) r = cudaMemcpyAsync(w.tfirst, w.h_tfirst, ((size_t)nh + 1) * 4, cudaMemcpyHostToDevice, st);
     return r;
   };
@@ -1871,6 +1878,8 @@ hull_status hull_compute_batched(hull_ctx* c, const int32_t* d_xy, const int64_t
   if (c->cfg.autotune && (c->tuned_block[0] == 0 || c->tuned_block[1] == 0 || c->tuned_block[2] == 0 ||
                           (c->tuned_seg == 0 && !fixed_seg))) {
     autotune_load(c);
+    todo.resize(B);
+    std::iota(todo.begin(), todo.end(), 0);
     e = layout(seg_boundary());
     if (e != cudaSuccess) return cuda_fail(e);
     for (int bucket = 0; bucket < 3; ++bucket) {
@@ -1904,14 +1913,69 @@ hull_status hull_compute_batched(hull_ctx* c, const int32_t* d_xy, const int64_t
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e);
   }
-  e = layout(seg_boundary());
-  if (e == cudaSuccess) e = run_all();
-  if (e == cudaSuccess)
-    e = launch_batch_output(w.hcount, w.slot0, w.out_tmp, B, reinterpret_cast<long long*>(d_out_offsets),
-                            d_out, (long long)cap, w.ctl + 2, c->num_sms * 4, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(w.h_ctl, w.ctl, 16, cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e != cudaSuccess) return cuda_fail(e);
+  // The output: the hulls' offsets, every hull copied to its place, the
+  // error bits and the number of undecided instances read back.
+  auto output = [&]() -> cudaError_t {
+    cudaError_t r = launch_batch_output(w.hcount, w.slot0, w.out_tmp, B, reinterpret_cast<long long*>(d_out_offsets),
+                                        d_out, (long long)cap, w.ctl + 2, c->num_sms * 4, st);
+    if (r == cudaSuccess) r = cudaMemcpyAsync(w.h_ctl, w.ctl, 32, cudaMemcpyDeviceToHost, st);
+    return r == cudaSuccess ? cudaStreamSynchronize(st) : r;
+  };
+  // The star path: the large instances (in index order: their points are
+  // streamed in one flat pass) and the small ones, by falling size class so
+  // that the longest blocks start first.
+  {
+    const int64_t stile = batch_star_tile();
+    if (!todo.empty()) e = cudaStreamSynchronize(st);      // the autotuner's layout may still be copied
+    if (e != cudaSuccess) return cuda_fail(e);
+    BatchStar a{};
+    constexpr int kClasses = 65;        // leading zeros of the size: larger instances first, empty ones last
+    int first[kClasses] = {};
+    auto cls = [](int64_t n) { return n > 0 ? __builtin_clzll((unsigned long long)n) : kClasses - 1; };
+    for (int i = 0; i < B; ++i) {
+      const int64_t ni = w.h_off[i + 1] - w.h_off[i];
+      if (ni > kStarSmall) {
+        w.h_tfirst[a.nh] = a.ntiles;
+        a.ntiles += (int)((ni + stile - 1) / stile);
+        w.h_order[a.nh++] = i;
+      } else {
+        ++first[cls(ni)];
+      }
+    }
+    w.h_tfirst[a.nh] = a.ntiles;
+    a.ns = B - a.nh;
+    int at = a.nh;
+    for (int k = 0; k < kClasses; ++k) { const int cn = first[k]; first[k] = at; at += cn; }
+    for (int i = 0; i < B; ++i) {
+      const int64_t ni = w.h_off[i + 1] - w.h_off[i];
+      if (ni <= kStarSmall) w.h_order[first[cls(ni)]++] = i;
+    }
+    a.xy = d_xy; a.offsets = reinterpret_cast<const long long*>(d_offsets);
+    a.order = w.order; a.tfirst = w.tfirst; a.slot0 = w.slot0; a.kb = w.kb; a.ib = w.ib; a.rec = w.rec;
+    a.out_tmp = w.out_tmp; a.hcount = w.hcount; a.error = w.ctl + 2; a.queue = w.ctl + 6;
+    a.redo = w.redo; a.nredo = w.ctl + 5;
+    e = cudaMemcpyAsync(w.order, w.h_order, (size_t)B * 4, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(w.tfirst, w.h_tfirst, ((size_t)a.nh + 1) * 4, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(w.ctl, 0, 64, st);
+    if (e == cudaSuccess) e = cudaEventRecord(c->bev[0], st);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(c->aux, c->bev[0], 0);
+    if (e == cudaSuccess) e = launch_batch_star_large(a, c->num_sms, st);
+    if (e == cudaSuccess) e = launch_batch_star_small(a, c->num_sms, c->aux);
+    if (e == cudaSuccess) e = cudaEventRecord(c->bev[1], c->aux);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, c->bev[1], 0);
+    if (e == cudaSuccess) e = output();
+    if (e != cudaSuccess) return cuda_fail(e);
+  }
+  const u32 nredo = w.h_ctl[5];
+  if (nredo > 0 && nredo <= (u32)B && !(w.h_ctl[2] & ERR_RANGE)) {
+    todo.resize(nredo);
+    e = cudaMemcpyAsync(todo.data(), w.redo, (size_t)nredo * 4, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = layout(seg_boundary());      // waits for the stream first
+    if (e == cudaSuccess) e = run_all();
+    if (e == cudaSuccess) e = output();
+    if (e != cudaSuccess) return cuda_fail(e);
+  }
   const u32 err = w.h_ctl[2];
   if (err & ERR_RANGE) return HULL_ERANGE;
   if (err & ERR_INTERNAL) return HULL_EINTERNAL;

@@ -174,6 +174,34 @@ struct BatchLaunch {
   void* rec;          // per-instance plan, polygon edges and witness table
 };
 
+// The star path over a batch (batch_star.cu).  order: the nh large instances,
+// then the ns small ones; tfirst: first tile (batch_star_tile() points) of
+// every large instance; rec: nh records of batch_star_rec_bytes().  Hulls go
+// to out_tmp at slot0 with their sizes in hcount; the instances that it does
+// not decide are listed in redo[0, *nredo).
+struct BatchStar {
+  const int* xy;
+  const long long* offsets;
+  const int* order;
+  int nh, ns, ntiles;
+  const int* tfirst;
+  const long long* slot0;
+  u64* kb;
+  u32* ib;
+  void* rec;
+  int* out_tmp;
+  u32* hcount;
+  u32* error;
+  u32* queue;
+  int* redo;
+  u32* nredo;
+};
+int batch_star_tile();
+size_t batch_star_rec_bytes();
+cudaError_t batch_star_configure();
+cudaError_t launch_batch_star_small(const BatchStar& a, int num_sms, cudaStream_t st);
+cudaError_t launch_batch_star_large(const BatchStar& a, int num_sms, cudaStream_t st);
+
 int batch_pad();
 int seg_tile();             // points per tile of the segmented path
 size_t seg_rec_bytes();     // bytes of one instance's record
