@@ -54,6 +54,8 @@ struct Workspace {
   u32* fcur = nullptr;         // per bin: next position of the coarse-to-fine split
   u64* wkey = nullptr;         // per region and witness bin: the sample's best witness (follows bcnt)
   int2* sample = nullptr;      // every kSampleStride-th point (K1 or k0 copies them out)
+  void* sect = nullptr;        // sector tables of the star path (k_sector.cu)
+  bool poly_clear = false;     // the head of *poly is zero (k_star leaves it so when it decides)
   PolyTab* poly = nullptr;     // the single-read front's frame, polygon and candidates
   unsigned long long* key_or = nullptr;
 };
@@ -229,6 +231,7 @@ hull_status ensure_ws(hull_ctx* c, size_t n) {
   const size_t o_bcnt = take(((size_t)kBins + kCoarse) * 4);
   const size_t o_wkey = take((size_t)2 * kWitnessBins * 8);   // right after bcnt: one memset clears both
   const size_t o_poly = take(sizeof(PolyTab));
+  const size_t o_sect = take(sector_bytes());
   const size_t o_sample = take((cap / kSampleStride + 1) * 8);
   const size_t o_bagg = take(((size_t)kBins + kBinPrefixBlocks) * 16);
   const size_t o_bpre = take((size_t)kBins * 16);
@@ -279,6 +282,7 @@ hull_status ensure_ws(hull_ctx* c, size_t n) {
   w.fcur = reinterpret_cast<u32*>(b + o_fcur);
   w.wkey = reinterpret_cast<u64*>(b + o_wkey);
   w.poly = reinterpret_cast<PolyTab*>(b + o_poly);
+  w.sect = b + o_sect;
   w.sample = reinterpret_cast<int2*>(b + o_sample);
   return HULL_OK;
 }
@@ -300,8 +304,10 @@ enum Next { NEXT_NONE = 0, NEXT_BUCKET, NEXT_RADIX };
 // and returns HULL_OK without recording anything: the caller goes on.
 hull_status read_summary(hull_ctx* c, const Plan& p, Next* next);
 
-hull_status finish(hull_ctx* c, cudaStream_t st, Next* next = nullptr) {
-  cudaError_t e = cudaMemcpyAsync(c->h_plan, c->plan, kSummaryBytes, cudaMemcpyDeviceToHost, st);
+// `there`: the kernels wrote the summary to h_plan themselves.
+hull_status finish(hull_ctx* c, cudaStream_t st, Next* next = nullptr, bool there = false) {
+  cudaError_t e = cudaSuccess;
+  if (!there) e = cudaMemcpyAsync(c->h_plan, c->plan, kSummaryBytes, cudaMemcpyDeviceToHost, st);
   if (e != cudaSuccess) return cuda_fail(e);
   e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_fail(e);
@@ -366,28 +372,38 @@ bool star_eligible(const hull_ctx* c, u32 n) {
          (single_read(n) || !(c->cfg.proposal == 1 && c->have_weights));
 }
 
+// The star path's front: the frame and the sample polygon, then the pass
+// over the input; the raw survivors are left in the chain buffers.
+cudaError_t star_front(hull_ctx* c, const int32_t* d_xy, u32 n, cudaStream_t st) {
+  Workspace& w = c->ws;
+  cudaError_t e = w.poly_clear ? cudaSuccess : cudaMemsetAsync(w.poly, 0, kPolyClearBytes, st);
+  w.poly_clear = false;
+  if (e == cudaSuccess) e = launch_poly(d_xy, n, w.poly, c->num_sms, st);
+  mark(c, 1, st);
+  if (e == cudaSuccess)
+    e = launch_k1_poly(d_xy, n, w.poly, w.h_xy[0], reinterpret_cast<u32*>(w.h_idx[0]), c->num_sms, st);
+  return e;
+}
+
 // The star path: the frame and the sample polygon, the pass over the input
 // that drops the points strictly inside it and writes the rest (raw
 // survivors, 0.3 % of a uniform 20M disk) to the chain buffers, and the hull
-// of those; a small input in one launch.  Ends with the summary in the Plan.
+// of those; a small input in one launch.  The last kernel writes the summary
+// to `sum`, pinned host memory (no copy behind it).
 // Profile slots: 0 sample polygon, 1 the pass, 11 the hull.
-hull_status run_star(hull_ctx* c, const int32_t* d_xy, u32 n, int32_t* d_out, int64_t cap, cudaStream_t st) {
+hull_status run_star(hull_ctx* c, const int32_t* d_xy, u32 n, int32_t* d_out, int64_t cap, Plan* sum, cudaStream_t st) {
   Workspace& w = c->ws;
   mark(c, 0, st);
   cudaError_t e = cudaSuccess;
   if (single_read(n)) {
-    u32* ridx = reinterpret_cast<u32*>(w.h_idx[0]);
-    e = cudaMemsetAsync(w.poly, 0, kPolyClearBytes, st);
-    if (e == cudaSuccess) e = launch_poly(d_xy, n, w.poly, c->num_sms, st);
-    mark(c, 1, st);
-    if (e == cudaSuccess) e = launch_k1_poly(d_xy, n, w.poly, w.h_xy[0], ridx, c->num_sms, st);
+    e = star_front(c, d_xy, n, st);
     for (int p = 2; p <= 3 + kMaxPasses; ++p) mark(c, p, st);
     if (e == cudaSuccess)
-      e = launch_star(d_xy, n, w.poly, w.h_xy[0], ridx, w.h_xy[1], reinterpret_cast<u32*>(w.h_idx[1]), c->plan, d_out,
+      e = launch_star(d_xy, n, w.poly, w.h_xy[0], reinterpret_cast<const u32*>(w.h_idx[0]), w.h_xy[1], reinterpret_cast<u32*>(w.h_idx[1]), sum, d_out,
                       (long long)cap, c->num_sms, st);
   } else {
     for (int p = 1; p <= 3 + kMaxPasses; ++p) mark(c, p, st);
-    e = launch_small(d_xy, n, c->plan, d_out, (long long)cap, st);
+    e = launch_small(d_xy, n, sum, d_out, (long long)cap, st);
   }
   mark(c, 4 + kMaxPasses, st);
   return e == cudaSuccess ? HULL_OK : cuda_fail(e);
@@ -524,30 +540,55 @@ hull_status run_final(hull_ctx* c, const int2* lo_xy, const int* lo_idx, const i
   return HULL_OK;
 }
 
-// One hull from a given step on: the star path, the bucket sort (on the raw
-// survivors that the star path left in this workspace, FROM_RAW), the radix
-// passes.  Each goes on to the next when it does not decide: the star path
-// on lists beyond one block and degenerate inputs, the bucket sort on a bin
-// it cannot sort in shared memory (heavily duplicated or extremely
-// clustered input); the radix passes take any input.
-enum From { FROM_STAR = 0, FROM_RAW, FROM_BUCKET, FROM_RADIX };
+// One hull from a given step on.  The star path goes on with the sectors
+// when its points are too many for one block (on the raw survivors that it
+// left in this workspace, or behind its front for a small input), and with
+// the bucket sort when it does not decide (degenerate inputs, crowded
+// angles); the bucket sort goes on with the radix passes when a bin is too
+// large for it (heavily duplicated or extremely clustered input); those take
+// any input.
+enum From { FROM_STAR = 0, FROM_FRONT, FROM_SECTORS, FROM_RAW, FROM_BUCKET, FROM_RADIX };
+
+// The step after an attempt of the star path with summary p that did not decide.
+From after_star(const Plan& p, u32 n, bool raw) {
+  const bool many = p.s_raw > kStarCap && (p.s == 0 || p.s > kStarCap);
+  if (many && p.s_raw <= sector_max_points()) return single_read(n) && raw ? FROM_SECTORS : FROM_FRONT;
+  return single_read(n) && raw ? FROM_RAW : FROM_BUCKET;
+}
 
 hull_status compute_from(hull_ctx* c, const int32_t* d_xy, u32 n, int32_t* d_out, int64_t cap, int64_t* h_count,
-                         cudaStream_t st, From from) {
+                         cudaStream_t st, From from, u32 bound = 0) {
+  Workspace& w = c->ws;
   hull_status r = HULL_OK;
   for (;;) {
     Next next = NEXT_NONE;
     c->prof_pending = c->prof;
     if (from == FROM_STAR) {
-      r = run_star(c, d_xy, n, d_out, cap, st);
+      r = run_star(c, d_xy, n, d_out, cap, c->h_plan, st);
+    } else if (from == FROM_FRONT || from == FROM_SECTORS) {
+      // bound: the raw survivors' number where the host knows it.
+      mark(c, 0, st);
+      cudaError_t e = cudaSuccess;
+      if (from == FROM_FRONT) { e = star_front(c, d_xy, n, st); bound = n; }
+      else mark(c, 1, st);
+      for (int p = 2; p <= 3 + kMaxPasses; ++p) mark(c, p, st);
+      if (e == cudaSuccess)
+        e = launch_sectors(n, bound, w.poly, w.sect, w.h_xy[0], reinterpret_cast<u32*>(w.h_idx[0]), w.h_xy[1],
+                           reinterpret_cast<u32*>(w.h_idx[1]), c->h_plan, d_out, (long long)cap, c->num_sms, st);
+      mark(c, 4 + kMaxPasses, st);
+      r = e == cudaSuccess ? HULL_OK : cuda_fail(e);
     } else {
       r = run_front(c, d_xy, n, st, from != FROM_RADIX, from == FROM_RAW);
-      if (r == HULL_OK)
-        r = run_final(c, c->ws.lo_xy, c->ws.lo_idx, c->ws.up_xy, c->ws.up_idx, (size_t)n, d_out, cap, st);
+      if (r == HULL_OK) r = run_final(c, w.lo_xy, w.lo_idx, w.up_xy, w.up_idx, (size_t)n, d_out, cap, st);
     }
     if (r != HULL_OK) { c->prof_pending = false; return r; }
-    r = finish(c, st, from == FROM_RADIX ? nullptr : &next);
-    if (next == NEXT_BUCKET) { from = single_read(n) ? FROM_RAW : FROM_BUCKET; continue; }
+    r = finish(c, st, from == FROM_RADIX ? nullptr : &next, from <= FROM_SECTORS);
+    if (from == FROM_STAR && single_read(n)) w.poly_clear = next == NEXT_NONE && r != HULL_ECUDA;
+    if (next == NEXT_BUCKET) {
+      from = from == FROM_STAR ? after_star(*c->h_plan, n, true) : FROM_BUCKET;
+      bound = c->h_plan->s_raw;
+      continue;
+    }
     if (next == NEXT_RADIX) { c->fallbacks += 1; from = FROM_RADIX; continue; }
     if (c->cfg.collect_stats) c->last.sort_fallback = from == FROM_RADIX ? 1 : 0;
     if (r == HULL_OK || r == HULL_ECAPACITY) *h_count = c->h_plan->h;
@@ -868,16 +909,17 @@ hull_status hull_compute_multi(hull_ctx* c, int32_t count, const int32_t* const*
     const cudaStream_t ls = lane1 ? c->aux : st;
     if (lane1) { std::swap(c->ws, c->ws2); std::swap(c->plan, c->plan2); }
     c->prof_pending = false;
-    if (star_eligible(c, (u32)n[k])) {
-      r = run_star(c, d_xy[k], (u32)n[k], d_out[k], cap[k], ls);
+    Plan* sum = reinterpret_cast<Plan*>(c->h_multi + (size_t)k * kSummaryBytes);
+    const bool star = star_eligible(c, (u32)n[k]);
+    if (star) {
+      r = run_star(c, d_xy[k], (u32)n[k], d_out[k], cap[k], sum, ls);
     } else {
       r = run_front(c, d_xy[k], (u32)n[k], ls, true);
       if (r == HULL_OK) r = run_final(c, c->ws.lo_xy, c->ws.lo_idx, c->ws.up_xy, c->ws.up_idx, (size_t)n[k], d_out[k],
                                       cap[k], ls);
     }
     cudaError_t e = cudaSuccess;
-    if (r == HULL_OK)
-      e = cudaMemcpyAsync(c->h_multi + (size_t)k * kSummaryBytes, c->plan, kSummaryBytes, cudaMemcpyDeviceToHost, ls);
+    if (r == HULL_OK && !star) e = cudaMemcpyAsync(sum, c->plan, kSummaryBytes, cudaMemcpyDeviceToHost, ls);
     if (lane1) { std::swap(c->ws, c->ws2); std::swap(c->plan, c->plan2); }
     if (r != HULL_OK) {
       if (two) cudaStreamSynchronize(c->aux);
@@ -909,8 +951,7 @@ hull_status hull_compute_multi(hull_ctx* c, int32_t count, const int32_t* const*
       if (lane1) { std::swap(c->ws, c->ws2); std::swap(c->plan, c->plan2); }
       if (next == NEXT_RADIX) c->fallbacks += 1;
       r = compute_from(c, d_xy[k], (u32)n[k], d_out[k], cap[k], &h_count[k], st,
-                       next == NEXT_RADIX ? FROM_RADIX
-                                          : single_read((u32)n[k]) && last ? FROM_RAW : FROM_BUCKET);
+                       next == NEXT_RADIX ? FROM_RADIX : after_star(p, (u32)n[k], last), p.s_raw);
       if (lane1) { std::swap(c->ws, c->ws2); std::swap(c->plan, c->plan2); }
     } else {
       if (c->cfg.collect_stats) c->last.sort_fallback = 0;

@@ -78,12 +78,8 @@ kb_small(BatchStar a) {
     const u32 n = (u32)(a.offsets[inst + 1] - off);
     const int2* P = reinterpret_cast<const int2*>(a.xy) + off;
     int* out = a.out_tmp + a.slot0[inst];
-    if (n < 3) {                       // at most one point: itself; two: the general path tells them apart
-      if (t == 0) {
-        bool bad = false;
-        if (n == 1) { bad = star::out_of_range(P[0].x, P[0].y); out[0] = 0; }
-        put_result(a, inst, n == 2 ? -1 : (int)n, bad);
-      }
+    if (n == 0) {
+      if (t == 0) put_result(a, inst, 0, false);
       __syncthreads();
       continue;
     }
@@ -129,6 +125,7 @@ kb_small(BatchStar a) {
     if (m0 <= (u32)BF_CAP && !err) {
       const u32 m = star::filter_list<BS_BLOCK, BF_CAP, BF_NB>(S.list, m0, F, S.key, S.cands);
       h = star::list_hull<BS_BLOCK, BF_CAP, BF_NB>(S.list, m, F, out, n);
+      if (h < 0) h = star::rest_hull<BS_BLOCK>(S.list, P, n, out, n);
     }
     if (t == 0) put_result(a, inst, err ? 0 : h, err);
     __syncthreads();

@@ -193,6 +193,29 @@ __device__ __forceinline__ bool aborted(const Plan* plan) {
   return (ld_volatile_u32(&plan->error) & (ERR_TIMEOUT | ERR_INTERNAL | ERR_FALLBACK)) != 0;
 }
 
+// Programmatic dependent launch: a kernel launched with launch_after may
+// start while the kernel before it in the stream still runs; pdl_wait returns
+// when that one has completed (at once in an ordinary launch), pdl_launch
+// lets the next one start.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... Par, typename... Arg>
+inline cudaError_t launch_after(void (*kernel)(Par...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                Arg... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<Par>(args)...);
+}
+
 // Exact orientation (b - a) x (c - a) in int64.  Coordinates are bounded by
 // 2^29, so each difference fits in int32 and each product in 2^60.
 __device__ __forceinline__ long long orient(int ax, int ay, int bx, int by, int cx, int cy) {

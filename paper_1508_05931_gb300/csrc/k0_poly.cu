@@ -45,6 +45,7 @@ k0_poly(const int2* __restrict__ P, u32 n, u32 ns, u32 slabs, PolyTab* __restric
     p = p1;
     i = i1;
   }
+  pdl_launch();
   __syncthreads();
   // The threads that update T->best order their updates before the block's
   // arrival; those of the last block order the arrivals before their reads.

@@ -330,13 +330,16 @@ k1_poly(const int2* __restrict__ P, u32 n, PolyTab* __restrict__ T, int2* __rest
   extern __shared__ __align__(16) unsigned char k1p_smem[];
   K1PSmem& S = *reinterpret_cast<K1PSmem*>(k1p_smem);
   const int wid = threadIdx.x >> 5;
-  const PolyHead H = T->head;
+  PolyHead H;
   star::RawSink<kStarBins, K1P_SLICE> sink{S.sxy[wid], S.sidx[wid], 0u, &T->frame, &T->raw_count, &T->error, T->key,
                                            rxy, ridx, n};
   star::stream_points<K1P_V>(P, n, 0u, blockIdx.x * K1P_WARPS + wid, gridDim.x * K1P_WARPS, H, S.tab, sink, [&] {
+    pdl_wait();              // the first loads are under way while K0 finishes
+    H = T->head;
     for (u32 q = threadIdx.x; q < H.nslab; q += K1P_BLOCK) S.tab[q] = T->tab[q];
     __syncthreads();
   });
+  pdl_launch();
   if (sink.fill) sink.flush();
 }
 
@@ -398,8 +401,8 @@ cudaError_t launch_k1_poly(const int* xy, u32 n, PolyTab* T, int2* rxy, u32* rid
   const u32 rounds = (n / 2 + K1P_BLOCK * K1P_V - 1) / (K1P_BLOCK * K1P_V);
   const u32 cap = (u32)num_sms * 2u;
   const u32 grid = rounds < 1u ? 1u : (rounds < cap ? rounds : cap);
-  k1_poly<<<grid, K1P_BLOCK, sizeof(K1PSmem), st>>>(reinterpret_cast<const int2*>(xy), n, T, rxy, ridx);
-  return cudaGetLastError();
+  return launch_after(k1_poly, dim3(grid), dim3(K1P_BLOCK), sizeof(K1PSmem), st, reinterpret_cast<const int2*>(xy), n,
+                      T, rxy, ridx);
 }
 
 cudaError_t launch_k1_raw(const int2* rxy, const u32* ridx, u32 n, u32 spin_limit, Plan* plan, ExtPartial* partials,

@@ -60,31 +60,19 @@ struct SmallSmem {
   u32 count, error;
 };
 
-// The call's summary (one thread).  h < 0: not decided.
-__device__ void write_summary(Plan* plan, u32 n, u32 raw, u32 s, int h, long long cap, u32 error) {
-  plan->n = n;
-  u32 e = error;
-  if (!(e & ERR_RANGE)) {
-    if (h < 0) e |= ERR_RETRY;
-    else if ((long long)h > cap) e |= ERR_CAPACITY;
-  }
-  plan->error = e;
-  plan->s = s; plan->s_quad = 0; plan->s_raw = raw; plan->r_lo = s; plan->r_up = 0;
-  plan->h = h > 0 ? (u32)h : 0u; plan->h_lo = 0; plan->h_up = 0;
-  plan->ncorner = 0; plan->learned_used = 0; plan->npasses = 0;
-  plan->sorted_in_b = 1; plan->ngroups = 1;
-}
-
 __global__ void __launch_bounds__(KS_BLOCK)
 k_star(const int2* __restrict__ P, u32 n, PolyTab* T, const int2* __restrict__ rxy, const u32* __restrict__ ridx,
        int2* lxy, u32* lidx, Plan* plan, int* out, long long cap) {
   extern __shared__ __align__(16) unsigned char ks_smem[];
   StarSmem& S = *reinterpret_cast<StarSmem*>(ks_smem);
   const int lane = threadIdx.x & 31, t = threadIdx.x;
+  pdl_wait();
   const u32 q = min(T->raw_count, n);
   const StarFrame F = T->frame;
-  if (q > KS_RAW_MAX && q > n / 4) {
-    if (blockIdx.x == 0 && t == 0) write_summary(plan, n, q, 0, -1, cap, T->error);
+  // No polygon: a degenerate input, not for the star path (s = 1 says so).
+  const bool flat = !T->head.ok;
+  if (flat || (q > KS_RAW_MAX && q > n / 4)) {
+    if (blockIdx.x == 0 && t == 0) star_summary(plan, n, q, flat ? 1u : 0u, -1, cap, T->error);
     return;
   }
   if (blockIdx.x * (u32)KS_BLOCK < q) {
@@ -142,7 +130,13 @@ k_star(const int2* __restrict__ P, u32 n, PolyTab* T, const int2* __restrict__ r
     __syncthreads();
     h = star::list_hull<KS_BLOCK, KS_CAP, kStarBins>(S.list, m, F, out, cap);
   }
-  if (t == 0) write_summary(plan, n, q, m, h, cap, err);
+  if (t == 0) star_summary(plan, n, q, m, h, cap, err);
+  // Decided: the table is left clear for the next call.
+  if (h >= 0 || (err & ERR_RANGE)) {
+    static_assert(kPolyClearBytes % sizeof(u64) == 0, "whole words");
+    u64* w = reinterpret_cast<u64*>(T);
+    for (u32 i = t; i < (u32)(kPolyClearBytes / sizeof(u64)); i += KS_BLOCK) w[i] = 0ull;
+  }
 }
 
 __global__ void __launch_bounds__(KS_BLOCK)
@@ -154,7 +148,7 @@ k_small(const int2* __restrict__ P, u32 n, Plan* plan, int* out, long long cap) 
   if (t < kPolyDirs) S.best[t] = 0ull;
   const StarFrame F = star::make_frame<KS_BLOCK>(P, n, S.frame);
   u32 m0 = n;
-  bool bad = false;
+  bool bad = false, flat = false;
   if (n <= KS_DIRECT) {
     for (u32 i = t; i < n; i += KS_BLOCK) {
       const int2 p = P[i];
@@ -184,6 +178,7 @@ k_small(const int2* __restrict__ P, u32 n, Plan* plan, int* out, long long cap) 
     star::ListSink<decltype(S.list)> sink{&S.list, &S.count, (u32)KS_CAP, false};
     star::stream_points<4>(P, n, 0u, (u32)wid, (u32)(KS_BLOCK / 32), H, S.tab, sink, [] {});
     bad = sink.bad;
+    flat = !H.ok;
     __syncthreads();
     m0 = S.count;
   }
@@ -196,7 +191,11 @@ k_small(const int2* __restrict__ P, u32 n, Plan* plan, int* out, long long cap) 
     m = star::filter_list<KS_BLOCK, KS_CAP, kStarBins>(S.list, m0, F, S.key, S.cands);
     h = star::list_hull<KS_BLOCK, KS_CAP, kStarBins>(S.list, m, F, out, cap);
   }
-  if (t == 0) write_summary(plan, n, m0, m, h, cap, err);
+  if (h < 0 && !err && (flat || m0 <= (u32)KS_CAP)) {
+    h = star::rest_hull<KS_BLOCK>(S.list, P, n, out, cap);
+    m = m0 = 0u;                      // not undecided for being too many
+  }
+  if (t == 0) star_summary(plan, n, m0, m, h, cap, err);
 }
 
 }  // namespace
@@ -212,9 +211,8 @@ cudaError_t launch_star(const int* xy, u32 n, PolyTab* T, const int2* rxy, const
                         Plan* plan, int* out, long long cap, int num_sms, cudaStream_t st) {
   const u32 want = n / (32u * KS_BLOCK) + 1u;      // a block per 32,768 input points
   const u32 grid = want < (u32)num_sms ? want : (u32)num_sms;
-  k_star<<<grid, KS_BLOCK, sizeof(StarSmem), st>>>(reinterpret_cast<const int2*>(xy), n, T, rxy, ridx, lxy, lidx, plan,
-                                                   out, cap);
-  return cudaGetLastError();
+  return launch_after(k_star, dim3(grid), dim3(KS_BLOCK), sizeof(StarSmem), st, reinterpret_cast<const int2*>(xy), n, T,
+                      rxy, ridx, lxy, lidx, plan, out, cap);
 }
 
 cudaError_t launch_small(const int* xy, u32 n, Plan* plan, int* out, long long cap, cudaStream_t st) {

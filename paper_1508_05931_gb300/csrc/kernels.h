@@ -75,6 +75,13 @@ cudaError_t star_configure();
 cudaError_t launch_star(const int* xy, u32 n, PolyTab* T, const int2* rxy, const u32* ridx, int2* lxy, u32* lidx,
                         Plan* plan, int* out, long long cap, int num_sms, cudaStream_t st);
 cudaError_t launch_small(const int* xy, u32 n, Plan* plan, int* out, long long cap, cudaStream_t st);
+// The hull of K1's raw survivors when they are many (k_sector.cu): at most
+// `bound` of them at (axy, aidx); both buffers hold n points and are
+// overwritten; tab: sector_bytes() of scratch.
+size_t sector_bytes();
+u32 sector_max_points();
+cudaError_t launch_sectors(u32 n, u32 bound, PolyTab* T, void* tab, int2* axy, u32* aidx, int2* bxy, u32* bidx,
+                           Plan* plan, int* out, long long cap, int num_sms, cudaStream_t st);
 cudaError_t launch_place(const u64* ak, const u32* ai, u32 n, Plan* plan, const u32* bstart, u32* ccur, u64* ok,
                          u32* oi, int num_sms, cudaStream_t st);
 size_t bucket_smem();

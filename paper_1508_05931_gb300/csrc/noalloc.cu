@@ -66,6 +66,8 @@ struct Carve {
   u32* cnt[2];
   int4* jobs;
   unsigned char* mask;
+  PolyTab* poly;
+  void* sect;
   size_t total;
 };
 
@@ -102,6 +104,8 @@ Carve carve(unsigned char* base, int num_sms) {
   for (int b = 0; b < 2; ++b) c.cnt[b] = reinterpret_cast<u32*>(take(nchunks * 4));
   c.jobs = reinterpret_cast<int4*>(take(nchunks * 16));
   c.mask = take(cap / 8 + 4096);
+  c.poly = reinterpret_cast<PolyTab*>(take(sizeof(PolyTab)));
+  c.sect = take(sector_bytes());
   c.total = off;
   return c;
 }
@@ -125,7 +129,7 @@ hull_status noalloc_setup(int dev, NoAllocDevice** out) {
     cudaDeviceProp prop;
     if (cudaGetDeviceProperties(&prop, dev) != cudaSuccess) { cudaGetLastError(); return HULL_ECUDA; }
     if (carve(nullptr, prop.multiProcessorCount).total > kNoAllocBytes) return HULL_EINTERNAL;
-    if (star_configure() != cudaSuccess || k2_configure() != cudaSuccess || k3_configure() != cudaSuccess ||
+    if (star_configure() != cudaSuccess || k1_poly_configure() != cudaSuccess || k2_configure() != cudaSuccess || k3_configure() != cudaSuccess ||
         k5_configure(&d.occ_k5) != cudaSuccess ||
         k2_occupancy(&d.occ_k2c, &d.occ_k2) != cudaSuccess || k3_occupancy(&d.occ_k3) != cudaSuccess ||
         k4_occupancy(&d.occ_k4) != cudaSuccess || d.occ_k5 < 1) {
@@ -166,12 +170,24 @@ extern "C" hull_status hull_compute_noalloc(const int32_t* d_xy, int64_t n, int3
   // pinned buffer is allocated) and the call waits for the stream.
   alignas(16) unsigned char summary[offsetof(Plan, ctr)];
   const Plan* p = reinterpret_cast<const Plan*>(summary);
-  // The star path first (one launch, no scratch but the Plan); what it does
-  // not decide takes the radix pipeline.
+  // The star path first (one launch, no scratch but the Plan), its sectors
+  // when many points lie next to the hull; what they do not decide takes the
+  // radix pipeline.
   static_assert(HULL_NOALLOC_MAX_POINTS <= kSmallMax, "one block takes every call");
   cudaError_t e = launch_small(d_xy, un, c.plan, d_out, (long long)cap, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(summary, c.plan, sizeof(summary), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e == cudaSuccess && (p->error & ERR_RETRY) && p->s > kStarCap) {
+    u32* ridx = reinterpret_cast<u32*>(c.h_idx[0]);
+    e = cudaMemsetAsync(c.poly, 0, kPolyClearBytes, st);
+    if (e == cudaSuccess) e = launch_poly(d_xy, un, c.poly, d->num_sms, st);
+    if (e == cudaSuccess) e = launch_k1_poly(d_xy, un, c.poly, c.h_xy[0], ridx, d->num_sms, st);
+    if (e == cudaSuccess)
+      e = launch_sectors(un, un, c.poly, c.sect, c.h_xy[0], ridx, c.h_xy[1], reinterpret_cast<u32*>(c.h_idx[1]), c.plan,
+                         d_out, (long long)cap, d->num_sms, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(summary, c.plan, sizeof(summary), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  }
   if (e == cudaSuccess && (p->error & ERR_RETRY)) {
     e = cudaMemsetAsync(c.plan, 0, c.zero_bytes, st);
     if (e == cudaSuccess)

@@ -1,5 +1,5 @@
 // The star path: the hull of the points that survive a sample polygon,
-// found in angular order around an interior input point c (Section 2.1
+// found in angular order around an interior point c (Section 2.1
 // steps 3-8 with the pivot moved inside: distance and angle about c, the
 // sort by angle, and the scan that pops non-left turns, run as rounds in
 // which every point looks at its neighbours).
@@ -9,9 +9,10 @@
 // bins and the choice of candidates are float and only steer; every
 // decision to drop a point is exact in 64-bit integers:
 //   a point q inside the closed triangle (c, a, b) of three input points
-//   with cross(a - c, b - c) > 0, not on the side a b, is no hull vertex
-//   (q = c aside); on the open segment a b neither; equal to a or b it is
-//   the duplicate with the larger index.
+//   with cross(a - c, b - c) > 0, not on the side a b, is no hull vertex; on
+//   the open segment a b neither; equal to a or b it is the duplicate with
+//   the larger index.  (This takes c strictly inside the hull, which the
+//   verification below proves before any result is used.)
 // The drops of a round may use points that the same round drops: those are
 // input points too.  The rounds end with a polygon that is verified: every
 // consecutive cross product about c positive and every turn strictly left
@@ -88,15 +89,14 @@ __device__ __forceinline__ u32 block_scan(u32 v, u32* ws, u32& total) {
 }
 
 // ---------------------------------------------------------------- frame
-// From BLOCK strided points of P[0, n): their mean and covariance, the
-// whitening map (the inverse Cholesky factor, determinant > 0) and c, the
-// sampled point nearest the mean.  Every block that calls it with the same
-// P and n gets the same frame.
+// From BLOCK strided points of P[0, n): c, their mean rounded to integers,
+// and the whitening map of their covariance (the inverse Cholesky factor,
+// determinant > 0).  Every block that calls it with the same P and n gets
+// the same frame.  Nothing is assumed of c: a polygon of input points that
+// verifies about it proves that it lies inside.
 template <int BLOCK>
 struct FrameSmem {
   float sum[BLOCK / 32][5];
-  u64 best;
-  int2 c;
 };
 
 template <int BLOCK>
@@ -113,7 +113,6 @@ __device__ __forceinline__ StarFrame make_frame(const int2* __restrict__ P, u32 
     for (int d = 16; d > 0; d >>= 1) s[k] += __shfl_xor_sync(0xFFFFFFFFu, s[k], d);
     if (lane == 0) S.sum[wid][k] = s[k];
   }
-  if (threadIdx.x == 0) S.best = ~0ull;
   __syncthreads();
   #pragma unroll
   for (int k = 0; k < 5; ++k) {
@@ -129,16 +128,10 @@ __device__ __forceinline__ StarFrame make_frame(const int2* __restrict__ P, u32 
   F.m00 = 1.0f / l11;
   F.m11 = 1.0f / l22;
   F.m10 = -(l21 / l11) / l22;
-  const float u = (fx - mx) * F.m00, v = fmaf(fy - my, F.m11, (fx - mx) * F.m10);
-  const u32 r = __float_as_uint(fmaf(u, u, v * v)) & 0x7FFFFFFFu;
-  const u32 rm = __reduce_min_sync(0xFFFFFFFFu, r);
-  const u32 who = __ballot_sync(0xFFFFFFFFu, r == rm);
-  if (lane == __ffs(who) - 1) atomicMin(&S.best, ((u64)rm << 32) | (u64)threadIdx.x);
-  __syncthreads();
-  if ((u32)S.best == threadIdx.x) S.c = p;
-  __syncthreads();
-  F.cx = S.c.x;
-  F.cy = S.c.y;
+  // Inside the coordinate range whatever the points hold.
+  const float L = (float)kCoordLimit;
+  F.cx = (int)rintf(fminf(fmaxf((float)o.x + mx, -L), L));
+  F.cy = (int)rintf(fminf(fmaxf((float)o.y + my, -L), L));
   return F;
 }
 
@@ -540,6 +533,94 @@ struct ListSmem {
   u32 flag;
 };
 
+// The rank of entry i of the bin's entries at[s, e) (positions in p) in the
+// order: counter-clockwise about c, along a ray the farther first, equal
+// points by index.  dead: not the first of its ray (a nearer point of a ray
+// is no vertex), or c itself.
+__device__ __forceinline__ u32 bin_rank(const int2* p, const u32* id, const unsigned short* at, u32 s, u32 e, u32 i,
+                                        const StarFrame& F, bool& dead) {
+  const u32 k = at[i];
+  const int2 w = p[k];
+  const int2 q = make_int2(w.x - F.cx, w.y - F.cy);
+  const u32 qr = (u32)abs(q.x) + (u32)abs(q.y), qi = id[k];
+  u32 r = 0;
+  dead = q.x == 0 && q.y == 0;
+  for (u32 j = s; j < e; ++j) {
+    if (j == i) continue;
+    const u32 kj = at[j];
+    const int2 v = p[kj];
+    const int2 d = make_int2(v.x - F.cx, v.y - F.cy);
+    const long long c = cross2(d.x, d.y, q.x, q.y);
+    if (c > 0) { ++r; continue; }
+    if (c < 0) continue;
+    const u32 dr = (u32)abs(d.x) + (u32)abs(d.y);
+    if (dr > qr || (dr == qr && id[kj] < qi)) { ++r; dead = true; }
+  }
+  return r;
+}
+
+// The rounds over the entries cur[0, m) (positions in S.p in angular order,
+// bit 15: marked for removal when `marked`): thread t owns a run of
+// consecutive entries and drops those that the wedge of their neighbours
+// covers.  OPEN: the entries are a run of a longer cyclic list and its two
+// ends stay; otherwise they are the whole cyclic list and `done` reports
+// that the last round dropped nothing and every entry is a vertex of a
+// convex polygon about c.  `cur` and `nxt` may be exchanged; returns the
+// number of entries left in cur.
+template <int BLOCK, bool OPEN, class L>
+__device__ u32 drop_rounds(L& S, u32 m, const StarFrame& F, unsigned short* nxt, unsigned short*& cur, bool marked,
+                           bool& done) {
+  const int t = threadIdx.x;
+  auto rel = [&](u32 k) { const int2 p = S.p[k]; return make_int2(p.x - F.cx, p.y - F.cy); };
+  u32 par = 1;
+  done = false;
+  for (int round = marked ? 0 : 1; round <= kRounds; ++round) {
+    const u32 per = (m + BLOCK - 1) / BLOCK;
+    const u32 i0 = min(m, t * per), i1 = min(m, i0 + per);
+    u32 kept = 0, mask = 0;                 // at most 32 entries a thread (the lists' assertions)
+    bool bad = false;
+    for (u32 i = i0; i < i1; ++i) {
+      const u32 k = cur[i];
+      bool keep;
+      if (round == 0) {
+        keep = !(k & 0x8000u);
+      } else if (OPEN && (i == 0 || i == m - 1)) {
+        keep = true;
+      } else {
+        const int2 q = rel(k);
+        const int2 a = rel(cur[i > 0 ? i - 1 : m - 1]), b = rel(cur[i + 1 < m ? i + 1 : 0]);
+        const long long ab = cross2(a.x, a.y, b.x, b.y);
+        const long long aq = cross2(a.x, a.y, q.x, q.y), qb = cross2(q.x, q.y, b.x, b.y);
+        const long long o = ab - aq - qb;
+        keep = !(ab > 0 && aq >= 0 && qb >= 0 && (o > 0 || (o == 0 && aq > 0 && qb > 0)));
+        // A vertex of the verified polygon: c strictly left of both its
+        // edges, a strict left turn (o < 0).
+        bad = bad || !(aq > 0 && qb > 0 && o < 0);
+        if (keep && round <= 3 && m > 8 && (!OPEN || (i >= 2 && i + 2 < m))) {
+          // A wider wedge drops runs of points in fewer rounds.
+          const int2 a2 = rel(cur[i >= 2 ? i - 2 : i + m - 2]), b2 = rel(cur[i + 2 < m ? i + 2 : i + 2 - m]);
+          keep = !dropped_by(a2, b2, q);
+        }
+      }
+      if (keep) { mask |= 1u << (i - i0); ++kept; }
+    }
+    u32 tot;
+    u32 pos = block_scan<BLOCK>(kept, S.ws[par], tot);
+    par ^= 1u;
+    if (round > 0 && tot == m) {         // uniform: nothing dropped
+      done = OPEN || !__syncthreads_or(bad);
+      break;
+    }
+    for (u32 i = i0; i < i1; ++i)
+      if ((mask >> (i - i0)) & 1u) nxt[pos++] = cur[i];
+    __syncthreads();
+    unsigned short* w = cur; cur = nxt; nxt = w;
+    m = tot;
+    if (m < 3) break;
+  }
+  return m;
+}
+
 // The hull of the m points named by S.ta (the whole block; S.p, S.id, S.ta
 // written and visible).  Returns its number of vertices, written as input
 // indices counter-clockwise from the lexicographic minimum into out[0, cap)
@@ -547,7 +628,7 @@ struct ListSmem {
 template <int BLOCK, int CAP, int NB>
 __device__ int list_hull(ListSmem<BLOCK, CAP, NB>& S, u32 m, const StarFrame& F, int* out, long long cap) {
   static_assert(NB % BLOCK == 0 || BLOCK % NB == 0, "whole bins per thread");
-  static_assert(CAP <= 32768, "a position and a flag in 16 bits");
+  static_assert(CAP <= 32768 && CAP / BLOCK <= 32, "a position and a flag in 16 bits, one mask bit per owned entry");
   constexpr int PER = NB / BLOCK > 0 ? NB / BLOCK : 1;
   const int t = threadIdx.x;
   if (m < 3 || m > (u32)CAP) return -1;
@@ -587,80 +668,18 @@ __device__ int list_hull(ListSmem<BLOCK, CAP, NB>& S, u32 m, const StarFrame& F,
     S.tb[atomicAdd(&S.cur[S.bn[k]], 1u)] = k;       // cur[b] ends at the bin's end
   }
   __syncthreads();
-  // Order inside the bins by counting: counter-clockwise about c, along a
-  // ray the farther first, equal points by index.  All but the first of a
-  // ray are marked (bit 15): nearer points of a ray are no vertices.
+  // Order inside the bins by counting, the removals marked (bit 15).
   for (u32 i = t; i < m; i += BLOCK) {
     const u32 k = S.tb[i], b = S.bn[k];
     const u32 e = S.cur[b], s = e - S.cnt[b];
-    const int2 p = S.p[k];
-    const int2 q = make_int2(p.x - F.cx, p.y - F.cy);
-    const u32 qr = (u32)abs(q.x) + (u32)abs(q.y), qi = S.id[k];
-    u32 r = 0;
-    bool dead = q.x == 0 && q.y == 0;
-    for (u32 j = s; j < e; ++j) {
-      if (j == i) continue;
-      const u32 kj = S.tb[j];
-      const int2 w = S.p[kj];
-      const int2 d = make_int2(w.x - F.cx, w.y - F.cy);
-      const long long c = cross2(d.x, d.y, q.x, q.y);
-      if (c > 0) { ++r; continue; }
-      if (c < 0) continue;
-      const u32 dr = (u32)abs(d.x) + (u32)abs(d.y);
-      if (dr > qr || (dr == qr && S.id[kj] < qi)) { ++r; dead = true; }
-    }
+    bool dead;
+    const u32 r = bin_rank(S.p, S.id, S.tb, s, e, i, F, dead);
     S.ta[min(s + r, m - 1u)] = (unsigned short)(k | (dead ? 0x8000u : 0u));
   }
   __syncthreads();
-  // Rounds: thread t owns a run of consecutive entries.
   unsigned short* cur = S.ta;
-  unsigned short* nxt = S.tb;
-  u32 par = 1;
   bool done = false;
-  auto rel = [&](u32 k) { const int2 p = S.p[k]; return make_int2(p.x - F.cx, p.y - F.cy); };
-  for (int round = 0; round <= kRounds; ++round) {
-    const u32 per = (m + BLOCK - 1) / BLOCK;
-    const u32 i0 = min(m, t * per), i1 = min(m, i0 + per);
-    u32 kept = 0, mask = 0;       // per <= CAP / BLOCK <= 32
-    static_assert(CAP / BLOCK <= 32, "one mask bit per owned entry");
-    bool bad = false;
-    for (u32 i = i0; i < i1; ++i) {
-      const u32 k = cur[i];
-      bool keep;
-      if (round == 0) {
-        keep = !(k & 0x8000u);
-      } else {
-        const int2 q = rel(k);
-        const int2 a = rel(cur[i > 0 ? i - 1 : m - 1]), b = rel(cur[i + 1 < m ? i + 1 : 0]);
-        const long long ab = cross2(a.x, a.y, b.x, b.y);
-        const long long aq = cross2(a.x, a.y, q.x, q.y), qb = cross2(q.x, q.y, b.x, b.y);
-        const long long o = ab - aq - qb;
-        keep = !(ab > 0 && aq >= 0 && qb >= 0 && (o > 0 || (o == 0 && aq > 0 && qb > 0)));
-        // A vertex of the verified polygon: c strictly left of both its
-        // edges, a strict left turn (o < 0).
-        bad = bad || !(aq > 0 && qb > 0 && o < 0);
-        if (keep && round <= 3 && m > 8) {
-          // A wider wedge drops runs of points in fewer rounds.
-          const int2 a2 = rel(cur[i >= 2 ? i - 2 : i + m - 2]), b2 = rel(cur[i + 2 < m ? i + 2 : i + 2 - m]);
-          keep = !dropped_by(a2, b2, q);
-        }
-      }
-      if (keep) { mask |= 1u << (i - i0); ++kept; }
-    }
-    u32 tot;
-    u32 pos = block_scan<BLOCK>(kept, S.ws[par], tot);
-    par ^= 1u;
-    if (round > 0 && tot == m) {         // uniform: nothing dropped
-      done = !__syncthreads_or(bad);
-      break;
-    }
-    for (u32 i = i0; i < i1; ++i)
-      if ((mask >> (i - i0)) & 1u) nxt[pos++] = cur[i];
-    __syncthreads();
-    unsigned short* w = cur; cur = nxt; nxt = w;
-    m = tot;
-    if (m < 3) return -1;
-  }
+  m = drop_rounds<BLOCK, false>(S, m, F, S.tb, cur, true, done);
   if (!done) return -1;
   // The lexicographic minimum starts the output.
   auto lex = [&](u32 i) {
@@ -737,5 +756,99 @@ __device__ u32 filter_list(ListSmem<BLOCK, CAP, NB>& S, u32 m0, const StarFrame&
   return m;
 }
 
+// A degenerate or tiny input that the rounds did not decide (n >= 1 points in
+// range; the whole block): all points equal or on one line, found from the
+// lexicographic extremes; up to 64 points by Andrew's chain in one thread.
+// The number of vertices (in out when they fit) or -1.
+template <int BLOCK, class L>
+__device__ int rest_hull(L& S, const int2* __restrict__ P, u32 n, int* out, long long cap) {
+  __shared__ u64 s_lo, s_hi;
+  __shared__ u32 s_il, s_ih;
+  const int t = threadIdx.x;
+  auto lex = [](int2 p) { return ((u64)((u32)p.x ^ 0x80000000u) << 32) | (u64)((u32)p.y ^ 0x80000000u); };
+  __syncthreads();
+  if (t == 0) { s_lo = ~0ull; s_hi = 0ull; s_il = s_ih = 0xFFFFFFFFu; }
+  __syncthreads();
+  u64 lo = ~0ull, hi = 0ull;
+  for (u32 i = t; i < n; i += BLOCK) {
+    const u64 v = lex(P[i]);
+    lo = v < lo ? v : lo; hi = v > hi ? v : hi;
+  }
+  #pragma unroll
+  for (int d = 16; d > 0; d >>= 1) {
+    const u64 a = __shfl_xor_sync(0xFFFFFFFFu, lo, d), b = __shfl_xor_sync(0xFFFFFFFFu, hi, d);
+    lo = a < lo ? a : lo; hi = b > hi ? b : hi;
+  }
+  if ((t & 31) == 0) { atomicMin(&s_lo, lo); atomicMax(&s_hi, hi); }
+  __syncthreads();
+  lo = s_lo; hi = s_hi;
+  const int2 A = make_int2((int)((u32)(lo >> 32) ^ 0x80000000u), (int)((u32)lo ^ 0x80000000u));
+  const int2 B = make_int2((int)((u32)(hi >> 32) ^ 0x80000000u), (int)((u32)hi ^ 0x80000000u));
+  bool off = false;
+  for (u32 i = t; i < n; i += BLOCK) {
+    const int2 p = P[i];
+    const u64 v = lex(p);
+    if (v == lo) atomicMin(&s_il, i);
+    if (v == hi) atomicMin(&s_ih, i);
+    off = off || orient(A.x, A.y, B.x, B.y, p.x, p.y) != 0;
+  }
+  if (!__syncthreads_or(off)) {
+    const int h = lo == hi ? 1 : 2;
+    if (t == 0 && h <= cap) { out[0] = (int)s_il; if (h == 2) out[1] = (int)s_ih; }
+    return h;
+  }
+  if (n > 64u) return -1;
+  // Sorted by (x, y), the smallest index of equal points only.
+  __shared__ u32 s_keep[2];
+  const u64 v = t < (int)n ? lex(P[t]) : 0ull;
+  bool keep = t < (int)n;
+  for (u32 j = 0; j < n && j < (u32)t && keep; ++j) keep = lex(P[j]) != v;
+  const u32 km = __ballot_sync(0xFFFFFFFFu, keep);
+  if (t < 64 && (t & 31) == 0) s_keep[t >> 5] = km;
+  __syncthreads();
+  u32 r = 0;
+  if (keep)
+    for (u32 j = 0; j < n; ++j) r += ((s_keep[j >> 5] >> (j & 31u)) & 1u) && lex(P[j]) < v ? 1u : 0u;
+  if (keep) S.ta[r] = (unsigned short)t;
+  const int m = __syncthreads_count(keep);
+  if (t == 0) {
+    int k = 0;
+    auto chain = [&](int i, int base) {
+      const int2 p = P[S.ta[i]];
+      while (k >= base + 2) {
+        const int2 a = P[S.tb[k - 2]], b = P[S.tb[k - 1]];
+        if (orient(a.x, a.y, b.x, b.y, p.x, p.y) > 0) break;
+        --k;
+      }
+      S.tb[k++] = S.ta[i];
+    };
+    for (int i = 0; i < m; ++i) chain(i, 0);
+    const int base = k - 1;
+    for (int i = m - 2; i >= 0; --i) chain(i, base);
+    --k;                                 // the first point again
+    S.flag = (u32)k;
+    if (k <= cap)
+      for (int i = 0; i < k; ++i) out[i] = (int)S.tb[i];
+  }
+  __syncthreads();
+  return (int)S.flag;
+}
+
 }  // namespace star
+
+// The call's summary (one thread).  h < 0: not decided.
+__device__ __forceinline__ void star_summary(Plan* plan, u32 n, u32 raw, u32 s, int h, long long cap, u32 error) {
+  plan->n = n;
+  u32 e = error;
+  if (!(e & ERR_RANGE)) {
+    if (h < 0) e |= ERR_RETRY;
+    else if ((long long)h > cap) e |= ERR_CAPACITY;
+  }
+  plan->error = e;
+  plan->s = s; plan->s_quad = 0; plan->s_raw = raw; plan->r_lo = s; plan->r_up = 0;
+  plan->h = h > 0 ? (u32)h : 0u; plan->h_lo = 0; plan->h_up = 0;
+  plan->ncorner = 0; plan->learned_used = 0; plan->npasses = 0;
+  plan->sorted_in_b = 1; plan->ngroups = 1;
+}
+
 }  // namespace gbh
