@@ -583,7 +583,7 @@ hull_status compute_from(hull_ctx* c, const int32_t* d_xy, u32 n, int32_t* d_out
     }
     if (r != HULL_OK) { c->prof_pending = false; return r; }
     r = finish(c, st, from == FROM_RADIX ? nullptr : &next, from <= FROM_SECTORS);
-    if (from == FROM_STAR && single_read(n)) w.poly_clear = next == NEXT_NONE && r != HULL_ECUDA;
+    if (from == FROM_STAR && single_read(n)) w.poly_clear = next == NEXT_NONE && (r == HULL_OK || r == HULL_ECAPACITY);
     if (next == NEXT_BUCKET) {
       from = from == FROM_STAR ? after_star(*c->h_plan, n, true) : FROM_BUCKET;
       bound = c->h_plan->s_raw;
@@ -2019,6 +2019,7 @@ hull_status hull_compute_batched(hull_ctx* c, const int32_t* d_xy, const int64_t
   }
   const u32 err = w.h_ctl[2];
   if (err & ERR_RANGE) return HULL_ERANGE;
+  if (err & ERR_TIMEOUT) return HULL_ETIMEOUT;
   if (err & ERR_INTERNAL) return HULL_EINTERNAL;
   if (err & ERR_CAPACITY) return HULL_ECAPACITY;
   return HULL_OK;

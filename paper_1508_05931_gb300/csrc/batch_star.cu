@@ -83,29 +83,39 @@ kb_small(BatchStar a) {
       __syncthreads();
       continue;
     }
-    const StarFrame F = star::make_frame<BS_BLOCK>(P, n, S.frame);
+    StarFrame F;
     u32 m0 = n;
     bool bad = false;
     if (n <= BS_DIRECT) {
-      for (u32 i = t; i < n; i += BS_BLOCK) {
-        const int2 p = P[i];
-        S.list.p[i] = p;
-        S.list.id[i] = i;
-        bad = bad || star::out_of_range(p.x, p.y);
-      }
-    } else {
-      constexpr u32 NS = BS_SAMPLES * BS_BLOCK;
-      static_assert(NS <= BS_DIRECT, "a stride of at least one point");
-      const u32 stride = n / NS;
+      static_assert(BS_DIRECT <= BS_SAMPLES * BS_BLOCK, "the points in registers");
       int2 p[BS_SAMPLES];
       #pragma unroll
-      for (int r = 0; r < BS_SAMPLES; ++r) p[r] = P[(r * BS_BLOCK + t) * stride];
+      for (int r = 0; r < BS_SAMPLES; ++r) p[r] = r * BS_BLOCK + t < n ? P[r * BS_BLOCK + t] : make_int2(0, 0);
+      F = star::make_frame<BS_BLOCK>(P, n, S.frame);
+      #pragma unroll
+      for (int r = 0; r < BS_SAMPLES; ++r) {
+        const u32 i = r * BS_BLOCK + t;
+        if (i < n) {
+          S.list.p[i] = p[r];
+          S.list.id[i] = i;
+          bad = bad || star::out_of_range(p[r].x, p[r].y);
+        }
+      }
+    } else {
+      // The sample, in runs of four points, also gives the frame.
+      constexpr u32 NS = BS_SAMPLES * BS_BLOCK;
+      static_assert(NS <= BS_DIRECT && BS_SAMPLES % 4 == 0, "whole runs, a stride of at least their length");
+      const u32 stride = n / (NS / 4u);
+      int2 p[BS_SAMPLES];
+      #pragma unroll
+      for (int r = 0; r < BS_SAMPLES; ++r) p[r] = P[star::sample_at(r * BS_BLOCK + t, stride)];
+      F = star::frame_of<BS_BLOCK>(p, P[0], S.frame);
       #pragma unroll
       for (int r = 0; r < BS_SAMPLES; ++r) star::offer_sample(F, p[r], r * BS_BLOCK + t, S.best);
       __syncthreads();
       if (t < kPolyDirs) {
         const u32 i = ~(u32)S.best[t];
-        S.poly.p[t] = i < NS ? P[i * stride] : make_int2(0, 0);
+        S.poly.p[t] = i < NS ? P[star::sample_at(i, stride)] : make_int2(0, 0);
         const u32 h = __ballot_sync(0xFFFFFFFFu, i < NS);
         if (lane == 0) S.poly.has[wid] = h;
       }
@@ -134,7 +144,7 @@ kb_small(BatchStar a) {
 
 // ---- large instances
 constexpr int BP_BLOCK = 512;
-constexpr int BP_ITEMS = 4;           // samples per thread loaded together
+constexpr int BP_ITEMS = 2;           // samples per thread loaded together
 
 struct PolyBlockSmem {
   star::FrameSmem<BP_BLOCK> frame;
@@ -142,8 +152,9 @@ struct PolyBlockSmem {
   u64 best[kPolyDirs];
 };
 
-// Sample: n / 128 points (1,024 to 8,192): 6 % of the input's DRAM granules,
-// and 1-2 % of a disk's points left outside the polygon.
+// Sample: n / 32 points (1,024 to 16,384) in runs of four: 6 % of the
+// input's DRAM granules, and 1-2 % of a disk's points left outside the
+// polygon.
 __global__ void __launch_bounds__(BP_BLOCK)
 kb_poly(BatchStar a) {
   __shared__ PolyBlockSmem S;
@@ -156,23 +167,30 @@ kb_poly(BatchStar a) {
   for (int b = t; b < BF_NB; b += BP_BLOCK) R.key[b] = 0ull;
   if (t == 0) R.raw_count = 0u;
   if (t < kPolyDirs) S.best[t] = 0ull;
-  const StarFrame F = star::make_frame<BP_BLOCK>(P, n, S.frame);
-  const u32 ns = min(max(n / 128u, 1024u), min(n, 8192u)), stride = n / ns;
+  const u32 ns = min(max(n / 32u, 1024u), 16384u) & ~3u, stride = n / (ns / 4u);
+  // The first round's points also give the frame (points past the sample
+  // repeat its last one).
+  int2 p[BP_ITEMS];
+  #pragma unroll
+  for (int r = 0; r < BP_ITEMS; ++r) p[r] = P[star::sample_at(min(t + r * BP_BLOCK, ns - 1u), stride)];
+  const StarFrame F = star::frame_of<BP_BLOCK>(p, P[0], S.frame);
   for (u32 i0 = t; i0 < ns; i0 += BP_ITEMS * BP_BLOCK) {
-    int2 p[BP_ITEMS];
+    int2 q[BP_ITEMS];
     #pragma unroll
     for (int r = 0; r < BP_ITEMS; ++r) {
-      const u32 i = i0 + r * BP_BLOCK;
-      p[r] = i < ns ? P[(size_t)i * stride] : make_int2(0, 0);
+      const u32 i = i0 + (BP_ITEMS + r) * BP_BLOCK;
+      q[r] = i < ns ? P[star::sample_at(i, stride)] : make_int2(0, 0);
     }
     #pragma unroll
-    for (int r = 0; r < BP_ITEMS; ++r)
+    for (int r = 0; r < BP_ITEMS; ++r) {
       if (i0 + r * BP_BLOCK < ns) star::offer_sample(F, p[r], i0 + r * BP_BLOCK, S.best);
+      p[r] = q[r];
+    }
   }
   __syncthreads();
   if (t < kPolyDirs) {
     const u32 i = ~(u32)S.best[t];
-    S.poly.p[t] = i < ns ? P[(size_t)i * stride] : make_int2(0, 0);
+    S.poly.p[t] = i < ns ? P[star::sample_at(i, stride)] : make_int2(0, 0);
     const u32 h = __ballot_sync(0xFFFFFFFFu, i < ns);
     if (lane == 0) S.poly.has[wid] = h;
   }
@@ -181,32 +199,43 @@ kb_poly(BatchStar a) {
   if (t == 0) { R.frame = F; R.head = H; }
 }
 
-constexpr int BT_BLOCK = 512;
+constexpr int BT_BLOCK = 128;
 constexpr int BT_WARPS = BT_BLOCK / 32;
-constexpr int BT_SLICE = 192;         // staged points per warp
-constexpr int BT_V = 4;               // pairs per lane and round
+constexpr int BT_SLICE = 256;         // staged points per warp: at least a chunk
+constexpr int BT_CH = 256;            // points per chunk
+constexpr int BT_STAGES = 4;          // chunks in flight per warp
 
 struct StreamSmem {
+  int4 ring[BT_WARPS][BT_STAGES][BT_CH / 2];
+  u64 bar[BT_WARPS][BT_STAGES];
   int2 sxy[BT_WARPS][BT_SLICE];
   u32 sidx[BT_WARPS][BT_SLICE];
   u32 tab[BF_SLABS];
 };
 
-// Block b streams the tiles [b T / G, (b + 1) T / G) in runs of one instance
-// each, raw survivors to the instance's second key / index scratch.
-__global__ void __launch_bounds__(BT_BLOCK, 2)
+// Four warps a block, each with its ring, four blocks an SM: the reads of an
+// instance's record at the start of a run overlap the other blocks' streams
+// (one block of sixteen warps took 75 us instead of 44 for 1,024 instances of
+// 19,531 points, where a run has five chunks a warp).  With a ballot per
+// point slot the pass over 232M points of 2,095 instances took 485 us, with
+// the survivors pushed lane by lane 359 (5.2 TB/s).
+// Block b of G streams its share of the T tiles, [b T / G, (b + 1) T / G), in
+// runs of one instance each, raw survivors to the instance's second key / index scratch.
+__global__ void __launch_bounds__(BT_BLOCK)
 kb_stream(BatchStar a) {
-  extern __shared__ __align__(16) unsigned char bt_smem[];
+  extern __shared__ __align__(128) unsigned char bt_smem[];
   StreamSmem& S = *reinterpret_cast<StreamSmem*>(bt_smem);
   const int wid = threadIdx.x >> 5;
   const int t1 = (int)(((long long)(blockIdx.x + 1) * a.ntiles) / gridDim.x);
   int t = (int)(((long long)blockIdx.x * a.ntiles) / gridDim.x);
-  while (t < t1) {
-    int lo = 0, hi = a.nh - 1;        // the last instance whose first tile is at most t
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (a.tfirst[mid] <= t) lo = mid; else hi = mid - 1;
-    }
+  star::Ring<BT_STAGES, BT_CH> ring{&S.ring[wid][0][0], S.bar[wid], 0u, true};
+  ring.init();
+  int lo = 0, hi = a.nh - 1;          // the last instance whose first tile is at most t
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (a.tfirst[mid] <= t) lo = mid; else hi = mid - 1;
+  }
+  for (; t < t1; ++lo) {
     const int tf = a.tfirst[lo], te = min(t1, a.tfirst[lo + 1]);
     const int inst = a.order[lo];
     const long long off = a.offsets[inst];
@@ -214,11 +243,12 @@ kb_stream(BatchStar a) {
     const long long sl = a.slot0[inst];
     BRec& R = reinterpret_cast<BRec*>(a.rec)[lo];
     const u32 p0 = (u32)(t - tf) * BF_TILE, p1 = min(n, (u32)(te - tf) * BF_TILE);
-    const PolyHead H = R.head;
+    PolyHead H;
     star::RawSink<BF_NB, BT_SLICE> sink{S.sxy[wid], S.sidx[wid], 0u, &R.frame, &R.raw_count, a.error, R.key,
                                         reinterpret_cast<int2*>(a.kb + sl), a.ib + sl, n};
-    star::stream_points<BT_V>(reinterpret_cast<const int2*>(a.xy) + off + p0, p1 - p0, p0, (u32)wid, (u32)BT_WARPS, H,
-                              S.tab, sink, [&] {
+    star::stream_ring(ring, reinterpret_cast<const int2*>(a.xy) + off + p0, p1 - p0, p0, (u32)wid, (u32)BT_WARPS, H,
+                      S.tab, sink, a.error, [&] {
+      H = R.head;
       for (u32 q = threadIdx.x; q < H.nslab; q += BT_BLOCK) S.tab[q] = R.tab[q];
       __syncthreads();
     });
@@ -228,7 +258,7 @@ kb_stream(BatchStar a) {
   }
 }
 
-constexpr int BE_BLOCK = 512;
+constexpr int BE_BLOCK = 256;
 
 struct FinishSmem {
   star::ListSmem<BE_BLOCK, BF_CAP, BF_NB> list;
@@ -236,7 +266,7 @@ struct FinishSmem {
   u32 count;
 };
 
-__global__ void __launch_bounds__(BE_BLOCK, 3)
+__global__ void __launch_bounds__(BE_BLOCK, 4)
 kb_finish(BatchStar a) {
   extern __shared__ __align__(16) unsigned char be_smem[];
   FinishSmem& S = *reinterpret_cast<FinishSmem*>(be_smem);
@@ -331,7 +361,7 @@ cudaError_t launch_batch_star_small(const BatchStar& a, int num_sms, cudaStream_
 cudaError_t launch_batch_star_large(const BatchStar& a, int num_sms, cudaStream_t st) {
   if (a.nh <= 0) return cudaSuccess;
   kb_poly<<<a.nh, BP_BLOCK, 0, st>>>(a);
-  const int cap = num_sms * 2;
+  const int cap = num_sms * (512 / BT_BLOCK);
   kb_stream<<<a.ntiles < cap ? a.ntiles : cap, BT_BLOCK, sizeof(StreamSmem), st>>>(a);
   kb_finish<<<a.nh, BE_BLOCK, sizeof(FinishSmem), st>>>(a);
   return cudaGetLastError();

@@ -9,9 +9,10 @@
 // polygon and the table built from it are exact.  The last block builds both
 // (star::build_poly).
 //
-// Sample: about n / 256 points (at least 4,096), one per thread and round: a
-// 20M disk keeps 0.3 % of its points against 0.64 % for 32 directions of n /
-// 1,024 points (the area outside a regular 32-gon alone), for 5 MB more read.
+// Sample: about n / 128 points (at least 4,096) in runs of four, one per
+// thread and round: a 20M disk keeps 0.3 % of its points against 0.64 % for
+// 32 directions of n / 1,024 points (the area outside a regular 32-gon
+// alone), for 2.5 MB read.
 #include "hull_internal.cuh"
 #include "kernels.h"
 #include "star.cuh"
@@ -33,14 +34,14 @@ __global__ void __launch_bounds__(K0_BLOCK)
 k0_poly(const int2* __restrict__ P, u32 n, u32 ns, u32 slabs, PolyTab* __restrict__ T) {
   __shared__ K0Smem S;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, t = threadIdx.x;
-  const u32 stride = n / ns, step = gridDim.x * K0_BLOCK;
+  const u32 stride = n / (ns / 4u), step = gridDim.x * K0_BLOCK;
   u32 i = blockIdx.x * K0_BLOCK + t;
-  int2 p = i < ns ? P[(size_t)i * stride] : make_int2(0, 0);
+  int2 p = i < ns ? P[star::sample_at(i, stride)] : make_int2(0, 0);
   if (t < kPolyDirs) S.best[t] = 0ull;
   const StarFrame F = star::make_frame<K0_BLOCK>(P, n, S.frame);    // its barriers publish S.best
   while (i < ns) {
     const u32 i1 = i + step;
-    const int2 p1 = i1 < ns ? P[(size_t)i1 * stride] : make_int2(0, 0);
+    const int2 p1 = i1 < ns ? P[star::sample_at(i1, stride)] : make_int2(0, 0);
     star::offer_sample(F, p, i, S.best);
     p = p1;
     i = i1;
@@ -60,7 +61,7 @@ k0_poly(const int2* __restrict__ P, u32 n, u32 ns, u32 slabs, PolyTab* __restric
   if (t < kPolyDirs) {
     __threadfence();
     const u64 v = *reinterpret_cast<volatile u64*>(&T->best[t]);
-    S.poly.p[t] = v ? P[(size_t)(~(u32)v) * stride] : make_int2(0, 0);
+    S.poly.p[t] = v ? P[star::sample_at(~(u32)v, stride)] : make_int2(0, 0);
     const u32 h = __ballot_sync(0xFFFFFFFFu, v != 0ull);
     if (lane == 0) S.poly.has[wid] = h;
   }
@@ -75,9 +76,10 @@ k0_poly(const int2* __restrict__ P, u32 n, u32 ns, u32 slabs, PolyTab* __restric
 }  // namespace
 
 cudaError_t launch_poly(const int* xy, u32 n, PolyTab* T, int num_sms, cudaStream_t st) {
-  u32 ns = n / 256u;
+  u32 ns = n / 128u;
   if (ns < 4096u) ns = 4096u;
   if (ns > n) ns = n;
+  ns &= ~3u;                          // whole runs; n is above 4,096
   u32 grid = (ns + K0_BLOCK - 1) / K0_BLOCK;
   if (grid > (u32)num_sms) grid = (u32)num_sms;
   // Slabs: the staircase left outside takes about one slab's width of every

@@ -172,6 +172,7 @@ ks_sectors(const PolyTab* __restrict__ T, u32 n, SectorTab* D, int2* xy, u32* id
   }
   __syncthreads();
   unsigned short* cur = S.ta;
+  star::mend_order<SB_BLOCK, true>(S, m, F, cur);
   bool done;
   const u32 left = star::drop_rounds<SB_BLOCK, true>(S, m, F, S.tb, cur, true, done);
   __syncthreads();
@@ -240,6 +241,7 @@ ks_rounds(const PolyTab* __restrict__ T, u32 n, SectorTab* D, int pass, const in
   }
   __syncthreads();
   unsigned short* cur = S.ta;
+  star::mend_order<SB_BLOCK, true>(S, m, F, cur);
   bool done;
   const u32 left = star::drop_rounds<SB_BLOCK, true>(S, m, F, S.tb, cur, false, done);
   __syncthreads();

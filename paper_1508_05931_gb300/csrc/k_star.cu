@@ -132,7 +132,7 @@ k_star(const int2* __restrict__ P, u32 n, PolyTab* T, const int2* __restrict__ r
   }
   if (t == 0) star_summary(plan, n, q, m, h, cap, err);
   // Decided: the table is left clear for the next call.
-  if (h >= 0 || (err & ERR_RANGE)) {
+  if (h >= 0) {
     static_assert(kPolyClearBytes % sizeof(u64) == 0, "whole words");
     u64* w = reinterpret_cast<u64*>(T);
     for (u32 i = t; i < (u32)(kPolyClearBytes / sizeof(u64)); i += KS_BLOCK) w[i] = 0ull;
@@ -146,29 +146,39 @@ k_small(const int2* __restrict__ P, u32 n, Plan* plan, int* out, long long cap) 
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, t = threadIdx.x;
   if (t == 0) { S.count = 0u; S.error = 0u; }
   if (t < kPolyDirs) S.best[t] = 0ull;
-  const StarFrame F = star::make_frame<KS_BLOCK>(P, n, S.frame);
+  StarFrame F;
   u32 m0 = n;
   bool bad = false, flat = false;
   if (n <= KS_DIRECT) {
-    for (u32 i = t; i < n; i += KS_BLOCK) {
-      const int2 p = P[i];
-      S.list.p[i] = p;
-      S.list.id[i] = i;
-      bad = bad || star::out_of_range(p.x, p.y);
-    }
-  } else {
-    constexpr u32 NS = KS_SAMPLES * KS_BLOCK;
-    static_assert(NS <= KS_DIRECT, "a stride of at least one point");
-    const u32 stride = n / NS;
+    static_assert(KS_DIRECT <= KS_SAMPLES * KS_BLOCK, "the points in registers");
     int2 p[KS_SAMPLES];
     #pragma unroll
-    for (int r = 0; r < KS_SAMPLES; ++r) p[r] = P[(r * KS_BLOCK + t) * stride];
+    for (int r = 0; r < KS_SAMPLES; ++r) p[r] = r * KS_BLOCK + t < n ? P[r * KS_BLOCK + t] : make_int2(0, 0);
+    F = star::make_frame<KS_BLOCK>(P, n, S.frame);
+    #pragma unroll
+    for (int r = 0; r < KS_SAMPLES; ++r) {
+      const u32 i = r * KS_BLOCK + t;
+      if (i < n) {
+        S.list.p[i] = p[r];
+        S.list.id[i] = i;
+        bad = bad || star::out_of_range(p[r].x, p[r].y);
+      }
+    }
+  } else {
+    // The sample, in runs of four points, also gives the frame.
+    constexpr u32 NS = KS_SAMPLES * KS_BLOCK;
+    static_assert(NS <= KS_DIRECT && KS_SAMPLES % 4 == 0, "whole runs, a stride of at least their length");
+    const u32 stride = n / (NS / 4u);
+    int2 p[KS_SAMPLES];
+    #pragma unroll
+    for (int r = 0; r < KS_SAMPLES; ++r) p[r] = P[star::sample_at(r * KS_BLOCK + t, stride)];
+    F = star::frame_of<KS_BLOCK>(p, P[0], S.frame);
     #pragma unroll
     for (int r = 0; r < KS_SAMPLES; ++r) star::offer_sample(F, p[r], r * KS_BLOCK + t, S.best);
     __syncthreads();
     if (t < kPolyDirs) {
       const u32 i = ~(u32)S.best[t];
-      S.poly.p[t] = i < NS ? P[i * stride] : make_int2(0, 0);
+      S.poly.p[t] = i < NS ? P[star::sample_at(i, stride)] : make_int2(0, 0);
       const u32 h = __ballot_sync(0xFFFFFFFFu, i < NS);
       if (lane == 0) S.poly.has[wid] = h;
     }

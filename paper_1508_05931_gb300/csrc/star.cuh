@@ -89,8 +89,8 @@ __device__ __forceinline__ u32 block_scan(u32 v, u32* ws, u32& total) {
 }
 
 // ---------------------------------------------------------------- frame
-// From BLOCK strided points of P[0, n): c, their mean rounded to integers,
-// and the whitening map of their covariance (the inverse Cholesky factor,
+// From strided points (V of every thread, relative to one point o of the
+// input): c, their mean rounded to integers, and the whitening map of their covariance (the inverse Cholesky factor,
 // determinant > 0).  Every block that calls it with the same P and n gets
 // the same frame.  Nothing is assumed of c: a polygon of input points that
 // verifies about it proves that it lies inside.
@@ -99,14 +99,16 @@ struct FrameSmem {
   float sum[BLOCK / 32][5];
 };
 
-template <int BLOCK>
-__device__ __forceinline__ StarFrame make_frame(const int2* __restrict__ P, u32 n, FrameSmem<BLOCK>& S) {
+template <int BLOCK, int V>
+__device__ __forceinline__ StarFrame frame_of(const int2 (&p)[V], int2 o, FrameSmem<BLOCK>& S) {
   constexpr int W = BLOCK / 32;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int2 o = P[0];
-  const int2 p = P[(u32)(((u64)threadIdx.x * n) / BLOCK)];
-  const float fx = (float)p.x - (float)o.x, fy = (float)p.y - (float)o.y;
-  float s[5] = {fx, fy, fx * fx, fx * fy, fy * fy};
+  float s[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+  #pragma unroll
+  for (int r = 0; r < V; ++r) {
+    const float fx = (float)p[r].x - (float)o.x, fy = (float)p[r].y - (float)o.y;
+    s[0] += fx; s[1] += fy; s[2] += fx * fx; s[3] += fx * fy; s[4] += fy * fy;
+  }
   #pragma unroll
   for (int k = 0; k < 5; ++k) {
     #pragma unroll
@@ -119,7 +121,7 @@ __device__ __forceinline__ StarFrame make_frame(const int2* __restrict__ P, u32 
     s[k] = lane < W ? S.sum[lane][k] : 0.0f;
     #pragma unroll
     for (int d = 16; d > 0; d >>= 1) s[k] += __shfl_xor_sync(0xFFFFFFFFu, s[k], d);
-    s[k] *= 1.0f / (float)BLOCK;
+    s[k] *= 1.0f / (float)(BLOCK * V);
   }
   const float mx = s[0], my = s[1];
   const float a = fmaxf(s[2] - mx * mx, 1.0f), d = fmaxf(s[4] - my * my, 1.0f), b = s[3] - mx * my;
@@ -135,12 +137,22 @@ __device__ __forceinline__ StarFrame make_frame(const int2* __restrict__ P, u32 
   return F;
 }
 
+template <int BLOCK>
+__device__ __forceinline__ StarFrame make_frame(const int2* __restrict__ P, u32 n, FrameSmem<BLOCK>& S) {
+  const int2 p[1] = {P[(u32)(((u64)threadIdx.x * n) / BLOCK)]};
+  return frame_of<BLOCK>(p, P[0], S);
+}
+
 // ---------------------------------------------------------------- sample polygon
 // The sample's candidates: per angular sector (kPolyDirs of them) the point
 // of the largest whitened radius (cand_key of the sample's position).  One
 // sector per sample: projecting every sample on every direction found the
 // same polygon at 30 times the instructions (8,500 cycles of a 1,024-thread
 // block for 2,048 samples).
+// Sample i of n / stride4 runs of four consecutive points (a run is one
+// 32-byte sector: four samples for the traffic of one).
+__device__ __forceinline__ size_t sample_at(u32 i, u32 stride4) { return (size_t)(i >> 2) * stride4 + (i & 3u); }
+
 __device__ __forceinline__ void offer_sample(const StarFrame& F, int2 p, u32 pos, u64* best) {
   float u, v;
   to_uv(F, p.x - F.cx, p.y - F.cy, u, v);
@@ -374,20 +386,152 @@ struct RawSink {
     __syncwarp();
     fill = 0;
   }
+  // Bit 2 u + v of m: the lane's point at[64 u + v] survives (index id + 64 u
+  // + v); the whole warp calls it, at most SLICE points in all.  A scan over
+  // the lanes and a loop over each one's few points: a ballot per slot cost
+  // as much as the tests themselves where one point in fifty survives.
+  __device__ __forceinline__ void push_lanes(u32 m, const int2* at, u32 id) {
+    const int lane = threadIdx.x & 31;
+    const u32 c = __popc(m);
+    u32 inc = c;
+    #pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const u32 t = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+      if (lane >= o) inc += t;
+    }
+    const u32 tot = __shfl_sync(0xFFFFFFFFu, inc, 31);
+    if (fill + tot > (u32)SLICE) flush();
+    u32 q = fill + inc - c;
+    while (m) {
+      const u32 e = __ffs(m) - 1u;
+      m &= m - 1u;
+      const u32 k = 64u * (e >> 1) + (e & 1u);
+      sxy[q] = at[k];
+      sidx[q] = id + k;
+      ++q;
+    }
+    fill += tot;
+  }
   // One point per lane (the whole warp calls it; out: the point survives).
   __device__ __forceinline__ void push(bool out, int x, int y, u32 id) {
     const u32 bal = __ballot_sync(0xFFFFFFFFu, out);
     if (bal) {
+      if (fill + __popc(bal) > (u32)SLICE) flush();
       if (out) {
         const u32 q = fill + __popc(bal & ((1u << (threadIdx.x & 31)) - 1u));
         sxy[q] = make_int2(x, y);
         sidx[q] = id;
       }
       fill += __popc(bal);
-      if (fill > (u32)SLICE - 32u) flush();
     }
   }
 };
+
+// N pairs of points per lane (pair u has indices id + 64 u and the next): all
+// tested first (independent lookups in flight together), one vote for the
+// warp, then the survivors pushed slot by slot.
+template <int N, class Sink>
+__device__ __forceinline__ void take_pairs(const PolyHead& H, const u32* tab, const int4* w, u32 id, Sink& sink) {
+  u32 m = 0;
+  #pragma unroll
+  for (int u = 0; u < N; ++u) {
+    m |= inside_poly(H, tab, w[u].x, w[u].y) ? 0u : 1u << (2 * u);
+    m |= inside_poly(H, tab, w[u].z, w[u].w) ? 0u : 2u << (2 * u);
+  }
+  if (__any_sync(0xFFFFFFFFu, m != 0u)) {
+    #pragma unroll
+    for (int u = 0; u < N; ++u) {
+      sink.push((m >> (2 * u)) & 1u, w[u].x, w[u].y, id + 64u * u);
+      sink.push((m >> (2 * u + 1)) & 1u, w[u].z, w[u].w, id + 64u * u + 1u);
+    }
+  }
+}
+
+// The same through a ring of bulk copies into shared memory, one ring per
+// warp (STAGES chunks of CH points; no block barrier, no registers held by
+// loads in flight: 64 registers a thread for the register double buffer kept
+// every other kernel off the SM).  The warp takes chunks first + k step.
+// Waits are bounded (kBulkWaitLimit); one that runs out sets ERR_TIMEOUT.
+template <int STAGES, int CH>
+struct Ring {
+  int4* buf;                // [STAGES][CH / 2], this warp's
+  u64* bar;                 // [STAGES]
+  u32 it;                   // chunks consumed so far
+  bool ok;                  // no wait has run out
+
+  // Whole warp, once; `buf` and `bar` are this warp's alone.
+  __device__ __forceinline__ void init() {
+    it = 0;
+    ok = true;
+    if ((threadIdx.x & 31) == 0) {
+      for (int k = 0; k < STAGES; ++k) mbar_init(&bar[k], 1u);
+      mbar_fence_init();
+    }
+    __syncwarp();
+  }
+  // Lane 0: chunk number `at` of the ring's sequence from src.
+  __device__ __forceinline__ void load(u32 at, const int4* src, u64 pol) {
+    const u32 st = at % STAGES;
+    mbar_arrive_expect_tx(&bar[st], CH * 8u);
+    bulk_load_hint(buf + st * (CH / 2), src, CH * 8u, &bar[st], pol);
+  }
+};
+
+template <int STAGES, int CH, class Sink, class Prep>
+__device__ __forceinline__ void stream_ring(Ring<STAGES, CH>& ring, const int2* __restrict__ Q, u32 cnt, u32 id0,
+                                            u32 first, u32 step, const PolyHead& H, const u32* tab, Sink& sink,
+                                            u32* error, Prep prep) {
+  static_assert(CH % 64 == 0 && CH <= 512, "whole pairs per lane, one mask bit per point");
+  constexpr u32 R = CH / 2;                       // pairs per chunk
+  const int lane = threadIdx.x & 31;
+  const u32 head = (reinterpret_cast<uintptr_t>(Q) & 15u) && cnt ? 1u : 0u;
+  const int4* p4 = reinterpret_cast<const int4*>(Q + head);
+  const u32 npair = (cnt - head) >> 1;
+  const u32 nfull = npair / R;
+  const u32 mine = ring.ok && first < nfull ? (nfull - 1u - first) / step + 1u : 0u;
+  const u64 pol = policy_evict_first();
+  if (lane == 0)
+    for (u32 k = 0; k < min(mine, (u32)STAGES); ++k) ring.load(ring.it + k, p4 + (size_t)(first + k * step) * R, pol);
+  prep();
+  for (u32 k = 0; k < mine; ++k, ++ring.it) {
+    const u32 st = ring.it % STAGES;
+    if (!mbar_wait(&ring.bar[st], (ring.it / STAGES) & 1u)) {
+      atomicOr(error, ERR_TIMEOUT);
+      ring.ok = false;                // the copies still in flight get their time too
+      for (u32 j = 1; j < (u32)STAGES && k + j < mine; ++j)
+        mbar_wait(&ring.bar[(ring.it + j) % STAGES], ((ring.it + j) / STAGES) & 1u);
+      break;
+    }
+    const int4* b = ring.buf + st * R + lane;
+    const u32 id = id0 + head + 2u * ((first + k * step) * R + lane);
+    u32 m = 0;                        // the lane's points outside, pair u's at bits 2 u and 2 u + 1
+    #pragma unroll
+    for (int u = 0; u < (int)R / 32; ++u) {
+      const int4 w = b[32 * u];
+      m |= inside_poly(H, tab, w.x, w.y) ? 0u : 1u << (2 * u);
+      m |= inside_poly(H, tab, w.z, w.w) ? 0u : 2u << (2 * u);
+    }
+    if (__any_sync(0xFFFFFFFFu, m != 0u)) sink.push_lanes(m, reinterpret_cast<const int2*>(b), id);
+    __syncwarp();
+    if (lane == 0 && k + STAGES < mine) ring.load(ring.it + STAGES, p4 + (size_t)(first + (k + STAGES) * step) * R, pol);
+  }
+  // The pairs past the last full chunk, and the points outside the pairs: one warp.
+  if (first == nfull % step) {
+    for (u32 b = nfull * R; b < npair; b += 32u) {
+      const u32 j = b + lane;
+      const bool in = j < npair;
+      const int4 w = in ? p4[j] : make_int4(0, 0, 0, 0);
+      const u32 id = id0 + head + 2u * j;
+      sink.push(in && !inside_poly(H, tab, w.x, w.y), w.x, w.y, id);
+      sink.push(in && !inside_poly(H, tab, w.z, w.w), w.z, w.w, id + 1u);
+    }
+    const u32 rest = (cnt - head) & 1u;
+    const bool in = lane < 2 && (lane == 0 ? head : rest) != 0u;
+    const u32 j = lane == 0 ? 0u : cnt - 1u;
+    const int2 p = in ? Q[j] : make_int2(0, 0);
+    sink.push(in && !inside_poly(H, tab, p.x, p.y), p.x, p.y, id0 + j);
+  }
+}
 
 // The stream's sink of a block that finishes its points itself: its list.
 template <class L>
@@ -439,12 +583,7 @@ __device__ __forceinline__ void stream_points(const int2* __restrict__ Q, u32 cn
       #pragma unroll
       for (int u = 0; u < V; ++u) nxt[u] = p4[w1 + lane + 32u * u];
     }
-    #pragma unroll
-    for (int u = 0; u < V; ++u) {
-      const u32 id = id0 + head + 2u * (w0 + lane + 32u * u);
-      sink.push(!inside_poly(H, tab, cur[u].x, cur[u].y), cur[u].x, cur[u].y, id);
-      sink.push(!inside_poly(H, tab, cur[u].z, cur[u].w), cur[u].z, cur[u].w, id + 1u);
-    }
+    take_pairs<V>(H, tab, cur, id0 + head + 2u * (w0 + lane), sink);
     #pragma unroll
     for (int u = 0; u < V; ++u) cur[u] = nxt[u];
     w0 = w1;
@@ -557,6 +696,27 @@ __device__ __forceinline__ u32 bin_rank(const int2* p, const u32* id, const unsi
     if (dr > qr || (dr == qr && id[kj] < qi)) { ++r; dead = true; }
   }
   return r;
+}
+
+// Neighbours in cur[0, m) that stand in the wrong order about c change
+// places, twice over the even and the odd pairs: points of adjacent bins
+// whose angles are closer than the float bins tell them apart (elongated
+// sets lose digits to the whitening).  OPEN: the ends are no neighbours.
+// Ends with a barrier.
+template <int BLOCK, bool OPEN, class L>
+__device__ __forceinline__ void mend_order(const L& S, u32 m, const StarFrame& F, unsigned short* cur) {
+  #pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    for (u32 i = 2u * threadIdx.x + (k & 1u); i < m; i += 2u * BLOCK) {
+      const u32 j = i + 1u < m ? i + 1u : 0u;
+      if (j == 0u && (OPEN || (i & 1u) == 0u)) continue;   // (no wrapping pair of an odd number of entries)
+      const unsigned short a = cur[i], b = cur[j];
+      const int2 p = S.p[a & 0x7FFFu], q = S.p[b & 0x7FFFu];
+      const int ax = p.x - F.cx, ay = p.y - F.cy, bx = q.x - F.cx, by = q.y - F.cy;
+      if (cross2(ax, ay, bx, by) < 0 && (long long)ax * bx + (long long)ay * by > 0) { cur[i] = b; cur[j] = a; }
+    }
+    __syncthreads();
+  }
 }
 
 // The rounds over the entries cur[0, m) (positions in S.p in angular order,
@@ -678,6 +838,7 @@ __device__ int list_hull(ListSmem<BLOCK, CAP, NB>& S, u32 m, const StarFrame& F,
   }
   __syncthreads();
   unsigned short* cur = S.ta;
+  mend_order<BLOCK, false>(S, m, F, cur);
   bool done = false;
   m = drop_rounds<BLOCK, false>(S, m, F, S.tb, cur, true, done);
   if (!done) return -1;
