@@ -157,7 +157,8 @@ struct hull_ctx {
   int* ext_xy = nullptr;        // and their coordinates
   unsigned long long* lab_cnt = nullptr;   // 33 label counters
   float* d_loss = nullptr;
-  float* grad = nullptr;
+  float* grad = nullptr;        // the gradient, then the loss (d_loss)
+  float* h_grad = nullptr;      // pinned copy of both
   size_t train_cap = 0;         // rows of the training scratch
   float* act = nullptr;
   float* scratch = nullptr;
@@ -771,15 +772,17 @@ hull_status hull_create(hull_ctx** out, int device, const hull_config* cfg) {
     const size_t np = (size_t)mlp_num_params();
     if (cudaMalloc(&c->W, np * 4) != cudaSuccess || cudaMalloc(&c->W16, np * 2) != cudaSuccess ||
         cudaMalloc(&c->adam_m, np * 4) != cudaSuccess || cudaMalloc(&c->adam_v, np * 4) != cudaSuccess ||
-        cudaMalloc(&c->grad, np * 4) != cudaSuccess || cudaMalloc(&c->feat, 64 * 4) != cudaSuccess ||
+        cudaMalloc(&c->grad, (np + 4) * 4) != cudaSuccess || cudaMalloc(&c->feat, 64 * 4) != cudaSuccess ||
         cudaMalloc(&c->ext, 32 * 4) != cudaSuccess || cudaMalloc(&c->ext_xy, 64 * 4) != cudaSuccess ||
-        cudaMalloc(&c->lab_cnt, 33 * 8) != cudaSuccess || cudaMalloc(&c->d_loss, 16) != cudaSuccess) {
+        cudaMalloc(&c->lab_cnt, 33 * 8) != cudaSuccess || cudaMallocHost(&c->h_grad, (np + 1) * 4) != cudaSuccess ||
+        mlp_configure() != cudaSuccess) {
       cudaGetLastError();
       *out = c;
       hull_destroy(c);
       *out = nullptr;
       return HULL_ENOMEM;
     }
+    c->d_loss = c->grad + np;
     cudaMemset(c->W, 0, np * 4);
     cudaMemset(c->W16, 0, np * 2);
     cudaMemset(c->adam_m, 0, np * 4);
@@ -808,7 +811,7 @@ void hull_destroy(hull_ctx* c) {
   for (int k = 0; k <= HULL_NUM_STAGES; ++k)
     if (c->ev[k]) cudaEventDestroy(c->ev[k]);
   for (void* p : {(void*)c->W, c->W16, (void*)c->adam_m, (void*)c->adam_v, (void*)c->grad, (void*)c->feat,
-                  (void*)c->ext, (void*)c->ext_xy, (void*)c->lab_cnt, (void*)c->d_loss, (void*)c->act,
+                  (void*)c->ext, (void*)c->ext_xy, (void*)c->lab_cnt, (void*)c->act,
                   (void*)c->scratch})
     if (p) cudaFree(p);
   if (c->bw.base) cudaFree(c->bw.base);
@@ -824,6 +827,7 @@ void hull_destroy(hull_ctx* c) {
   if (c->aux) cudaStreamDestroy(c->aux);
   if (c->plan) cudaFree(c->plan);
   if (c->h_plan) cudaFreeHost(c->h_plan);
+  if (c->h_grad) cudaFreeHost(c->h_grad);
   if (c->h_multi) cudaFreeHost(c->h_multi);
   delete c;
 }
@@ -1632,7 +1636,7 @@ static hull_status ensure_train(hull_ctx* c, int B) {
   c->act = nullptr; c->scratch = nullptr; c->train_cap = 0;
   const size_t rows = (size_t)B;
   if (cudaMalloc(&c->act, rows * (128 + 128 + 32) * 4) != cudaSuccess ||
-      cudaMalloc(&c->scratch, rows * (128 + 128 + 32) * 4) != cudaSuccess) {
+      cudaMalloc(&c->scratch, mlp_scratch_floats(B) * 4) != cudaSuccess) {
     cudaGetLastError();
     return HULL_ENOMEM;
   }
@@ -1660,15 +1664,15 @@ hull_status hull_mlp_gradient(hull_ctx* c, const float* d_X, const float* d_Y, i
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   hull_status r = ensure_train(c, B);
   if (r != HULL_OK) return r;
-  cudaError_t e = mlp_forward(c->W, d_X, B, c->act, st);
-  if (e == cudaSuccess) e = mlp_backward(c->W, d_X, d_Y, B, c->act, c->grad, c->d_loss, c->scratch, st);
-  if (e == cudaSuccess && h_grad)
-    e = cudaMemcpyAsync(h_grad, c->grad, (size_t)mlp_num_params() * 4, cudaMemcpyDeviceToHost, st);
-  float loss = 0.f;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&loss, c->d_loss, 4, cudaMemcpyDeviceToHost, st);
+  const size_t np = (size_t)mlp_num_params();
+  cudaError_t e = mlp_gradient(c->W, d_X, d_Y, B, c->act, c->grad, c->d_loss, c->scratch, st);
+  // Gradient and loss (behind it) in one copy to pinned memory: a pageable
+  // destination would be staged by the driver, twice.
+  if (e == cudaSuccess) e = cudaMemcpyAsync(c->h_grad, c->grad, (np + 1) * 4, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_fail(e);
-  if (h_loss) *h_loss = loss;
+  if (h_grad) std::memcpy(h_grad, c->h_grad, np * 4);
+  if (h_loss) *h_loss = c->h_grad[np];
   return HULL_OK;
 }
 
@@ -1679,8 +1683,7 @@ hull_status hull_mlp_train_step(hull_ctx* c, const float* d_X, const float* d_Y,
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   hull_status r = ensure_train(c, B);
   if (r != HULL_OK) return r;
-  cudaError_t e = mlp_forward(c->W, d_X, B, c->act, st);
-  if (e == cudaSuccess) e = mlp_backward(c->W, d_X, d_Y, B, c->act, c->grad, c->d_loss, c->scratch, st);
+  cudaError_t e = mlp_gradient(c->W, d_X, d_Y, B, c->act, c->grad, c->d_loss, c->scratch, st);
   if (e == cudaSuccess) e = mlp_adam(c->W, c->grad, c->adam_m, c->adam_v, c->adam_step + 1, lr, c->W16, st);
   float loss = 0.f;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&loss, c->d_loss, 4, cudaMemcpyDeviceToHost, st);

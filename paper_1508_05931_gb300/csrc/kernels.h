@@ -237,8 +237,10 @@ cudaError_t launch_labels(const int* xy, u32 n, const int* quad, int nq, const i
                           unsigned long long* counts, int grid, cudaStream_t st);
 cudaError_t launch_to_half(const float* w, void* w16, int count, cudaStream_t st);
 cudaError_t mlp_forward(const float* W, const float* X, int B, float* act, cudaStream_t st);
-cudaError_t mlp_backward(const float* W, const float* X, const float* Y, int B, const float* act,
-                         float* grad, float* loss, float* scratch, cudaStream_t st);
+size_t mlp_scratch_floats(int B);
+cudaError_t mlp_configure();
+cudaError_t mlp_gradient(const float* W, const float* X, const float* Y, int B, float* act, float* grad, float* loss,
+                         float* scratch, cudaStream_t st);
 cudaError_t mlp_adam(float* W, const float* grad, float* m, float* v, int step, float lr,
                      void* w16, cudaStream_t st);
 

@@ -14,9 +14,9 @@
 //       points, so the hull stays exact whatever the weights;
 //   K10 labels for training: for every direction j the discard fraction of
 //       hull(quad corners + e_j) minus the quadrilateral's, counted exactly;
-//   training: batched forward / backward of the MLP (FP32 FFMA tiles, the
-//       forward pass on the FP16-rounded weights used at inference), mean
-//       squared error on the labels, Adam on FP32 master weights.
+//   training: batched forward / backward of the MLP (FP32 FFMA, on the
+//       FP16-rounded weights used at inference), mean squared error on the
+//       labels, Adam on FP32 master weights.
 #include <cmath>
 
 #include "hull_internal.cuh"
@@ -152,13 +152,11 @@ k10_labels(const int* __restrict__ xy, u32 n, const int* __restrict__ quad, int 
 }
 
 // ---------------------------------------------------------------- training
-// C[M x N] (row-major, ldc = N) = op(A) * op(B) (+ bias[N]) (ReLU) with
-// op(A): A (M x K, lda) or A^T; op(B): B^T (B stored N x K) or B (K x N).
-// Weights used by the forward pass are rounded to FP16 (round_b).
-template <bool TA, bool TB>
+// C[M x N] (row-major) = A (M x K) B^T (B stored N x K) + bias (ReLU), the
+// weights and biases rounded to FP16.
 __global__ void __launch_bounds__(256)
-k_gemm(const float* __restrict__ A, int lda, const float* __restrict__ Bm, int ldb, float* __restrict__ C,
-       int M, int N, int K, const float* __restrict__ bias, int relu, int round_b, float beta) {
+k_gemm(const float* __restrict__ A, const float* __restrict__ Bm, float* __restrict__ C, int M, int N, int K,
+       const float* __restrict__ bias, int relu) {
   __shared__ float sa[16][17], sb[16][17];
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   const int row = blockIdx.y * 16 + ty, col = blockIdx.x * 16 + tx;
@@ -166,10 +164,8 @@ k_gemm(const float* __restrict__ A, int lda, const float* __restrict__ Bm, int l
   for (int k0 = 0; k0 < K; k0 += 16) {
     const int ka = k0 + tx, kb = k0 + ty;
     float av = 0.f, bv = 0.f;
-    if (row < M && ka < K) av = TA ? A[(size_t)ka * lda + row] : A[(size_t)row * lda + ka];
-    const int bc = blockIdx.x * 16 + tx;
-    if (bc < N && kb < K) bv = TB ? Bm[(size_t)kb * ldb + bc] : Bm[(size_t)bc * ldb + kb];
-    if (round_b) bv = fp16r(bv);
+    if (row < M && ka < K) av = A[(size_t)row * K + ka];
+    if (col < N && kb < K) bv = fp16r(Bm[(size_t)col * K + kb]);
     sa[ty][tx] = av;
     sb[ty][tx] = bv;
     __syncthreads();
@@ -178,39 +174,167 @@ k_gemm(const float* __restrict__ A, int lda, const float* __restrict__ Bm, int l
     __syncthreads();
   }
   if (row < M && col < N) {
-    if (bias) acc += round_b ? fp16r(bias[col]) : bias[col];
+    acc += fp16r(bias[col]);
     if (relu) acc = fmaxf(acc, 0.f);
-    C[(size_t)row * N + col] = beta != 0.f ? acc + beta * C[(size_t)row * N + col] : acc;
+    C[(size_t)row * N + col] = acc;
   }
 }
 
-// dZ = 2 (Z - Y) / (B * 32); loss partial sums.
-__global__ void k_mse(const float* __restrict__ Z, const float* __restrict__ Y, float* __restrict__ dZ,
-                      int count, float scale, float* __restrict__ loss) {
-  float l = 0.f;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
-    const float d = Z[i] - Y[i];
-    dZ[i] = 2.f * d * scale;
-    l += d * d;
+// The forward pass and the backward pass down to the layers' pre-activation
+// gradients, in one launch: everything but the parameter gradients is local
+// to a row.  A block takes MR_ROWS rows and all weights (rounded to FP16, 57
+// KB of shared memory, odd word pitches); a thread owns one unit of every
+// layer for two rows, its sums in increasing order of the inputs, as the tile
+// kernel's.  Bound by latency: 14 launches of 3-7 us each (tiles, column sums
+// of one block, masks) took 70 us of device time for 64 rows.
+constexpr int MR_ROWS = 4;
+constexpr int MR_BLOCK = 256;
+
+struct RowSmem {
+  __half w1[D1][D0 + 2], w2[D2][D1 + 2], w3[D3][D2 + 2];
+  float b1[D1], b2[D2], b3[D3];
+  float x[MR_ROWS][D0], h1[MR_ROWS][D1], h2[MR_ROWS][D2], dz[MR_ROWS][D3], d2[MR_ROWS][D2];
+  float loss[MR_ROWS];
+};
+
+// sum over k of in[k] w[k], then + bias, in the tile kernel's order.
+template <int K>
+__device__ __forceinline__ float unit(const float* in, const __half* w, float bias) {
+  float acc = 0.f;
+  #pragma unroll 8
+  for (int k = 0; k < K; k += 2) {
+    const float2 v = __half22float2(*reinterpret_cast<const __half2*>(w + k));
+    acc = fmaf(in[k], v.x, acc);
+    acc = fmaf(in[k + 1], v.y, acc);
+  }
+  return acc + bias;
+}
+
+template <int K, int N>
+__device__ __forceinline__ void load_weights(const float* __restrict__ W, __half (&w)[N][K + 2]) {
+  #pragma unroll 4
+  for (int q = threadIdx.x; q < N * K / 4; q += MR_BLOCK) {
+    const float4 v = reinterpret_cast<const float4*>(W)[q];
+    __half2* d = reinterpret_cast<__half2*>(&w[4 * q / K][4 * q % K]);
+    d[0] = __floats2half2_rn(v.x, v.y);
+    d[1] = __floats2half2_rn(v.z, v.w);
+  }
+}
+
+__global__ void __launch_bounds__(MR_BLOCK)
+k_mlp_rows(const float* __restrict__ W, const float* __restrict__ X, const float* __restrict__ Y, int B, float scale,
+           float* __restrict__ H1, float* __restrict__ H2, float* __restrict__ dZ, float* __restrict__ dH2,
+           float* __restrict__ dH1, float* __restrict__ lossp) {
+  extern __shared__ __align__(16) unsigned char mr_smem[];
+  RowSmem& S = *reinterpret_cast<RowSmem*>(mr_smem);
+  const int t = threadIdx.x, r0 = blockIdx.x * MR_ROWS, nr = min(MR_ROWS, B - r0);
+  static_assert((OFF_W1 % 4) == 0 && (OFF_W2 % 4) == 0 && (OFF_W3 % 4) == 0, "16-byte rows of the weights");
+  load_weights<D0, D1>(W + OFF_W1, S.w1);
+  load_weights<D1, D2>(W + OFF_W2, S.w2);
+  load_weights<D2, D3>(W + OFF_W3, S.w3);
+  if (t < D1) { S.b1[t] = fp16r(W[OFF_B1 + t]); S.b2[t] = fp16r(W[OFF_B2 + t]); }
+  if (t < D3) S.b3[t] = fp16r(W[OFF_B3 + t]);
+  static_assert(MR_ROWS * D0 == MR_BLOCK && D1 == 128 && D2 == 128 && MR_BLOCK == 2 * D1, "thread layout");
+  S.x[t / D0][t % D0] = t / D0 < nr ? X[(size_t)r0 * D0 + t] : 0.f;
+  __syncthreads();
+  const int j = t & (D1 - 1), p = t / D1 * 2;          // unit j of rows p, p + 1
+  #pragma unroll
+  for (int r = p; r < p + 2; ++r) {
+    const float v = fmaxf(unit<D0>(S.x[r], S.w1[j], S.b1[j]), 0.f);
+    S.h1[r][j] = v;
+    if (r < nr) H1[(size_t)(r0 + r) * D1 + j] = v;
+  }
+  __syncthreads();
+  #pragma unroll
+  for (int r = p; r < p + 2; ++r) {
+    const float v = fmaxf(unit<D1>(S.h1[r], S.w2[j], S.b2[j]), 0.f);
+    S.h2[r][j] = v;
+    if (r < nr) H2[(size_t)(r0 + r) * D2 + j] = v;
+  }
+  __syncthreads();
+  if (t < MR_ROWS * D3) {                              // a warp per row
+    const int r = t / D3, q = t % D3;
+    float d = 0.f;
+    if (r < nr) d = unit<D2>(S.h2[r], S.w3[q], S.b3[q]) - Y[(size_t)(r0 + r) * D3 + q];
+    const float g = 2.f * d * scale;
+    S.dz[r][q] = g;
+    if (r < nr) dZ[(size_t)(r0 + r) * D3 + q] = g;
+    float l = d * d;
+    #pragma unroll
+    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xFFFFFFFFu, l, o);
+    if (q == 0) S.loss[r] = l * scale;
+  }
+  __syncthreads();
+  if (t == 0) {
+    float l = 0.f;
+    for (int r = 0; r < MR_ROWS; ++r) l += S.loss[r];
+    lossp[blockIdx.x] = l;
   }
   #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xFFFFFFFFu, l, o);
-  if ((threadIdx.x & 31) == 0) atomicAdd(loss, l * scale);
+  for (int r = p; r < p + 2; ++r) {
+    float acc = 0.f;
+    #pragma unroll 8
+    for (int k = 0; k < D3; ++k) acc = fmaf(S.dz[r][k], __half2float(S.w3[k][j]), acc);
+    if (!(S.h2[r][j] > 0.f)) acc = 0.f;
+    S.d2[r][j] = acc;
+    if (r < nr) dH2[(size_t)(r0 + r) * D2 + j] = acc;
+  }
+  __syncthreads();
+  #pragma unroll
+  for (int r = p; r < p + 2; ++r) {
+    float acc = 0.f;
+    #pragma unroll 8
+    for (int k = 0; k < D2; ++k) acc = fmaf(S.d2[r][k], __half2float(S.w2[k][j]), acc);
+    if (!(S.h1[r][j] > 0.f)) acc = 0.f;
+    if (r < nr) dH1[(size_t)(r0 + r) * D1 + j] = acc;
+  }
 }
 
-// dH *= (H > 0)
-__global__ void k_relu_mask(float* __restrict__ dH, const float* __restrict__ H, int count) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x)
-    if (!(H[i] > 0.f)) dH[i] = 0.f;
-}
+// The parameter gradients, one 16 x 16 tile a block over all three layers:
+// dW = D^T A summed over the rows in increasing order, with D the layer's
+// pre-activation gradient and A its input; the tiles of the first columns
+// also sum db, the first block the loss.
+constexpr int MG_ROWS = 64;            // rows staged at a time
+constexpr int MG_T3 = (D3 / 16) * (D2 / 16), MG_T2 = (D2 / 16) * (D1 / 16), MG_T1 = (D1 / 16) * (D0 / 16);
 
-// db[j] = sum over rows of dZ[:, j]
-__global__ void k_colsum(const float* __restrict__ dZ, int M, int N, float* __restrict__ db) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= N) return;
-  float s = 0.f;
-  for (int r = 0; r < M; ++r) s += dZ[(size_t)r * N + j];
-  db[j] = s;
+__global__ void __launch_bounds__(256)
+k_mlp_grad(const float* __restrict__ X, const float* __restrict__ H1, const float* __restrict__ H2,
+           const float* __restrict__ dZ, const float* __restrict__ dH2, const float* __restrict__ dH1, int B,
+           const float* __restrict__ lossp, int nloss, float* __restrict__ grad, float* __restrict__ loss) {
+  __shared__ float sa[MG_ROWS][17], sb[MG_ROWS][17];
+  int b = blockIdx.x;
+  if (b == 0 && threadIdx.x < 32) {
+    float l = 0.f;
+    for (int q = threadIdx.x; q < nloss; q += 32) l += lossp[q];
+    #pragma unroll
+    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xFFFFFFFFu, l, o);
+    if (threadIdx.x == 0) *loss = l;
+  }
+  const float *D, *A;
+  float *g, *gb;
+  int M, N;
+  if (b < MG_T3) { D = dZ; A = H2; g = grad + OFF_W3; gb = grad + OFF_B3; M = D3; N = D2; }
+  else if (b < MG_T3 + MG_T2) { b -= MG_T3; D = dH2; A = H1; g = grad + OFF_W2; gb = grad + OFF_B2; M = D2; N = D1; }
+  else { b -= MG_T3 + MG_T2; D = dH1; A = X; g = grad + OFF_W1; gb = grad + OFF_B1; M = D1; N = D0; }
+  const int m0 = b / (N / 16) * 16, n0 = b % (N / 16) * 16;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  float acc = 0.f, sum = 0.f;
+  for (int k0 = 0; k0 < B; k0 += MG_ROWS) {
+    const int kn = min(MG_ROWS, B - k0);
+    #pragma unroll
+    for (int q = ty; q < MG_ROWS; q += 16) {
+      sa[q][tx] = q < kn ? D[(size_t)(k0 + q) * M + m0 + tx] : 0.f;
+      sb[q][tx] = q < kn ? A[(size_t)(k0 + q) * N + n0 + tx] : 0.f;
+    }
+    __syncthreads();
+    #pragma unroll 16
+    for (int q = 0; q < MG_ROWS; ++q) acc = fmaf(sa[q][ty], sb[q][tx], acc);
+    if (n0 == 0 && ty == 0)
+      for (int q = 0; q < kn; ++q) sum += sa[q][tx];
+    __syncthreads();
+  }
+  g[(size_t)(m0 + ty) * N + n0 + tx] = acc;
+  if (n0 == 0 && ty == 0) gb[m0 + tx] = sum;
 }
 
 __global__ void k_adam(float* __restrict__ w, const float* __restrict__ g, float* __restrict__ m,
@@ -232,11 +356,10 @@ __global__ void k_to_half(const float* __restrict__ w, __half* __restrict__ w16,
     w16[i] = __float2half_rn(w[i]);
 }
 
-template <bool TA, bool TB>
-void gemm(const float* A, int lda, const float* Bm, int ldb, float* C, int M, int N, int K,
-          const float* bias, int relu, int round_b, float beta, cudaStream_t st) {
+void gemm(const float* A, const float* Bm, float* C, int M, int N, int K, const float* bias, int relu,
+          cudaStream_t st) {
   dim3 grid((N + 15) / 16, (M + 15) / 16);
-  k_gemm<TA, TB><<<grid, 256, 0, st>>>(A, lda, Bm, ldb, C, M, N, K, bias, relu, round_b, beta);
+  k_gemm<<<grid, 256, 0, st>>>(A, Bm, C, M, N, K, bias, relu);
 }
 
 }  // namespace
@@ -277,38 +400,33 @@ cudaError_t mlp_forward(const float* W, const float* X, int B, float* act, cudaS
   float* H1 = act;
   float* H2 = H1 + (size_t)B * D1;
   float* Z = H2 + (size_t)B * D2;
-  gemm<false, false>(X, D0, W + OFF_W1, D0, H1, B, D1, D0, W + OFF_B1, 1, 1, 0.f, st);
-  gemm<false, false>(H1, D1, W + OFF_W2, D1, H2, B, D2, D1, W + OFF_B2, 1, 1, 0.f, st);
-  gemm<false, false>(H2, D2, W + OFF_W3, D2, Z, B, D3, D2, W + OFF_B3, 0, 1, 0.f, st);
+  gemm(X, W + OFF_W1, H1, B, D1, D0, W + OFF_B1, 1, st);
+  gemm(H1, W + OFF_W2, H2, B, D2, D1, W + OFF_B2, 1, st);
+  gemm(H2, W + OFF_W3, Z, B, D3, D2, W + OFF_B3, 0, st);
   return cudaGetLastError();
 }
 
-// Gradient of the mean squared error (over B x 32 entries) with respect to
-// the parameters (evaluated at the FP16-rounded weights); grad and loss are
-// overwritten.  scratch holds 2 * B * 128 + B * 32 floats.
-cudaError_t mlp_backward(const float* W, const float* X, const float* Y, int B, const float* act,
-                         float* grad, float* loss, float* scratch, cudaStream_t st) {
-  const float* H1 = act;
-  const float* H2 = H1 + (size_t)B * D1;
-  const float* Z = H2 + (size_t)B * D2;
+// Forward pass and gradient of the mean squared error (over B x 32 entries)
+// with respect to the parameters (evaluated at the FP16-rounded weights);
+// grad and loss are overwritten.  act holds B * 256 floats, scratch
+// mlp_scratch_floats(B).
+size_t mlp_scratch_floats(int B) { return (size_t)B * (D3 + D2 + D1) + (size_t)(B + MR_ROWS - 1) / MR_ROWS; }
+
+cudaError_t mlp_configure() {
+  return cudaFuncSetAttribute(k_mlp_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RowSmem));
+}
+
+cudaError_t mlp_gradient(const float* W, const float* X, const float* Y, int B, float* act, float* grad, float* loss,
+                         float* scratch, cudaStream_t st) {
+  float* H1 = act;
+  float* H2 = H1 + (size_t)B * D1;
   float* dZ = scratch;
   float* dH2 = dZ + (size_t)B * D3;
   float* dH1 = dH2 + (size_t)B * D2;
-  cudaMemsetAsync(loss, 0, sizeof(float), st);
-  k_mse<<<64, 256, 0, st>>>(Z, Y, dZ, B * D3, 1.f / (float)(B * D3), loss);
-  // layer 3
-  gemm<true, true>(dZ, D3, H2, D2, grad + OFF_W3, D3, D2, B, nullptr, 0, 0, 0.f, st);
-  k_colsum<<<1, D3, 0, st>>>(dZ, B, D3, grad + OFF_B3);
-  gemm<false, true>(dZ, D3, W + OFF_W3, D2, dH2, B, D2, D3, nullptr, 0, 1, 0.f, st);
-  k_relu_mask<<<64, 256, 0, st>>>(dH2, H2, B * D2);
-  // layer 2
-  gemm<true, true>(dH2, D2, H1, D1, grad + OFF_W2, D2, D1, B, nullptr, 0, 0, 0.f, st);
-  k_colsum<<<1, D2, 0, st>>>(dH2, B, D2, grad + OFF_B2);
-  gemm<false, true>(dH2, D2, W + OFF_W2, D1, dH1, B, D1, D2, nullptr, 0, 1, 0.f, st);
-  k_relu_mask<<<64, 256, 0, st>>>(dH1, H1, B * D1);
-  // layer 1
-  gemm<true, true>(dH1, D1, X, D0, grad + OFF_W1, D1, D0, B, nullptr, 0, 0, 0.f, st);
-  k_colsum<<<1, D1, 0, st>>>(dH1, B, D1, grad + OFF_B1);
+  float* lossp = dH1 + (size_t)B * D1;
+  const int blocks = (B + MR_ROWS - 1) / MR_ROWS;
+  k_mlp_rows<<<blocks, MR_BLOCK, sizeof(RowSmem), st>>>(W, X, Y, B, 1.f / (float)(B * D3), H1, H2, dZ, dH2, dH1, lossp);
+  k_mlp_grad<<<MG_T3 + MG_T2 + MG_T1, 256, 0, st>>>(X, H1, H2, dZ, dH2, dH1, B, lossp, blocks, grad, loss);
   return cudaGetLastError();
 }
 
