@@ -37,10 +37,12 @@ PAPER_MPTS = 40.0 / 0.8645
 # Kernels per hull_compute with the bucket sort, two-read front: extremes,
 # witnesses, fused filter (+ bin scan), placement into coarse bins, split
 # into bins, bin prefixes, sort (+ second round), compaction, finalisation;
-# the single-read front adds the sample polygon before its extremes pass.  A
+# on the single-read front, where the star path decides the hull: the sample
+# polygon, the pass over the input, the candidates' filter, the hull.  A
 # call rerun on the radix passes adds extremes, filter count + write, 8
 # radix passes, region scan + compact, finalisation.
 LAUNCHES_PER_HULL = 9
+LAUNCHES_SINGLE_READ = 4
 LAUNCHES_PER_RADIX_RERUN = 1 + 2 + 8 + 2 + 1
 
 
@@ -320,19 +322,23 @@ STAGE_KERNELS = {
     "regions": ("k4_compact", lambda n, s, r: 24.0 * r, "pairs"),
     "final": ("k5_final", lambda n, s, r: 12.0 * r, "pairs"),
 }
-# The single-read front (inputs of 65,536 points or more, aligned, no
-# statistics): the "polygon" stage is the sample polygon (every 1024th point
-# read, 8 B each); the "extremes" stage is the extremes pass that filters
-# with it (8 B per point read, the q raw survivors, 12 B each, written); the
-# witnesses come from the raw survivors' points (8 B each read); the fused
-# filter then reads those q raw survivors and writes the s pairs.  On the
-# two-read front the polygon stage is empty.
+# The single-read front (inputs of 65,536 points or more, no statistics): the
+# "polygon" stage is the frame and the sample polygon (counted as one point
+# in 1,024, 8 B each: the kernel reads one in 128); the "extremes" stage is
+# the pass that filters with it (8 B per point read, the q raw survivors, 12
+# B each, written); "final" is the star path's filter and hull of those (s
+# points reach the hull's block).  The stages between are empty unless the
+# star path hands the hull on to the bucket sort: then the witnesses come
+# from the raw survivors' points (8 B each read) and the fused filter reads
+# the q raw survivors and writes the s pairs.  On the two-read front the
+# polygon stage is empty.
 POLY_STRIDE = 1024
 SINGLE_STAGE_KERNELS = dict(STAGE_KERNELS)
 SINGLE_STAGE_KERNELS["polygon"] = ("k0_poly", lambda n, s, r, q: 8.0 * n / POLY_STRIDE, "points")
 SINGLE_STAGE_KERNELS["extremes"] = ("k1_poly", lambda n, s, r, q: 8.0 * n + 12.0 * q, "points")
 SINGLE_STAGE_KERNELS["witness"] = ("k_witness", lambda n, s, r, q: 8.0 * q, "raw")
 SINGLE_STAGE_KERNELS["filter"] = ("k2_fused", lambda n, s, r, q: 12.0 * q + 12.0 * s, "raw")
+SINGLE_STAGE_KERNELS["final"] = ("k_cand + k_star", lambda n, s, r, q: 12.0 * q + 12.0 * s, "raw")
 DOMINANT_CANDIDATES = ("polygon", "extremes", "witness", "filter", "scatter", "split", "sort")
 
 
@@ -353,7 +359,7 @@ def roofline_of(prof, hbm, peak_src):
     kernels = {}
     for name, (kern, nbytes, unit) in table.items():
         ms = stage_ms.get(name, 0.0)
-        b = nbytes(n, s, r, q) if single and name in ("polygon", "extremes", "witness", "filter") else nbytes(n, s, r)
+        b = nbytes(n, s, r, q) if single and name in ("polygon", "extremes", "witness", "filter", "final") else nbytes(n, s, r)
         units = n if unit == "points" else (q if unit == "raw" else s)
         kernels[name] = {"kernel": kern, "ms": ms, "algorithmic_bytes": b, "units": units,
                          "gbs": b / (ms / 1e3) / 1e9 if ms > 0 else None}
@@ -778,8 +784,8 @@ def main():
                        "survivors_per_hull": sum(first_round) / len(first_round),
                        "witness_survivors_per_hull": prof["witness_survivors"] / calls,
                        "second_round_per_hull": prof["second_round"] / calls},
-            "gpu_launches": prof["calls"] * LAUNCHES_PER_HULL + prof.get("single_read_calls", 0)
-            + prof["radix_calls"] * LAUNCHES_PER_RADIX_RERUN,
+            "gpu_launches": (prof["calls"] - prof.get("single_read_calls", 0)) * LAUNCHES_PER_HULL
+            + prof.get("single_read_calls", 0) * LAUNCHES_SINGLE_READ + prof["radix_calls"] * LAUNCHES_PER_RADIX_RERUN,
             "e2e": {"value": e2e_val, "unit": UNIT, "h2d_bytes_per_step": 8 * pts_step,
                     "d2h_bytes_per_step": 4 * sum(h_counts), "api": "hull_compute_host_multi"},
             "roofline": roofline}

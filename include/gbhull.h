@@ -63,7 +63,9 @@ typedef struct {
                          (on the two-read front and in batched mode; the single-read
                          front's sample polygon and witness test leave it nothing to gain) */
   int collect_stats;  /* 1 = keep survivor counts of the last call for hull_last_stats */
-  uint32_t spin_limit;/* iteration limit of every device wait; 0 = default (1 << 22) */
+  uint32_t spin_limit;/* iteration limit of the device waits between blocks and of the radix
+                         path's copies; 0 = default (1 << 22).  The single-read pass's copies
+                         into shared memory have a fixed limit (1 << 24) */
   int autotune;       /* 1 = time the batched kernels' block sizes per size bucket and the
                          boundary of the segmented path on first use and cache the choice
                          (file: $GBHULL_AUTOTUNE_CACHE, else ~/.cache/gbhull_autotune.json);
@@ -110,15 +112,21 @@ void hull_destroy(hull_ctx *ctx);
  * Section 2.1).  d_xy: device int32[n][2], read-only.  d_out: device
  * int32[cap] receiving the CCW vertex indices.  *h_count (host) receives the
  * hull size on HULL_OK and on HULL_ECAPACITY (then d_out is untouched).
- * Synchronises `stream` before returning.  n must be < 2^30.  Inputs of
- * 65,536 points or more, 16-byte aligned, in a context without
- * collect_stats take the single-read front (one pass over the input after a
- * sample polygon drops the points strictly inside a polygon spanned by
- * sampled input points); the others the two-read front (the extremes pass,
- * then the filter pass over the input).  The survivors are sorted by the
- * bucket sort (hull_stage_bucket_sort); an input it cannot handle in shared
- * memory is rerun on the radix passes (hull_stats.sort_fallback), with the
- * same result. */
+ * Synchronises `stream` before returning.  n must be < 2^30.
+ *
+ * In a context without collect_stats and reverse_round the star path comes
+ * first: an input below 65,536 points (unless the learned proposal is on) in
+ * one launch, a larger one through the single-read front (one pass over the
+ * input that drops the points strictly inside a polygon spanned by sampled
+ * input points) and the hull of the rest in angular order about an interior
+ * point, by sectors where many points lie next to the hull.  What it does
+ * not decide, and contexts with those switches, take the paper's steps: the
+ * two-read front (the extremes pass, then the filter pass over the input;
+ * the raw survivors instead where the single-read front left them), the
+ * bucket sort (hull_stage_bucket_sort), the second round and the chains; an
+ * input that the bucket sort cannot handle in shared memory is rerun on the
+ * radix passes (hull_stats.sort_fallback).  The result is the same on every
+ * path. */
 hull_status hull_compute(hull_ctx *ctx, const int32_t *d_xy, int64_t n, int32_t *d_out,
                          int64_t cap, int64_t *h_count, void *stream);
 
@@ -177,7 +185,11 @@ hull_status hull_compute_host_multi(hull_ctx *ctx, int32_t count, const int32_t 
  * leaves d_out untouched but still writes d_out_offsets).  Total points must
  * be < 2^30 and every instance at most hull_batched_max_instance() points
  * (else HULL_EINVAL).  Copies d_offsets to the host and synchronises
- * `stream`. */
+ * `stream`. *
+ * The star path (see hull_compute) takes every instance first: one block per
+ * instance of at most 16,384 points, the larger ones through one flat pass
+ * over all their points.  The two ways above are for the instances that it
+ * does not decide, and what autotune times. */
 hull_status hull_compute_batched(hull_ctx *ctx, const int32_t *d_xy, const int64_t *d_offsets,
                                  int32_t B, int32_t *d_out, int64_t cap, int64_t *d_out_offsets,
                                  void *stream);
@@ -241,8 +253,9 @@ typedef struct {
   int64_t second_round;          /* second-round survivors, summed */
   double ms[HULL_NUM_STAGES];    /* per stage; with the bucket sort (the default): polygon
                                     (single-read front: the sample polygon; empty on the
-                                    two-read front), extremes (single-read front: the extremes
-                                    pass that filters with the polygon), witnesses (the
+                                    two-read front), extremes (single-read front: the
+                                    pass that filters with the polygon; the star path's hull
+                                    is then in `final`, the slots between empty), witnesses (the
                                     sample's best witness per bin), filter (the
                                     fused filter: witness test, filter polygon, compaction, bin
                                     scan), scatter (survivors into coarse bins), split (coarse bins
@@ -250,11 +263,12 @@ typedef struct {
                                     sorted, second round), 3 empty slots, regions (compaction),
                                     final; on the radix passes: extremes, filter, radix pass 0..7,
                                     regions, final */
-  int64_t witness_survivors;     /* survivors of the fused filter (the bucket sort's input),
+  int64_t witness_survivors;     /* survivors of the fused filter (the bucket sort's input), on
+                                    the star path the points that its last block sorts,
                                     summed; the first-round survivors on the radix passes */
   int64_t raw_survivors;         /* single-read front: points on or outside the sample polygon
-                                    (the fused filter's input), summed; 0 for calls on the
-                                    two-read front */
+                                    (the star path's or the fused filter's input), summed; 0 for
+                                    calls on the two-read front and small inputs */
   int64_t single_read_calls;     /* calls that took the single-read front */
 } hull_profile;
 

@@ -552,7 +552,7 @@ enum From { FROM_STAR = 0, FROM_FRONT, FROM_SECTORS, FROM_RAW, FROM_BUCKET, FROM
 
 // The step after an attempt of the star path with summary p that did not decide.
 From after_star(const Plan& p, u32 n, bool raw) {
-  const bool many = p.s_raw > kStarCap && (p.s == 0 || p.s > kStarCap);
+  const bool many = p.s > kStarCap || (p.s == 0 && p.s_raw > kStarCap);
   if (many && p.s_raw <= sector_max_points()) return single_read(n) && raw ? FROM_SECTORS : FROM_FRONT;
   return single_read(n) && raw ? FROM_RAW : FROM_BUCKET;
 }
@@ -774,8 +774,7 @@ hull_status hull_create(hull_ctx** out, int device, const hull_config* cfg) {
         cudaMalloc(&c->adam_m, np * 4) != cudaSuccess || cudaMalloc(&c->adam_v, np * 4) != cudaSuccess ||
         cudaMalloc(&c->grad, (np + 4) * 4) != cudaSuccess || cudaMalloc(&c->feat, 64 * 4) != cudaSuccess ||
         cudaMalloc(&c->ext, 32 * 4) != cudaSuccess || cudaMalloc(&c->ext_xy, 64 * 4) != cudaSuccess ||
-        cudaMalloc(&c->lab_cnt, 33 * 8) != cudaSuccess || cudaMallocHost(&c->h_grad, (np + 1) * 4) != cudaSuccess ||
-        mlp_configure() != cudaSuccess) {
+        cudaMalloc(&c->lab_cnt, 33 * 8) != cudaSuccess) {
       cudaGetLastError();
       *out = c;
       hull_destroy(c);
@@ -1631,6 +1630,7 @@ hull_status hull_learned_labels(hull_ctx* c, const int32_t* d_xy, int64_t n, flo
 
 static hull_status ensure_train(hull_ctx* c, int B) {
   if ((size_t)B <= c->train_cap) return HULL_OK;
+  if (mlp_configure() != cudaSuccess) return cuda_fail(cudaErrorUnknown);
   if (c->act) cudaFree(c->act);
   if (c->scratch) cudaFree(c->scratch);
   c->act = nullptr; c->scratch = nullptr; c->train_cap = 0;
@@ -1665,6 +1665,11 @@ hull_status hull_mlp_gradient(hull_ctx* c, const float* d_X, const float* d_Y, i
   hull_status r = ensure_train(c, B);
   if (r != HULL_OK) return r;
   const size_t np = (size_t)mlp_num_params();
+  if (!c->h_grad && cudaMallocHost(&c->h_grad, (np + 1) * 4) != cudaSuccess) {
+    c->h_grad = nullptr;
+    cudaGetLastError();
+    return HULL_ENOMEM;
+  }
   cudaError_t e = mlp_gradient(c->W, d_X, d_Y, B, c->act, c->grad, c->d_loss, c->scratch, st);
   // Gradient and loss (behind it) in one copy to pinned memory: a pageable
   // destination would be staged by the driver, twice.

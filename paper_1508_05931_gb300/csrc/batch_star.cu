@@ -28,7 +28,11 @@ struct BRec {
   u32 raw_count, pad;
   u64 key[BF_NB];
   u32 tab[BF_SLABS];
+  float2 nrm[BF_NB];
 };
+
+// More raw survivors than this: not for one block.
+__device__ __forceinline__ u32 many(u32 n) { return max(16384u, n / 4u); }
 
 // ---- small instances
 constexpr int BS_BLOCK = 256;
@@ -85,7 +89,7 @@ kb_small(BatchStar a) {
     }
     StarFrame F;
     u32 m0 = n;
-    bool bad = false;
+    bool bad = false, dirs = false;
     if (n <= BS_DIRECT) {
       static_assert(BS_DIRECT <= BS_SAMPLES * BS_BLOCK, "the points in registers");
       int2 p[BS_SAMPLES];
@@ -121,6 +125,8 @@ kb_small(BatchStar a) {
       }
       __syncthreads();
       const PolyHead H = star::build_poly<BS_BLOCK>(S.poly, F, S.tab, BS_SLABS);
+      dirs = H.ok != 0;
+      if (dirs) star::bin_normals<BS_BLOCK, BF_NB>(S.poly, F, S.list.dirs());
       __syncthreads();
       star::ListSink<decltype(S.list)> sink{&S.list, &S.count, (u32)BF_CAP, false};
       star::stream_points<4>(P, n, 0u, (u32)wid, (u32)(BS_BLOCK / 32), H, S.tab, sink, [] {});
@@ -133,7 +139,7 @@ kb_small(BatchStar a) {
     const bool err = S.bad != 0u;
     int h = -1;
     if (m0 <= (u32)BF_CAP && !err) {
-      const u32 m = star::filter_list<BS_BLOCK, BF_CAP, BF_NB>(S.list, m0, F, S.key, S.cands);
+      const u32 m = star::filter_list<BS_BLOCK, BF_CAP, BF_NB>(S.list, m0, F, S.key, S.cands, dirs ? S.list.dirs() : nullptr);
       h = star::list_hull<BS_BLOCK, BF_CAP, BF_NB>(S.list, m, F, out, n);
       if (h < 0) h = star::rest_hull<BS_BLOCK>(S.list, P, n, out, n);
     }
@@ -196,6 +202,7 @@ kb_poly(BatchStar a) {
   }
   __syncthreads();
   const PolyHead H = star::build_poly<BP_BLOCK>(S.poly, F, R.tab, BF_SLABS);
+  if (H.ok) star::bin_normals<BP_BLOCK, BF_NB>(S.poly, F, R.nrm);
   if (t == 0) { R.frame = F; R.head = H; }
 }
 
@@ -244,8 +251,8 @@ kb_stream(BatchStar a) {
     BRec& R = reinterpret_cast<BRec*>(a.rec)[lo];
     const u32 p0 = (u32)(t - tf) * BF_TILE, p1 = min(n, (u32)(te - tf) * BF_TILE);
     PolyHead H;
-    star::RawSink<BF_NB, BT_SLICE> sink{S.sxy[wid], S.sidx[wid], 0u, &R.frame, &R.raw_count, a.error, R.key,
-                                        reinterpret_cast<int2*>(a.kb + sl), a.ib + sl, n};
+    star::RawSink<BF_NB, BT_SLICE> sink{S.sxy[wid], S.sidx[wid], 0u, &R.frame, &R.raw_count, a.error, R.key, R.nrm,
+                                        reinterpret_cast<int2*>(a.kb + sl), a.ib + sl, n, many(n)};
     star::stream_ring(ring, reinterpret_cast<const int2*>(a.xy) + off + p0, p1 - p0, p0, (u32)wid, (u32)BT_WARPS, H,
                       S.tab, sink, a.error, [&] {
       H = R.head;
@@ -281,7 +288,7 @@ kb_finish(BatchStar a) {
   const u32* ridx = a.ib + sl;
   const u32 q = min(R.raw_count, n);
   // Most points next to the hull: not for one block.
-  if ((q > 16384u && q > n / 4u) || q == 0u) {
+  if (q > many(n) || q == 0u) {
     if (t == 0) put_result(a, inst, -1, false);
     return;
   }

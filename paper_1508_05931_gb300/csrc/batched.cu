@@ -1,4 +1,5 @@
-// Batched hulls: many independent point sets in one call.
+// Batched hulls: many independent point sets in one call.  The general path,
+// for the instances that the star path (batch_star.cu) does not decide.
 //
 // k_batch, mode 0: every block takes instances from a queue ordered largest
 // first (so the longest jobs start early and the small ones fill the tail)

@@ -133,8 +133,12 @@ struct PolyTab {
   StarFrame frame;
   PolyHead head;
   u32 tab[kPolySlabs];
+  float2 nrm[kStarBins];  // directions of the bins' candidates
 };
 constexpr size_t kPolyClearBytes = offsetof(PolyTab, frame);
+// More raw survivors of n points than this: most points lie next to the hull,
+// the candidates cannot bring them below kStarCap.
+__host__ __device__ inline u32 many_raw(u32 n) { return n / 4u > (1u << 18) ? n / 4u : 1u << 18; }
 
 struct Plan {
   // summary fields first: the host copies back everything before `ctr`

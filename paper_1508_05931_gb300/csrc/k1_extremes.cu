@@ -311,7 +311,7 @@ k1_extremes(const int* __restrict__ xy, u32 n, u32 spin_limit, Plan* plan,
 // shared-memory passes per warp).  Every warp streams its own ring of bulk
 // copies, tests eight points a lane and votes once; survivors are well below
 // one in a hundred of ordinary inputs.  20M square / disk, launch included:
-// 34 / 36 us with one block of 16 warps and rings of 4 x 256 points; 41 with
+// 34 / 36 us with one block of 16 warps and rings of 256-point chunks; 41 with
 // two blocks on register double buffers; 37 with 32 warps, 38 / 41 with two
 // blocks of smaller rings; 43 for the eight-byte table with a scan per round.  An input that starts on an odd row
 // (8-byte aligned) gives its first point to one lane and streams the rest.
@@ -319,7 +319,7 @@ constexpr int K1P_BLOCK = 512;
 constexpr int K1P_WARPS = K1P_BLOCK / 32;
 constexpr int K1P_SLICE = 256;                 // staged points per warp
 constexpr int K1P_CH = 256;                    // points per chunk
-constexpr int K1P_STAGES = 4;                  // chunks in flight per warp
+constexpr int K1P_STAGES = 3;                  // chunks in flight per warp (a fourth gains nothing and keeps k_cand out)
 
 struct K1PSmem {
   int4 ring[K1P_WARPS][K1P_STAGES][K1P_CH / 2];
@@ -336,7 +336,7 @@ k1_poly(const int2* __restrict__ P, u32 n, PolyTab* __restrict__ T, int2* __rest
   const int wid = threadIdx.x >> 5;
   PolyHead H;
   star::RawSink<kStarBins, K1P_SLICE> sink{S.sxy[wid], S.sidx[wid], 0u, &T->frame, &T->raw_count, &T->error, T->key,
-                                           rxy, ridx, n};
+                                           T->nrm, rxy, ridx, n, many_raw(n)};
   star::Ring<K1P_STAGES, K1P_CH> ring{&S.ring[wid][0][0], S.bar[wid], 0u, true};
   ring.init();
   // Consecutive chunks go to consecutive blocks.
@@ -401,12 +401,20 @@ cudaError_t launch_k1(const int* xy, u32 n, u32 spin_limit, Plan* plan, ExtParti
 
 
 cudaError_t k1_poly_configure() {
-  return cudaFuncSetAttribute(k1_poly, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(K1PSmem));
+  // The whole of an SM's L1 as shared memory: the split is fixed as long as a
+  // block is resident, and another lane's K0 only fits beside this kernel if
+  // it is (20M square + disk 161 -> 147 us).
+  const cudaError_t e = cudaFuncSetAttribute(k1_poly, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                             cudaSharedmemCarveoutMaxShared);
+  return e == cudaSuccess
+             ? cudaFuncSetAttribute(k1_poly, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(K1PSmem))
+             : e;
 }
 
 cudaError_t launch_k1_poly(const int* xy, u32 n, PolyTab* T, int2* rxy, u32* ridx, int num_sms, cudaStream_t st) {
+  const u32 most = num_sms > 4 ? (u32)num_sms - 2u : (u32)num_sms;    // two SMs for another lane's k_star
   const u32 blocks = (n + K1P_WARPS * K1P_CH - 1) / (K1P_WARPS * K1P_CH);
-  const u32 grid = blocks < 1u ? 1u : (blocks < (u32)num_sms ? blocks : (u32)num_sms);
+  const u32 grid = blocks < 1u ? 1u : (blocks < most ? blocks : most);
   return launch_after(k1_poly, dim3(grid), dim3(K1P_BLOCK), sizeof(K1PSmem), st, reinterpret_cast<const int2*>(xy), n,
                       T, rxy, ridx);
 }

@@ -1,11 +1,13 @@
 // The star path's finishing kernels (star.cuh): the hull of the single-read
 // front's raw survivors, and the whole hull of a small input in one launch.
 //
-// k_star   all blocks test K1's raw survivors against the polygon of the
-//          angular candidates (about 129k of 20M uniform points come in,
-//          a few thousand at most go on) and append the rest to a list; the
-//          last block to finish sorts the list by angle and finds the hull
-//          in shared memory.
+// k_cand   tests K1's raw survivors against the polygon of the angular
+//          candidates (about 60k of 20M points of a disk come in, 3k go on)
+//          and appends the rest to a list;
+// k_star   one block sorts the list by angle and finds the hull in shared
+//          memory.  It is a kernel of its own, not k_cand's last block, so
+//          that k_cand's blocks need little shared memory and fit beside
+//          another lane's K1, which leaves two SMs free for this one.
 // k_small  one block: frame, sample polygon, one pass over the points, then
 //          the same on the points left.
 //
@@ -24,10 +26,6 @@ namespace {
 
 constexpr int KS_BLOCK = 1024;
 constexpr int KS_CAP = (int)kStarCap;
-// More raw survivors than this and more than a quarter of the input: the
-// candidates cannot bring them below kStarCap (most points lie next to the
-// hull), so the blocks leave at once.
-constexpr u32 KS_RAW_MAX = 1u << 18;
 // Up to this many points k_small takes them all into its list: the sample
 // polygon would cost more than it saves.
 constexpr u32 KS_DIRECT = 4096;
@@ -36,14 +34,6 @@ constexpr int KS_SAMPLES = 4;         // samples per thread of k_small's polygon
 
 typedef star::ListSmem<KS_BLOCK, KS_CAP, kStarBins> List;
 typedef star::CandTab<kStarBins> Cands;
-
-struct StarSmem {
-  union {
-    List list;
-    Cands cands;
-  };
-  bool last;
-};
 
 struct SmallSmem {
   List list;
@@ -60,75 +50,93 @@ struct SmallSmem {
   u32 count, error;
 };
 
-__global__ void __launch_bounds__(KS_BLOCK)
-k_star(const int2* __restrict__ P, u32 n, PolyTab* T, const int2* __restrict__ rxy, const u32* __restrict__ ridx,
-       int2* lxy, u32* lidx, Plan* plan, int* out, long long cap) {
-  extern __shared__ __align__(16) unsigned char ks_smem[];
-  StarSmem& S = *reinterpret_cast<StarSmem*>(ks_smem);
+// No polygon: a degenerate input (1); too many raw survivors for one block
+// (2): the star path leaves both to others.
+__device__ __forceinline__ int not_here(const PolyTab* T, u32 q, u32 n) {
+  return !T->head.ok ? 1 : q > many_raw(n) ? 2 : 0;
+}
+
+constexpr int KC_BLOCK = 512;
+
+__global__ void __launch_bounds__(KC_BLOCK)
+k_cand(const int2* __restrict__ P, u32 n, PolyTab* T, const int2* __restrict__ rxy, const u32* __restrict__ ridx,
+       int2* lxy, u32* lidx) {
+  __shared__ Cands S;
   const int lane = threadIdx.x & 31, t = threadIdx.x;
+  if (t < kStarBins / 32) S.occ[t] = 0u;
   pdl_wait();
+  // Everything that hangs on nothing else is under way at once: the keys, the
+  // head and this thread's first survivor (its slot exists, whatever it holds).
+  constexpr int PER = kStarBins / KC_BLOCK;
+  u64 k[PER];
+  int2 p[PER];
+  #pragma unroll
+  for (int j = 0; j < PER; ++j) k[j] = __ldcg(&T->key[t + j * KC_BLOCK]);
+  u32 i = blockIdx.x * (u32)KC_BLOCK + t;
+  int2 w = i < n ? rxy[i] : make_int2(0, 0);
+  u32 id = i < n ? ridx[i] : 0u;
   const u32 q = min(T->raw_count, n);
   const StarFrame F = T->frame;
-  // No polygon: a degenerate input, not for the star path (s = 1 says so).
-  const bool flat = !T->head.ok;
-  if (flat || (q > KS_RAW_MAX && q > n / 4)) {
-    if (blockIdx.x == 0 && t == 0) star_summary(plan, n, q, flat ? 1u : 0u, -1, cap, T->error);
+  if (not_here(T, q, n) || blockIdx.x * (u32)KC_BLOCK >= q) return;
+  __syncthreads();
+  #pragma unroll
+  for (int j = 0; j < PER; ++j) p[j] = k[j] ? P[min(~(u32)k[j], n - 1u)] : make_int2(0, 0);
+  #pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    const int b = t + j * KC_BLOCK;
+    if (k[j]) {
+      S.cand[b] = p[j];
+      S.cid[b] = ~(u32)k[j];
+      atomicOr(&S.occ[b >> 5], 1u << (b & 31));
+    }
+  }
+  __syncthreads();
+  const u32 step = gridDim.x * (u32)KC_BLOCK;
+  for (u32 i0 = blockIdx.x * (u32)KC_BLOCK; i0 < q; i0 += step, i += step) {
+    const int2 w1 = i + step < q ? rxy[i + step] : make_int2(0, 0);
+    const u32 id1 = i + step < q ? ridx[i + step] : 0u;
+    bool keep = false;
+    if (i < q) {
+      float u, v;
+      star::to_uv(F, w.x - F.cx, w.y - F.cy, u, v);
+      keep = !star::dropped_by_cands<kStarBins>(S, F, star::bin_of<kStarBins>(u, v), w.x, w.y, id);
+    }
+    const u32 bal = __ballot_sync(0xFFFFFFFFu, keep);
+    u32 base = 0;
+    if (lane == 0 && bal) base = atomicAdd(&T->list_count, (u32)__popc(bal));
+    base = __shfl_sync(0xFFFFFFFFu, base, 0) + __popc(bal & ((1u << lane) - 1u));
+    if (keep && base < kStarCap) { lxy[base] = w; lidx[base] = id; }
+    w = w1;
+    id = id1;
+  }
+}
+
+__global__ void __launch_bounds__(KS_BLOCK)
+k_star(u32 n, PolyTab* T, const int2* __restrict__ lxy, const u32* __restrict__ lidx, Plan* plan, int* out,
+       long long cap) {
+  extern __shared__ __align__(16) unsigned char ks_smem[];
+  List& S = *reinterpret_cast<List*>(ks_smem);
+  const int t = threadIdx.x;
+  pdl_wait();
+  const int2 p0 = lxy[t];             // the first entries with the sizes (the slots exist)
+  const u32 id0 = lidx[t];
+  const u32 q = min(T->raw_count, n), err = T->error;
+  const int why = not_here(T, q, n);
+  if (why) {                          // s = 1 tells the degenerate case from too many points
+    if (t == 0) star_summary(plan, n, q, why == 1 ? 1u : 0u, -1, cap, err);
     return;
   }
-  if (blockIdx.x * (u32)KS_BLOCK < q) {
-    if (t < kStarBins / 32) S.cands.occ[t] = 0u;
-    __syncthreads();
-    constexpr int PER = kStarBins / KS_BLOCK;
-    u64 k[PER];
-    #pragma unroll
-    for (int j = 0; j < PER; ++j) k[j] = __ldcg(&T->key[t + j * KS_BLOCK]);
-    #pragma unroll
-    for (int j = 0; j < PER; ++j) {
-      const int b = t + j * KS_BLOCK;
-      if (k[j]) {
-        const u32 id = min(~(u32)k[j], n - 1u);
-        S.cands.cand[b] = P[id];
-        S.cands.cid[b] = id;
-        atomicOr(&S.cands.occ[b >> 5], 1u << (b & 31));
-      }
-    }
-    __syncthreads();
-    for (u32 i0 = blockIdx.x * (u32)KS_BLOCK; i0 < q; i0 += gridDim.x * (u32)KS_BLOCK) {
-      const u32 i = i0 + t;
-      bool keep = false;
-      int2 p = make_int2(0, 0);
-      u32 id = 0;
-      if (i < q) {
-        p = rxy[i];
-        id = ridx[i];
-        float u, v;
-        star::to_uv(F, p.x - F.cx, p.y - F.cy, u, v);
-        keep = !star::dropped_by_cands<kStarBins>(S.cands, F, star::bin_of<kStarBins>(u, v), p.x, p.y, id);
-      }
-      const u32 bal = __ballot_sync(0xFFFFFFFFu, keep);
-      u32 base = 0;
-      if (lane == 0 && bal) base = atomicAdd(&T->list_count, (u32)__popc(bal));
-      base = __shfl_sync(0xFFFFFFFFu, base, 0) + __popc(bal & ((1u << lane) - 1u));
-      if (keep && base < kStarCap) { lxy[base] = p; lidx[base] = id; }
-    }
-  }
-  __threadfence();
-  __syncthreads();
-  if (t == 0) S.last = atomicAdd(&T->done2, 1u) == gridDim.x - 1;
-  __syncthreads();
-  if (!S.last) return;
-  __threadfence();
-  const u32 m = *(volatile u32*)&T->list_count;
+  const u32 m = T->list_count;
   int h = -1;
-  const u32 err = T->error;
   if (m <= kStarCap && !(err & ERR_RANGE)) {
     for (u32 i = t; i < m; i += KS_BLOCK) {
-      S.list.p[i] = __ldcg(&lxy[i]);
-      S.list.id[i] = __ldcg(&lidx[i]);
-      S.list.ta[i] = (unsigned short)i;
+      S.p[i] = i < (u32)KS_BLOCK ? p0 : lxy[i];
+      S.id[i] = i < (u32)KS_BLOCK ? id0 : lidx[i];
+      S.ta[i] = (unsigned short)i;
     }
+    const StarFrame F = T->frame;
     __syncthreads();
-    h = star::list_hull<KS_BLOCK, KS_CAP, kStarBins>(S.list, m, F, out, cap);
+    h = star::list_hull<KS_BLOCK, KS_CAP, kStarBins>(S, m, F, out, cap);
   }
   if (t == 0) star_summary(plan, n, q, m, h, cap, err);
   // Decided: the table is left clear for the next call.
@@ -148,7 +156,7 @@ k_small(const int2* __restrict__ P, u32 n, Plan* plan, int* out, long long cap) 
   if (t < kPolyDirs) S.best[t] = 0ull;
   StarFrame F;
   u32 m0 = n;
-  bool bad = false, flat = false;
+  bool bad = false, flat = false, dirs = false;
   if (n <= KS_DIRECT) {
     static_assert(KS_DIRECT <= KS_SAMPLES * KS_BLOCK, "the points in registers");
     int2 p[KS_SAMPLES];
@@ -184,6 +192,8 @@ k_small(const int2* __restrict__ P, u32 n, Plan* plan, int* out, long long cap) 
     }
     __syncthreads();
     const PolyHead H = star::build_poly<KS_BLOCK>(S.poly, F, S.tab, KS_SLABS);
+    dirs = H.ok != 0;
+    if (dirs) star::bin_normals<KS_BLOCK, kStarBins>(S.poly, F, S.list.dirs());
     __syncthreads();
     star::ListSink<decltype(S.list)> sink{&S.list, &S.count, (u32)KS_CAP, false};
     star::stream_points<4>(P, n, 0u, (u32)wid, (u32)(KS_BLOCK / 32), H, S.tab, sink, [] {});
@@ -198,20 +208,20 @@ k_small(const int2* __restrict__ P, u32 n, Plan* plan, int* out, long long cap) 
   int h = -1;
   u32 m = m0;
   if (m0 <= (u32)KS_CAP && !err) {
-    m = star::filter_list<KS_BLOCK, KS_CAP, kStarBins>(S.list, m0, F, S.key, S.cands);
+    m = star::filter_list<KS_BLOCK, KS_CAP, kStarBins>(S.list, m0, F, S.key, S.cands, dirs ? S.list.dirs() : nullptr);
     h = star::list_hull<KS_BLOCK, KS_CAP, kStarBins>(S.list, m, F, out, cap);
   }
   if (h < 0 && !err && (flat || m0 <= (u32)KS_CAP)) {
     h = star::rest_hull<KS_BLOCK>(S.list, P, n, out, cap);
-    m = m0 = 0u;                      // not undecided for being too many
+    m = 0u;                           // not undecided for being too many
   }
-  if (t == 0) star_summary(plan, n, m0, m, h, cap, err);
+  if (t == 0) star_summary(plan, n, 0, m, h, cap, err);
 }
 
 }  // namespace
 
 cudaError_t star_configure() {
-  cudaError_t e = cudaFuncSetAttribute(k_star, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(StarSmem));
+  cudaError_t e = cudaFuncSetAttribute(k_star, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(List));
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmallSmem));
   return e;
@@ -219,10 +229,13 @@ cudaError_t star_configure() {
 
 cudaError_t launch_star(const int* xy, u32 n, PolyTab* T, const int2* rxy, const u32* ridx, int2* lxy, u32* lidx,
                         Plan* plan, int* out, long long cap, int num_sms, cudaStream_t st) {
-  const u32 want = n / (32u * KS_BLOCK) + 1u;      // a block per 32,768 input points
-  const u32 grid = want < (u32)num_sms ? want : (u32)num_sms;
-  return launch_after(k_star, dim3(grid), dim3(KS_BLOCK), sizeof(StarSmem), st, reinterpret_cast<const int2*>(xy), n, T,
-                      rxy, ridx, lxy, lidx, plan, out, cap);
+  // A block per 32,768 input points, half the SMs at most: every block
+  // gathers all candidates, and two points a thread hide that as well.
+  const u32 want = n / (64u * KC_BLOCK) + 1u, most = ((u32)num_sms + 1u) / 2u;
+  const cudaError_t e = launch_after(k_cand, dim3(want < most ? want : most), dim3(KC_BLOCK), 0, st,
+                                     reinterpret_cast<const int2*>(xy), n, T, rxy, ridx, lxy, lidx);
+  if (e != cudaSuccess) return e;
+  return launch_after(k_star, dim3(1), dim3(KS_BLOCK), sizeof(List), st, n, T, lxy, lidx, plan, out, cap);
 }
 
 cudaError_t launch_small(const int* xy, u32 n, Plan* plan, int* out, long long cap, cudaStream_t st) {

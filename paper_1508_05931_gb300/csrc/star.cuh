@@ -43,10 +43,15 @@ __device__ __forceinline__ u32 bin_of(float u, float v) {
   return (u32)min(max(b, 0), NB - 1);
 }
 
-// Candidate key of a point: the whitened radius, then the smaller index (all
-// duplicates of a point share its bin and radius).
-__device__ __forceinline__ u64 cand_key(float u, float v, u32 idx) {
-  return ((u64)__float_as_uint(__fmaf_rn(u, u, __fmul_rn(v, v))) << 32) | (u64)(~idx);
+// Candidate key of a point: how far it reaches along the bin's direction w,
+// then the smaller index (all duplicates of a point share its bin and reach).
+// Without a polygon w is the point itself (its radius); with one, the outward
+// normal of the polygon's edge that the bin looks at: along a flat side the
+// largest radius is at the bin's far end, not nearest the side (a 20M square
+// left 5,600 points of 17k that way).
+__device__ __forceinline__ u64 cand_key(float2 w, float u, float v, u32 idx) {
+  const float r = fmaxf(__fmaf_rn(w.x, u, __fmul_rn(w.y, v)), 0.0f);
+  return ((u64)__float_as_uint(r) << 32) | (u64)(~idx);
 }
 
 __device__ __forceinline__ bool out_of_range(int x, int y) {
@@ -156,7 +161,7 @@ __device__ __forceinline__ size_t sample_at(u32 i, u32 stride4) { return (size_t
 __device__ __forceinline__ void offer_sample(const StarFrame& F, int2 p, u32 pos, u64* best) {
   float u, v;
   to_uv(F, p.x - F.cx, p.y - F.cy, u, v);
-  const u64 k = cand_key(u, v, pos);
+  const u64 k = cand_key(make_float2(u, v), u, v, pos);
   u64* slot = &best[bin_of<kPolyDirs>(u, v)];
   if (k > *(volatile u64*)slot) atomicMax(slot, k);
 }
@@ -167,6 +172,7 @@ struct PolySmem {
   int hx[kPolyDirs + 2], hy[kPolyDirs + 2];
   float slope[kPolyDirs + 2];
   int k, ir, ymin, ymax;
+  u64 alive;                            // sectors of the polygon's corners
 };
 
 // The polygon of the candidates (in angular order about c) and the table of
@@ -189,7 +195,11 @@ struct PolySmem {
 // and ceil(p - e) of the upper one are strictly inside.  For small
 // coordinates that is the exact test.  The heights are stored in 16 bits, in
 // units of 2^shy rounded inwards.
-template <int BLOCK>
+// PAD: word s goes to tab[s + s / 32] (a thread's run of slabs then spreads
+// over the shared-memory banks).
+__device__ __forceinline__ u32 pad_slab(u32 s) { return s + (s >> 5); }
+
+template <int BLOCK, bool PAD = false>
 __device__ PolyHead build_poly(PolySmem& S, const StarFrame& F, u32* tab, u32 slabs) {
   static_assert(kPolyDirs == 64, "two candidates per lane of a warp, one mask word");
   const int lane = threadIdx.x & 31, t = threadIdx.x;
@@ -277,7 +287,7 @@ __device__ PolyHead build_poly(PolySmem& S, const StarFrame& F, u32* tab, u32 sl
       }
       if (lane == 0) { S.ir = r1 >= r0 ? r1 - r0 : r1 - r0 + k; S.ymin = ylo; S.ymax = yhi; S.hx[k] = S.hx[0]; }
     }
-    if (lane == 0) S.k = k;
+    if (lane == 0) { S.k = k; S.alive = alive; }
   }
   __syncthreads();
   const int k = S.k;
@@ -331,11 +341,42 @@ __device__ PolyHead build_poly(PolySmem& S, const StarFrame& F, u32* tab, u32 sl
       const u32 A = ((u32)(ylo - ymin) >> H.shy) + 1u, B = (u32)(yhi - ymin) >> H.shy;
       if (B > A) w = A | ((B - A) << 16);
     }
-    tab[s] = w;
+    tab[PAD ? pad_slab(s) : s] = w;
     if (!H.sh && s + 1 < s1) heights(column(s + 1), lo1, hi1);
     lo0 = lo1; hi0 = hi1;
   }
   return H;
+}
+
+// The directions of the bins' candidates (cand_key): the outward normals, in
+// the whitened plane, of the edges that the bins' middles look at.  After a
+// build_poly that gave a polygon, the whole block.
+template <int BLOCK, int NB>
+__device__ __forceinline__ void bin_normals(const PolySmem& S, const StarFrame& F, float2* nrm) {
+  const u64 alive = S.alive;
+  auto before = [&](int j) {            // the last corner's sector below j, cyclically
+    const u64 m = alive & ((1ull << j) - 1ull);
+    return 63 - __clzll((long long)(m ? m : alive));
+  };
+  for (int b = threadIdx.x; b < NB; b += BLOCK) {
+    const int j = b / (NB / kPolyDirs);
+    int ja = j;
+    if ((alive >> j) & 1ull) {
+      const int2 p = S.p[j];
+      float u, v;
+      to_uv(F, p.x - F.cx, p.y - F.cy, u, v);
+      if ((int)bin_of<NB>(u, v) > b) ja = before(j);
+    } else {
+      ja = before(j);
+    }
+    const u64 above = ja < 63 ? alive >> (ja + 1) << (ja + 1) : 0ull;
+    const int jb = __ffsll((long long)(above ? above : alive)) - 1;
+    const int2 A = S.p[ja], B = S.p[jb];
+    float ua, va, ub, vb;
+    to_uv(F, A.x - F.cx, A.y - F.cy, ua, va);
+    to_uv(F, B.x - F.cx, B.y - F.cy, ub, vb);
+    nrm[b] = make_float2(vb - va, ua - ub);
+  }
 }
 
 // Strictly inside the sample polygon (its table): word w holds the first
@@ -361,9 +402,11 @@ struct RawSink {
   u32* raw_count;
   u32* error;
   u64* key;
+  const float2* nrm;
   int2* rxy;
   u32* ridx;
   u32 bound;                // capacity of (rxy, ridx)
+  u32 many;                 // past this many raw survivors nobody reads the candidates
 
   __device__ __forceinline__ void flush() {
     const int lane = threadIdx.x & 31;
@@ -377,11 +420,12 @@ struct RawSink {
       const u32 id = sidx[q];
       if (base + q < bound) { rxy[base + q] = p; ridx[base + q] = id; }
       if (out_of_range(p.x, p.y)) atomicOr(error, ERR_RANGE);
+      if (base > many) continue;
       float u, v;
       to_uv(F, p.x - F.cx, p.y - F.cy, u, v);
-      const u64 k = cand_key(u, v, id);
-      u64* slot = &key[bin_of<NB>(u, v)];
-      if (k > __ldcg(slot)) atomicMax(slot, k);
+      const u32 b = bin_of<NB>(u, v);
+      const u64 k = cand_key(__ldcg(&nrm[b]), u, v, id);
+      if (k > __ldcg(&key[b])) atomicMax(&key[b], k);
     }
     __syncwarp();
     fill = 0;
@@ -666,10 +710,13 @@ struct ListSmem {
   u32 id[CAP];
   unsigned short bn[CAP];
   unsigned short ta[CAP], tb[CAP];
-  u32 cnt[NB], cur[NB];
+  __align__(8) u32 cnt[NB];
+  u32 cur[NB];
   u32 ws[2][BLOCK / 32];
   u64 first;
   u32 flag;
+  // The bins' directions for filter_list, in the place of the counts that list_hull needs later.
+  __device__ float2* dirs() { return reinterpret_cast<float2*>(cnt); }
 };
 
 // The rank of entry i of the bin's entries at[s, e) (positions in p) in the
@@ -870,9 +917,10 @@ __device__ int list_hull(ListSmem<BLOCK, CAP, NB>& S, u32 m, const StarFrame& F,
 
 // The candidates of the list S.p[0, m0) and the points that they do not
 // drop: their positions to S.ta, their number returned (the whole block;
-// key: NB words of scratch).
+// key: NB words of scratch; nrm: the bins' directions, null without a polygon).
 template <int BLOCK, int CAP, int NB>
-__device__ u32 filter_list(ListSmem<BLOCK, CAP, NB>& S, u32 m0, const StarFrame& F, u64* key, CandTab<NB>& C) {
+__device__ u32 filter_list(ListSmem<BLOCK, CAP, NB>& S, u32 m0, const StarFrame& F, u64* key, CandTab<NB>& C,
+                           const float2* nrm) {
   const int t = threadIdx.x;
   for (int b = t; b < NB; b += BLOCK) key[b] = 0ull;
   for (int b = t; b < NB / 32; b += BLOCK) C.occ[b] = 0u;
@@ -883,7 +931,7 @@ __device__ u32 filter_list(ListSmem<BLOCK, CAP, NB>& S, u32 m0, const StarFrame&
     float u, v;
     to_uv(F, p.x - F.cx, p.y - F.cy, u, v);
     const u32 b = bin_of<NB>(u, v);
-    const u64 k = cand_key(u, v, S.id[i]);
+    const u64 k = cand_key(nrm ? nrm[b] : make_float2(u, v), u, v, S.id[i]);
     S.bn[i] = (unsigned short)b;
     if (k > *(volatile u64*)&key[b]) atomicMax(&key[b], k);
   }

@@ -119,16 +119,27 @@ def _check(code: int, where: str):
         raise HullError(code, where)
 
 
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
 
 
 def _stream_handle(stream):
-    torch = _torch()
     if stream is None:
-        stream = torch.cuda.current_stream()
+        stream = _torch().cuda.current_stream()
     return ctypes.c_void_p(stream.cuda_stream)
+
+
+def _is_points(pts, torch):
+    """A tensor that the library reads as it is: int32 (n, 2), CUDA, contiguous."""
+    return (isinstance(pts, torch.Tensor) and pts.is_cuda and pts.dtype is torch.int32 and pts.dim() == 2
+            and pts.shape[1] == 2 and pts.is_contiguous())
 
 
 def _ptr(t):
@@ -185,14 +196,20 @@ class Context:
         """CCW hull vertex indices (int32 device tensor) of an (n, 2) int32
         point tensor; see hull_compute."""
         torch = _torch()
-        dev = torch.device("cuda", self.device)
-        pts = _as_points(pts, dev)
+        # The short way for a tensor that needs no conversion (a call on a
+        # thousand points takes as long in Python as on the GPU).
+        if not _is_points(pts, torch):
+            pts = _as_points(pts, torch.device("cuda", self.device))
         n = pts.shape[0]
         if out is None:
-            out = torch.empty(max(n, 1), dtype=torch.int32, device=dev)
+            out = torch.empty(max(n, 1), dtype=torch.int32, device=torch.device("cuda", self.device))
         cnt = ctypes.c_int64()
-        _check(_lib.hull_compute(self._h, _ptr(pts), n, _ptr(out), out.numel(), ctypes.byref(cnt),
-                                 _stream_handle(stream)), "hull_compute")
+        if stream is None:
+            stream = torch.cuda.current_stream()
+        code = _lib.hull_compute(self._h, pts.data_ptr(), n, out.data_ptr(), out.numel(), ctypes.byref(cnt),
+                                 stream.cuda_stream)
+        if code:
+            _check(code, "hull_compute")
         return out[: cnt.value]
 
     def compute_raw(self, pts, out, stream=None) -> int:
