@@ -228,7 +228,7 @@ struct StreamSmem {
 // the survivors pushed lane by lane 359 (5.2 TB/s).
 // Block b of G streams its share of the T tiles, [b T / G, (b + 1) T / G), in
 // runs of one instance each, raw survivors to the instance's second key / index scratch.
-__global__ void __launch_bounds__(BT_BLOCK)
+__global__ void __launch_bounds__(BT_BLOCK, 4)
 kb_stream(BatchStar a) {
   extern __shared__ __align__(128) unsigned char bt_smem[];
   StreamSmem& S = *reinterpret_cast<StreamSmem*>(bt_smem);
@@ -252,7 +252,8 @@ kb_stream(BatchStar a) {
     const u32 p0 = (u32)(t - tf) * BF_TILE, p1 = min(n, (u32)(te - tf) * BF_TILE);
     PolyHead H;
     star::RawSink<BF_NB, BT_SLICE> sink{S.sxy[wid], S.sidx[wid], 0u, &R.frame, &R.raw_count, a.error, R.key, R.nrm,
-                                        reinterpret_cast<int2*>(a.kb + sl), a.ib + sl, n, many(n)};
+                                        reinterpret_cast<int2*>(a.kb + sl), a.ib + sl, n, many(n), 0u,
+                                        reinterpret_cast<const int2*>(a.xy) + off};
     star::stream_ring(ring, reinterpret_cast<const int2*>(a.xy) + off + p0, p1 - p0, p0, (u32)wid, (u32)BT_WARPS, H,
                       S.tab, sink, a.error, [&] {
       H = R.head;

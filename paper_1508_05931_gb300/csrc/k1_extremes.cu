@@ -329,14 +329,14 @@ struct K1PSmem {
   u32 tab[kPolySlabs];
 };
 
-__global__ void __launch_bounds__(K1P_BLOCK)
+__global__ void __launch_bounds__(K1P_BLOCK, 1)
 k1_poly(const int2* __restrict__ P, u32 n, PolyTab* __restrict__ T, int2* __restrict__ rxy, u32* __restrict__ ridx) {
   extern __shared__ __align__(128) unsigned char k1p_smem[];
   K1PSmem& S = *reinterpret_cast<K1PSmem*>(k1p_smem);
   const int wid = threadIdx.x >> 5;
   PolyHead H;
   star::RawSink<kStarBins, K1P_SLICE> sink{S.sxy[wid], S.sidx[wid], 0u, &T->frame, &T->raw_count, &T->error, T->key,
-                                           T->nrm, rxy, ridx, n, many_raw(n)};
+                                           T->nrm, rxy, ridx, n, many_raw(n), 0u, P};
   star::Ring<K1P_STAGES, K1P_CH> ring{&S.ring[wid][0][0], S.bar[wid], 0u, true};
   ring.init();
   // Consecutive chunks go to consecutive blocks.

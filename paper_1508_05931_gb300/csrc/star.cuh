@@ -408,24 +408,54 @@ struct RawSink {
   u32 bound;                // capacity of (rxy, ridx)
   u32 many;                 // past this many raw survivors nobody reads the candidates
 
+  u32 last;                 // the raw survivors' number at this warp's last flush
+  const int2* pts;          // the input (point of index id)
+
+  // A duplicate of its bin's candidate with a larger index goes no further
+  // (4M points of 40 distinct ones would leave a million); any other point
+  // is one more load away from it only when it reaches exactly as far.
   __device__ __forceinline__ void flush() {
     const int lane = threadIdx.x & 31;
     __syncwarp();
-    u32 base = 0;
-    if (lane == 0) base = atomicAdd(raw_count, fill);
-    base = __shfl_sync(0xFFFFFFFFu, base, 0);
+    u32 keep = 0;
+    static_assert(SLICE <= 1024, "a mask bit per round");
+    const bool cands = last <= many;
     const StarFrame F = *frame;
-    for (u32 q = lane; q < fill; q += 32) {
+    for (u32 r = 0; r * 32u < fill; ++r) {
+      const u32 q = lane + 32u * r;
+      if (q >= fill) break;
       const int2 p = sxy[q];
       const u32 id = sidx[q];
-      if (base + q < bound) { rxy[base + q] = p; ridx[base + q] = id; }
+      bool dup = false;
       if (out_of_range(p.x, p.y)) atomicOr(error, ERR_RANGE);
-      if (base > many) continue;
-      float u, v;
-      to_uv(F, p.x - F.cx, p.y - F.cy, u, v);
-      const u32 b = bin_of<NB>(u, v);
-      const u64 k = cand_key(__ldcg(&nrm[b]), u, v, id);
-      if (k > __ldcg(&key[b])) atomicMax(&key[b], k);
+      if (cands) {
+        float u, v;
+        to_uv(F, p.x - F.cx, p.y - F.cy, u, v);
+        const u32 b = bin_of<NB>(u, v);
+        const u64 k = cand_key(__ldcg(&nrm[b]), u, v, id), c = __ldcg(&key[b]);
+        if (k > c) {
+          atomicMax(&key[b], k);
+        } else if ((u32)(k >> 32) == (u32)(c >> 32)) {
+          const u32 cid = ~(u32)c;
+          const int2 w = pts[cid];
+          dup = w.x == p.x && w.y == p.y && id > cid;
+        }
+      }
+      if (!dup) keep |= 1u << r;
+    }
+    __syncwarp();
+    u32 tot = 0;
+    for (u32 r = 0; r * 32u < fill; ++r) tot += __popc(__ballot_sync(0xFFFFFFFFu, (keep >> r) & 1u));
+    u32 at = 0;
+    if (lane == 0) at = atomicAdd(raw_count, tot);
+    last = at = __shfl_sync(0xFFFFFFFFu, at, 0);
+    for (u32 r = 0; r * 32u < fill; ++r) {
+      const u32 bal = __ballot_sync(0xFFFFFFFFu, (keep >> r) & 1u);
+      if ((keep >> r) & 1u) {
+        const u32 o = at + __popc(bal & ((1u << lane) - 1u));
+        if (o < bound) { rxy[o] = sxy[lane + 32u * r]; ridx[o] = sidx[lane + 32u * r]; }
+      }
+      at += __popc(bal);
     }
     __syncwarp();
     fill = 0;

@@ -57,6 +57,15 @@ def test_sizes(ctx, family, n):
     check(ctx, points(family, n, n))
 
 
+@pytest.mark.parametrize("distinct", [5, 40, 3000])
+@pytest.mark.parametrize("n", [70001, 300000])
+def test_duplicates_of_few(ctx, n, distinct):
+    """Most raw survivors are duplicates of a candidate: the smallest index of
+    every vertex, whichever copy came first."""
+    rng = np.random.default_rng(distinct)
+    check(ctx, W.uniform_disk(distinct, 2.0 ** 29, 3)[rng.integers(0, distinct, size=n)])
+
+
 @pytest.mark.parametrize("n", [65536, 70001, 131071])
 def test_odd_rows_and_repeated_calls(ctx, n):
     """Views that start on an odd row, twice each (the tables are left clear
