@@ -144,8 +144,9 @@ hull_status hull_compute_host(hull_ctx *ctx, const int32_t *h_xy, int64_t n, int
  * `stream`, odd ones on an internal stream that first waits for the work
  * queued on `stream` before the call; each lane has its own workspace (the
  * second is allocated by the first such call and kept).  One
- * synchronisation at the end, after both lanes (an input whose bucket sort
- * needs the radix passes is rerun afterwards, alone).  With a single input
+ * synchronisation at the end, after both lanes (an input that the star path
+ * did not decide, or whose bucket sort needs the radix passes, goes on
+ * afterwards, alone).  With a single input
  * or the learned proposal, the hulls run back to back on `stream`.
  * Returns the first failing input's status (every
  * other input is still computed; h_count as hull_compute sets it).  With

@@ -909,6 +909,10 @@ hull_status hull_compute_multi(hull_ctx* c, int32_t count, const int32_t* const*
     if (e == cudaSuccess) e = cudaStreamWaitEvent(c->aux, c->bev[0], 0);
     if (e != cudaSuccess) return cuda_fail(e);
   }
+  // The input whose raw survivors lane l's workspace holds (-1: none): the
+  // last one that went through the single-read front there, until anything
+  // else writes the lane's chain buffers (a small input's one launch does not).
+  int32_t held[2] = {-1, -1};
   for (int32_t k = 0; k < count; ++k) {
     if (n[k] == 0) continue;
     const bool lane1 = two && (k & 1);
@@ -917,6 +921,8 @@ hull_status hull_compute_multi(hull_ctx* c, int32_t count, const int32_t* const*
     c->prof_pending = false;
     Plan* sum = reinterpret_cast<Plan*>(c->h_multi + (size_t)k * kSummaryBytes);
     const bool star = star_eligible(c, (u32)n[k]);
+    if (!star) held[lane1] = -1;
+    else if (single_read((u32)n[k])) held[lane1] = k;
     if (star) {
       r = run_star(c, d_xy[k], (u32)n[k], d_out[k], cap[k], sum, ls);
     } else {
@@ -940,29 +946,48 @@ hull_status hull_compute_multi(hull_ctx* c, int32_t count, const int32_t* const*
   }
   const cudaError_t e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_fail(e);
+  // An input that was not decided goes on alone, from the next step on, in
+  // its lane's workspace: the input that the lane still holds first, from its
+  // raw survivors, every other one from its points (whatever goes on in a
+  // workspace writes over the raw survivors there).
+  auto summary = [&](int32_t k) -> const Plan& {
+    return *reinterpret_cast<const Plan*>(c->h_multi + (size_t)k * kSummaryBytes);
+  };
+  auto settle = [&](int32_t k) -> hull_status {
+    Next next = NEXT_NONE;
+    const Plan& p = summary(k);
+    hull_status s = read_summary(c, p, &next);
+    if (next == NEXT_NONE) {
+      if (c->cfg.collect_stats) c->last.sort_fallback = 0;
+      if (s == HULL_OK || s == HULL_ECAPACITY) h_count[k] = p.h;
+      return s;
+    }
+    const bool lane1 = two && (k & 1);
+    const From from = next == NEXT_RADIX ? FROM_RADIX : after_star(p, (u32)n[k], held[lane1] == k);
+    held[lane1] = -1;
+    if (next == NEXT_RADIX) c->fallbacks += 1;
+    if (lane1) { std::swap(c->ws, c->ws2); std::swap(c->plan, c->plan2); }
+    s = compute_from(c, d_xy[k], (u32)n[k], d_out[k], cap[k], &h_count[k], st, from, p.s_raw);
+    if (lane1) { std::swap(c->ws, c->ws2); std::swap(c->plan, c->plan2); }
+    return s;
+  };
+  const int32_t early[2] = {held[0], held[1]};
+  hull_status early_status[2] = {HULL_OK, HULL_OK};
+  int32_t early_learned[2] = {0, 0};
+  for (int l = 0; l < 2; ++l)
+    if (early[l] >= 0) {
+      early_status[l] = settle(early[l]);
+      early_learned[l] = c->last.learned_used;
+    }
   hull_status first = HULL_OK;
   for (int32_t k = 0; k < count; ++k) {
     if (n[k] == 0) {
       if (c->cfg.collect_stats) c->last = hull_stats{};
       continue;
     }
-    Next next = NEXT_NONE;
-    const Plan& p = *reinterpret_cast<const Plan*>(c->h_multi + (size_t)k * kSummaryBytes);
-    r = read_summary(c, p, &next);
-    if (next != NEXT_NONE) {
-      // Not decided: this input again, alone, from the next step on.  The
-      // last input of a lane still has its raw survivors in the lane's workspace.
-      const bool lane1 = two && (k & 1);
-      const bool last = two ? k + 2 >= count : k + 1 >= count;
-      if (lane1) { std::swap(c->ws, c->ws2); std::swap(c->plan, c->plan2); }
-      if (next == NEXT_RADIX) c->fallbacks += 1;
-      r = compute_from(c, d_xy[k], (u32)n[k], d_out[k], cap[k], &h_count[k], st,
-                       next == NEXT_RADIX ? FROM_RADIX : after_star(p, (u32)n[k], last), p.s_raw);
-      if (lane1) { std::swap(c->ws, c->ws2); std::swap(c->plan, c->plan2); }
-    } else {
-      if (c->cfg.collect_stats) c->last.sort_fallback = 0;
-      if (r == HULL_OK || r == HULL_ECAPACITY) h_count[k] = p.h;
-    }
+    const int l = k == early[0] ? 0 : k == early[1] ? 1 : -1;
+    if (l >= 0) c->last.learned_used = early_learned[l];
+    r = l >= 0 ? early_status[l] : settle(k);
     if (r != HULL_OK && first == HULL_OK) first = r;
   }
   return first;
