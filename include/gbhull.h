@@ -63,9 +63,7 @@ typedef struct {
                          (on the two-read front and in batched mode; the single-read
                          front's sample polygon and witness test leave it nothing to gain) */
   int collect_stats;  /* 1 = keep survivor counts of the last call for hull_last_stats */
-  uint32_t spin_limit;/* iteration limit of the device waits between blocks and of the radix
-                         path's copies; 0 = default (1 << 22).  The single-read pass's copies
-                         into shared memory have a fixed limit (1 << 24) */
+  uint32_t spin_limit;/* iteration limit of every device wait; 0 = default (1 << 22) */
   int autotune;       /* 1 = time the batched kernels' block sizes per size bucket and the
                          boundary of the segmented path on first use and cache the choice
                          (file: $GBHULL_AUTOTUNE_CACHE, else ~/.cache/gbhull_autotune.json);

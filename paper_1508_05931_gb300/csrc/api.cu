@@ -385,7 +385,7 @@ cudaError_t star_front(hull_ctx* c, const int32_t* d_xy, u32 n, cudaStream_t st)
   if (e == cudaSuccess) e = launch_poly(d_xy, n, w.poly, c->num_sms, st);
   mark(c, 1, st);
   if (e == cudaSuccess)
-    e = launch_k1_poly(d_xy, n, w.poly, w.h_xy[0], reinterpret_cast<u32*>(w.h_idx[0]), c->num_sms, st);
+    e = launch_k1_poly(d_xy, n, c->cfg.spin_limit, w.poly, w.h_xy[0], reinterpret_cast<u32*>(w.h_idx[0]), c->num_sms, st);
   return e;
 }
 
@@ -2030,7 +2030,7 @@ hull_status hull_compute_batched(hull_ctx* c, const int32_t* d_xy, const int64_t
     a.xy = d_xy; a.offsets = reinterpret_cast<const long long*>(d_offsets);
     a.order = w.order; a.tfirst = w.tfirst; a.slot0 = w.slot0; a.kb = w.kb; a.ib = w.ib; a.rec = w.rec;
     a.out_tmp = w.out_tmp; a.hcount = w.hcount; a.error = w.ctl + 2; a.queue = w.ctl + 6;
-    a.redo = w.redo; a.nredo = w.ctl + 5;
+    a.redo = w.redo; a.nredo = w.ctl + 5; a.spin_limit = c->cfg.spin_limit;
     e = cudaMemcpyAsync(w.order, w.h_order, (size_t)B * 4, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(w.tfirst, w.h_tfirst, ((size_t)a.nh + 1) * 4, cudaMemcpyHostToDevice, st);

@@ -255,7 +255,7 @@ kb_stream(BatchStar a) {
                                         reinterpret_cast<int2*>(a.kb + sl), a.ib + sl, n, many(n), 0u,
                                         reinterpret_cast<const int2*>(a.xy) + off};
     star::stream_ring(ring, reinterpret_cast<const int2*>(a.xy) + off + p0, p1 - p0, p0, (u32)wid, (u32)BT_WARPS, H,
-                      S.tab, sink, a.error, [&] {
+                      S.tab, sink, a.error, a.spin_limit, [&] {
       H = R.head;
       for (u32 q = threadIdx.x; q < H.nslab; q += BT_BLOCK) S.tab[q] = R.tab[q];
       __syncthreads();

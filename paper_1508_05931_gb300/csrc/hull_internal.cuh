@@ -332,6 +332,14 @@ __device__ __forceinline__ bool mbar_try_wait(u64* bar, u32 parity) {
       : "=r"(ok) : "r"(smem_addr(bar)), "r"(parity) : "memory");
   return ok != 0u;
 }
+__device__ __forceinline__ bool mbar_test_wait(u64* bar, u32 parity) {
+  u32 ok;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+      " selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(ok) : "r"(smem_addr(bar)), "r"(parity) : "memory");
+  return ok != 0u;
+}
 // Waits for the given phase of `bar` to complete; false if it did not within
 // `limit` rounds (the call's spin limit for the waits of a ring; the fixed
 // kBulkWaitLimit for the drain at a kernel's end).

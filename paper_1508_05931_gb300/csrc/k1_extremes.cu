@@ -330,7 +330,8 @@ struct K1PSmem {
 };
 
 __global__ void __launch_bounds__(K1P_BLOCK, 1)
-k1_poly(const int2* __restrict__ P, u32 n, PolyTab* __restrict__ T, int2* __restrict__ rxy, u32* __restrict__ ridx) {
+k1_poly(const int2* __restrict__ P, u32 n, u32 spin_limit, PolyTab* __restrict__ T, int2* __restrict__ rxy,
+        u32* __restrict__ ridx) {
   extern __shared__ __align__(128) unsigned char k1p_smem[];
   K1PSmem& S = *reinterpret_cast<K1PSmem*>(k1p_smem);
   const int wid = threadIdx.x >> 5;
@@ -340,7 +341,8 @@ k1_poly(const int2* __restrict__ P, u32 n, PolyTab* __restrict__ T, int2* __rest
   star::Ring<K1P_STAGES, K1P_CH> ring{&S.ring[wid][0][0], S.bar[wid], 0u, true};
   ring.init();
   // Consecutive chunks go to consecutive blocks.
-  star::stream_ring(ring, P, n, 0u, wid * gridDim.x + blockIdx.x, gridDim.x * K1P_WARPS, H, S.tab, sink, &T->error, [&] {
+  star::stream_ring(ring, P, n, 0u, wid * gridDim.x + blockIdx.x, gridDim.x * K1P_WARPS, H, S.tab, sink, &T->error,
+                    spin_limit, [&] {
     pdl_wait();              // the first loads are under way while K0 finishes
     H = T->head;
     for (u32 q = threadIdx.x; q < H.nslab; q += K1P_BLOCK) S.tab[q] = T->tab[q];
@@ -411,12 +413,13 @@ cudaError_t k1_poly_configure() {
              : e;
 }
 
-cudaError_t launch_k1_poly(const int* xy, u32 n, PolyTab* T, int2* rxy, u32* ridx, int num_sms, cudaStream_t st) {
+cudaError_t launch_k1_poly(const int* xy, u32 n, u32 spin_limit, PolyTab* T, int2* rxy, u32* ridx, int num_sms,
+                           cudaStream_t st) {
   const u32 most = num_sms > 4 ? (u32)num_sms - 2u : (u32)num_sms;    // two SMs for another lane's k_star
   const u32 blocks = (n + K1P_WARPS * K1P_CH - 1) / (K1P_WARPS * K1P_CH);
   const u32 grid = blocks < 1u ? 1u : (blocks < most ? blocks : most);
   return launch_after(k1_poly, dim3(grid), dim3(K1P_BLOCK), sizeof(K1PSmem), st, reinterpret_cast<const int2*>(xy), n,
-                      T, rxy, ridx);
+                      spin_limit, T, rxy, ridx);
 }
 
 cudaError_t launch_k1_raw(const int2* rxy, const u32* ridx, u32 n, u32 spin_limit, Plan* plan, ExtPartial* partials,

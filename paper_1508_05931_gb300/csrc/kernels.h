@@ -70,7 +70,8 @@ cudaError_t launch_k2_fused(const int* xy, u32 n, Plan* plan, const u64* wkey, c
 constexpr u32 kSmallMax = 1u << 16;
 cudaError_t launch_poly(const int* xy, u32 n, PolyTab* T, int num_sms, cudaStream_t st);
 cudaError_t k1_poly_configure();
-cudaError_t launch_k1_poly(const int* xy, u32 n, PolyTab* T, int2* rxy, u32* ridx, int num_sms, cudaStream_t st);
+cudaError_t launch_k1_poly(const int* xy, u32 n, u32 spin_limit, PolyTab* T, int2* rxy, u32* ridx, int num_sms,
+                           cudaStream_t st);
 cudaError_t launch_k1_raw(const int2* rxy, const u32* ridx, u32 n, u32 spin_limit, Plan* plan, ExtPartial* partials,
                           const PolyTab* T, int num_sms, cudaStream_t st);
 cudaError_t star_configure();
@@ -204,6 +205,7 @@ struct BatchStar {
   u32* queue;
   int* redo;
   u32* nredo;
+  u32 spin_limit;
 };
 int batch_star_tile();
 size_t batch_star_rec_bytes();

@@ -181,7 +181,7 @@ extern "C" hull_status hull_compute_noalloc(const int32_t* d_xy, int64_t n, int3
     u32* ridx = reinterpret_cast<u32*>(c.h_idx[0]);
     e = cudaMemsetAsync(c.poly, 0, kPolyClearBytes, st);
     if (e == cudaSuccess) e = launch_poly(d_xy, un, c.poly, d->num_sms, st);
-    if (e == cudaSuccess) e = launch_k1_poly(d_xy, un, c.poly, c.h_xy[0], ridx, d->num_sms, st);
+    if (e == cudaSuccess) e = launch_k1_poly(d_xy, un, kDefaultSpinLimit, c.poly, c.h_xy[0], ridx, d->num_sms, st);
     if (e == cudaSuccess)
       e = launch_sectors(un, un, c.poly, c.sect, c.h_xy[0], ridx, c.h_xy[1], reinterpret_cast<u32*>(c.h_idx[1]), c.plan,
                          d_out, (long long)cap, d->num_sms, st);

@@ -389,6 +389,10 @@ __device__ __forceinline__ bool inside_poly(const PolyHead& H, const u32* tab, i
 }
 
 // ---------------------------------------------------------------- the stream
+// Flag in a lane's mask of survivors (which has at most 16 bits): its chunk
+// did not come in time.
+constexpr u32 kLate = 0x80000000u;
+
 // Where a warp puts the points on or outside the polygon: its slice of
 // SLICE staged points, flushed with one atomic reservation into (rxy, ridx),
 // in no particular order; every flushed point is offered as the candidate of
@@ -463,10 +467,12 @@ struct RawSink {
   // Bit 2 u + v of m: the lane's point at[64 u + v] survives (index id + 64 u
   // + v); the whole warp calls it, at most SLICE points in all.  A scan over
   // the lanes and a loop over each one's few points: a ballot per slot cost
-  // as much as the tests themselves where one point in fifty survives.
-  __device__ __forceinline__ void push_lanes(u32 m, const int2* at, u32 id) {
+  // as much as the tests themselves where one point in fifty survives.  A lane
+  // with kLate set in m: nothing is pushed and all lanes get false (its vote
+  // rides on the scan: a vote of its own took 1 % of the batched pass).
+  __device__ __forceinline__ bool push_lanes(u32 m, const int2* at, u32 id) {
     const int lane = threadIdx.x & 31;
-    const u32 c = __popc(m);
+    const u32 c = __popc(m & ~kLate) + (m >> 31 << 16);
     u32 inc = c;
     #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -474,6 +480,7 @@ struct RawSink {
       if (lane >= o) inc += t;
     }
     const u32 tot = __shfl_sync(0xFFFFFFFFu, inc, 31);
+    if (tot >> 16) return false;
     if (fill + tot > (u32)SLICE) flush();
     u32 q = fill + inc - c;
     while (m) {
@@ -485,6 +492,7 @@ struct RawSink {
       ++q;
     }
     fill += tot;
+    return true;
   }
   // One point per lane (the whole warp calls it; out: the point survives).
   __device__ __forceinline__ void push(bool out, int x, int y, u32 id) {
@@ -525,7 +533,8 @@ __device__ __forceinline__ void take_pairs(const PolyHead& H, const u32* tab, co
 // warp (STAGES chunks of CH points; no block barrier, no registers held by
 // loads in flight: 64 registers a thread for the register double buffer kept
 // every other kernel off the SM).  The warp takes chunks first + k step.
-// Waits are bounded (kBulkWaitLimit); one that runs out sets ERR_TIMEOUT.
+// Waits are bounded by the call's spin limit; one that runs out sets
+// ERR_TIMEOUT and ends the warp's stream.
 template <int STAGES, int CH>
 struct Ring {
   int4* buf;                // [STAGES][CH / 2], this warp's
@@ -554,8 +563,8 @@ struct Ring {
 template <int STAGES, int CH, class Sink, class Prep>
 __device__ __forceinline__ void stream_ring(Ring<STAGES, CH>& ring, const int2* __restrict__ Q, u32 cnt, u32 id0,
                                             u32 first, u32 step, const PolyHead& H, const u32* tab, Sink& sink,
-                                            u32* error, Prep prep) {
-  static_assert(CH % 64 == 0 && CH <= 512, "whole pairs per lane, one mask bit per point");
+                                            u32* error, u32 spin, Prep prep) {
+  static_assert(CH % 64 == 0 && CH <= 512, "whole pairs per lane, a mask bit per point below kLate");
   constexpr u32 R = CH / 2;                       // pairs per chunk
   const int lane = threadIdx.x & 31;
   const u32 head = (reinterpret_cast<uintptr_t>(Q) & 15u) && cnt ? 1u : 0u;
@@ -569,23 +578,28 @@ __device__ __forceinline__ void stream_ring(Ring<STAGES, CH>& ring, const int2* 
   prep();
   for (u32 k = 0; k < mine; ++k, ++ring.it) {
     const u32 st = ring.it % STAGES;
-    if (!mbar_wait(&ring.bar[st], (ring.it / STAGES) & 1u)) {
-      atomicOr(error, ERR_TIMEOUT);
-      ring.ok = false;                // the copies still in flight get their time too
-      for (u32 j = 1; j < (u32)STAGES && k + j < mine; ++j)
-        mbar_wait(&ring.bar[(ring.it + j) % STAGES], ((ring.it + j) / STAGES) & 1u);
-      break;
-    }
+    // A limit of one gives up on what is not there at once (a try suspends for
+    // as long as the hardware likes).
+    const u32 par = (ring.it / STAGES) & 1u;
+    const bool got = spin > 1u ? mbar_wait(&ring.bar[st], par, spin) : mbar_test_wait(&ring.bar[st], par);
     const int4* b = ring.buf + st * R + lane;
     const u32 id = id0 + head + 2u * ((first + k * step) * R + lane);
-    u32 m = 0;                        // the lane's points outside, pair u's at bits 2 u and 2 u + 1
+    u32 m = got ? 0u : kLate;         // the lane's points outside, pair u's at bits 2 u and 2 u + 1
     #pragma unroll
     for (int u = 0; u < (int)R / 32; ++u) {
       const int4 w = b[32 * u];
       m |= inside_poly(H, tab, w.x, w.y) ? 0u : 1u << (2 * u);
       m |= inside_poly(H, tab, w.z, w.w) ? 0u : 2u << (2 * u);
     }
-    if (__any_sync(0xFFFFFFFFu, m != 0u)) sink.push_lanes(m, reinterpret_cast<const int2*>(b), id);
+    if (__any_sync(0xFFFFFFFFu, m != 0u) && !sink.push_lanes(m, reinterpret_cast<const int2*>(b), id)) {
+      // The whole warp gives up, whichever lane's wait ran out.
+      if (lane == 0) atomicOr(error, ERR_TIMEOUT);
+      ring.ok = false;                // no further copy; those in flight, this one too, get their time
+      for (u32 j = 0; j < (u32)STAGES && k + j < mine; ++j)
+        mbar_wait(&ring.bar[(ring.it + j) % STAGES], ((ring.it + j) / STAGES) & 1u);
+      __syncwarp();
+      break;
+    }
     __syncwarp();
     if (lane == 0 && k + STAGES < mine) ring.load(ring.it + STAGES, p4 + (size_t)(first + (k + STAGES) * step) * R, pol);
   }
