@@ -2044,8 +2044,10 @@ hull_status hull_compute_batched(hull_ctx* c, const int32_t* d_xy, const int64_t
     if (e == cudaSuccess) e = output();
     if (e != cudaSuccess) return cuda_fail(e);
   }
+  // A pass that failed ends the call: the next one would clear its error
+  // bits, and instances with points left out could pass for decided.
   const u32 nredo = w.h_ctl[5];
-  if (nredo > 0 && nredo <= (u32)B && !(w.h_ctl[2] & ERR_RANGE)) {
+  if (nredo > 0 && nredo <= (u32)B && !(w.h_ctl[2] & (ERR_RANGE | ERR_TIMEOUT | ERR_INTERNAL))) {
     todo.resize(nredo);
     e = cudaMemcpyAsync(todo.data(), w.redo, (size_t)nredo * 4, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = layout(seg_boundary());      // waits for the stream first
