@@ -1990,11 +1990,11 @@ hull_status hull_compute_batched(hull_ctx* c, const int32_t* d_xy, const int64_t
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e);
   }
-  // The output: the hulls' offsets, every hull copied to its place, the
-  // error bits and the number of undecided instances read back.
+  // The output: the hulls' offsets, every hull copied to its place (when none
+  // is undecided), the error bits and the number of undecided instances read back.
   auto output = [&]() -> cudaError_t {
     cudaError_t r = launch_batch_output(w.hcount, w.slot0, w.out_tmp, B, reinterpret_cast<long long*>(d_out_offsets),
-                                        d_out, (long long)cap, w.ctl + 2, c->num_sms * 4, st);
+                                        d_out, (long long)cap, w.ctl + 2, w.ctl + 5, c->num_sms * 4, st);
     if (r == cudaSuccess) r = cudaMemcpyAsync(w.h_ctl, w.ctl, 32, cudaMemcpyDeviceToHost, st);
     return r == cudaSuccess ? cudaStreamSynchronize(st) : r;
   };

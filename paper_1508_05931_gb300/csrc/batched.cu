@@ -1152,10 +1152,13 @@ __global__ void k_batch_scan(const u32* __restrict__ hcount, int B, long long* o
   }
 }
 
+// Nothing is copied while instances are undecided (their hulls would still
+// shift the others' places and may exceed the capacity), after an error, or
+// past the capacity (k_batch_scan has flagged it).
 __global__ void k_batch_copy(const u32* __restrict__ hcount, const long long* __restrict__ slot0,
                              const int* __restrict__ out_tmp, const long long* __restrict__ out_off,
-                             int B, int* out, long long cap) {
-  if (out_off[B] > cap) return;
+                             int B, int* out, const u32* __restrict__ error, const u32* __restrict__ undecided) {
+  if (*error | *undecided) return;
   for (int i = blockIdx.x; i < B; i += gridDim.x) {
     const u32 h = hcount[i];
     const long long o = out_off[i], s0 = slot0[i];
@@ -1463,9 +1466,9 @@ cudaError_t launch_batch(int block, int grid, const BatchLaunch& L, cudaStream_t
 
 cudaError_t launch_batch_output(const u32* hcount, const long long* slot0, const int* out_tmp,
                                 int B, long long* out_off, int* out, long long cap, u32* error,
-                                int grid, cudaStream_t st) {
+                                const u32* undecided, int grid, cudaStream_t st) {
   k_batch_scan<<<1, 1024, 0, st>>>(hcount, B, out_off, cap, error);
-  k_batch_copy<<<grid, 256, 0, st>>>(hcount, slot0, out_tmp, out_off, B, out, cap);
+  k_batch_copy<<<grid, 256, 0, st>>>(hcount, slot0, out_tmp, out_off, B, out, error, undecided);
   return cudaGetLastError();
 }
 

@@ -226,7 +226,7 @@ cudaError_t batch_configure(int* occ256, int* occ512);
 cudaError_t launch_batch(int block, int grid, const BatchLaunch& L, cudaStream_t st);
 cudaError_t launch_batch_output(const u32* hcount, const long long* slot0, const int* out_tmp,
                                 int B, long long* out_off, int* out, long long cap, u32* error,
-                                int grid, cudaStream_t st);
+                                const u32* undecided, int grid, cudaStream_t st);
 
 int mlp_num_params();
 cudaError_t launch_features(const int* xy, u32 n, float* feat, int* ext, int* ext_xy, cudaStream_t st);
