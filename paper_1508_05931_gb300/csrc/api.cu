@@ -1774,7 +1774,7 @@ hull_status hull_compute_batched(hull_ctx* c, const int32_t* d_xy, const int64_t
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     return e == cudaSuccess ? HULL_OK : cuda_fail(e);
   }
-  if (!d_xy) return HULL_EINVAL;
+  if (!d_xy || (w.h_off[B] > 0 && !aligned8(d_xy))) return HULL_EINVAL;
   // Workspace.
   if ((size_t)slots > w.cap_slots || (size_t)B > w.cap_b) {
     cudaDeviceSynchronize();

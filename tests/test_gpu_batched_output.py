@@ -42,3 +42,16 @@ def test_range_with_undecided_instances(hull_lib):
     with hull_lib.Context(0) as c, pytest.raises(hull_lib.HullError) as e:
         c.compute_batched(torch.as_tensor(np.concatenate(parts)).cuda(), torch.as_tensor(off).cuda(), out=out)
     assert e.value.code == hull_lib.HULL_ERANGE and (out == -7).all()
+
+
+def test_misaligned_points_are_refused(hull_lib):
+    """Points are read eight bytes at a time: a pointer between two of them is
+    an error before any launch, as in the single-hull calls."""
+    flat = torch.zeros(2 * 300 + 1, dtype=torch.int32, device="cuda")
+    off = torch.tensor([0, 100, 300], device="cuda")
+    with hull_lib.Context(0) as c:
+        with pytest.raises(hull_lib.HullError) as e:
+            c.compute_batched(flat[1:].view(300, 2), off)
+        assert e.value.code == hull_lib.HULL_EINVAL
+        v, o = c.compute_batched(flat[:-1].view(300, 2), off)
+        assert o.cpu().numpy().tolist() == [0, 1, 2] and v[:2].cpu().numpy().tolist() == [0, 0]
