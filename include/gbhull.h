@@ -60,8 +60,9 @@ typedef enum {
 
 typedef struct {
   int proposal;       /* 0 = quadrilateral of the four extremes (the paper), 1 = learned
-                         (on the two-read front and in batched mode; the single-read
-                         front's sample polygon and witness test leave it nothing to gain) */
+                         (on the two-read front and, in batched mode, for instances of
+                         262,144 points or more that the star path does not take; the
+                         single-read front's sample polygon leaves it nothing to gain) */
   int collect_stats;  /* 1 = keep survivor counts of the last call for hull_last_stats */
   uint32_t spin_limit;/* iteration limit of every device wait; 0 = default (1 << 22) */
   int autotune;       /* 1 = time the batched kernels' block sizes per size bucket and the
@@ -75,9 +76,10 @@ typedef struct {
                          hull is the same, r_lower / r_upper count the points it keeps);
                          0 = the paper's single second round */
   int batched_seg_min;/* hull_compute_batched: instances of at least this many points take
-                         the segmented path (streaming passes over all their tiles at once);
-                         0 = the autotuned boundary (autotune = 1) or 65,536; above
-                         hull_batched_max_instance(): no instance takes it */
+                         the segmented path (streaming passes over all their tiles at once),
+                         the others one block each; above hull_batched_max_instance(): no
+                         instance takes it.  0 = the star path first, these two for what it
+                         does not decide, with the autotuned boundary (autotune = 1) or 65,536 */
 } hull_config;
 
 typedef struct {
@@ -169,26 +171,26 @@ hull_status hull_compute_host_multi(hull_ctx *ctx, int32_t count, const int32_t 
                                     int64_t *h_count, void *stream);
 
 /* B independent hulls in one call (Section 2.1's pipeline on every
- * instance).  Instances of at least hull_config.batched_seg_min points (or
- * the autotuned / default boundary) take the segmented path: two flat
- * streaming passes over all their 16,384-point tiles at once (extremes;
- * witness test and filter polygon), with one block per instance for its
- * plan and, after the passes, for its sort, second round and chains.  The
- * others go one block per instance through a persistent launch per size
- * bucket (up to 16,384 points, more), instances taken largest first, on
- * the context's second stream.  d_offsets: device int64[B+1], instance b is points
- * [d_offsets[b], d_offsets[b+1]) of d_xy (non-decreasing, d_offsets[0] = 0).
+ * instance).  The star path (see hull_compute) takes every instance first:
+ * one block per instance of at most 16,384 points, the larger ones through
+ * one flat pass over all their points.  The instances that it does not
+ * decide, or all of them when hull_config.batched_seg_min is set, go one of
+ * two ways.  Instances of at least that many points (else the autotuned or
+ * default boundary) take the segmented path: two flat streaming passes over
+ * all their 16,384-point tiles at once (extremes; witness test and filter
+ * polygon), with one block per instance for its plan and, after the passes,
+ * for its sort, second round and chains.  The others go one block per
+ * instance through a persistent launch per size bucket (up to 16,384 points,
+ * more), instances taken largest first, on the context's second stream.
+ * autotune times these two ways.  d_offsets: device int64[B+1], instance b is
+ * points [d_offsets[b], d_offsets[b+1]) of d_xy (non-decreasing, d_offsets[0] = 0).
  * Vertex indices are relative to their instance and are written to d_out at
  * d_out_offsets[b] (device int64[B+1], written by the call;
  * d_out_offsets[B] = total vertices).  cap bounds the total (HULL_ECAPACITY
  * leaves d_out untouched but still writes d_out_offsets).  Total points must
  * be < 2^30 and every instance at most hull_batched_max_instance() points
  * (else HULL_EINVAL).  Copies d_offsets to the host and synchronises
- * `stream`. *
- * The star path (see hull_compute) takes every instance first: one block per
- * instance of at most 16,384 points, the larger ones through one flat pass
- * over all their points.  The two ways above are for the instances that it
- * does not decide, and what autotune times. */
+ * `stream`. */
 hull_status hull_compute_batched(hull_ctx *ctx, const int32_t *d_xy, const int64_t *d_offsets,
                                  int32_t B, int32_t *d_out, int64_t cap, int64_t *d_out_offsets,
                                  void *stream);

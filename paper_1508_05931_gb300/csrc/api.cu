@@ -2000,8 +2000,10 @@ hull_status hull_compute_batched(hull_ctx* c, const int32_t* d_xy, const int64_t
   };
   // The star path: the large instances (in index order: their points are
   // streamed in one flat pass) and the small ones, by falling size class so
-  // that the longest blocks start first.
-  {
+  // that the longest blocks start first.  A caller who sets the segmented
+  // path's boundary gets the two paths that it divides.
+  const bool star = fixed_seg == 0;
+  if (star) {
     const int64_t stile = batch_star_tile();
     if (!todo.empty()) e = cudaStreamSynchronize(st);      // the autotuner's layout may still be copied
     if (e != cudaSuccess) return cuda_fail(e);
@@ -2046,10 +2048,11 @@ hull_status hull_compute_batched(hull_ctx* c, const int32_t* d_xy, const int64_t
   }
   // A pass that failed ends the call: the next one would clear its error
   // bits, and instances with points left out could pass for decided.
-  const u32 nredo = w.h_ctl[5];
-  if (nredo > 0 && nredo <= (u32)B && !(w.h_ctl[2] & (ERR_RANGE | ERR_TIMEOUT | ERR_INTERNAL))) {
+  const u32 nredo = star ? w.h_ctl[5] : (u32)B;
+  if (nredo > 0 && nredo <= (u32)B && !(star && (w.h_ctl[2] & (ERR_RANGE | ERR_TIMEOUT | ERR_INTERNAL)))) {
     todo.resize(nredo);
-    e = cudaMemcpyAsync(todo.data(), w.redo, (size_t)nredo * 4, cudaMemcpyDeviceToHost, st);
+    if (star) e = cudaMemcpyAsync(todo.data(), w.redo, (size_t)nredo * 4, cudaMemcpyDeviceToHost, st);
+    else std::iota(todo.begin(), todo.end(), 0);
     if (e == cudaSuccess) e = layout(seg_boundary());      // waits for the stream first
     if (e == cudaSuccess) e = run_all();
     if (e == cudaSuccess) e = output();
