@@ -200,7 +200,9 @@ __device__ __forceinline__ bool aborted(const Plan* plan) {
 // Programmatic dependent launch: a kernel launched with launch_after may
 // start while the kernel before it in the stream still runs; pdl_wait returns
 // when that one has completed (at once in an ordinary launch), pdl_launch
-// lets the next one start.
+// lets the next one start.  Such a kernel's __restrict__ is for the call's
+// input only: everything else may still be written by the kernel before while
+// this one runs, and read-only loads are for data that nobody writes then.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -330,8 +330,7 @@ struct K1PSmem {
 };
 
 __global__ void __launch_bounds__(K1P_BLOCK, 1)
-k1_poly(const int2* __restrict__ P, u32 n, u32 spin_limit, PolyTab* __restrict__ T, int2* __restrict__ rxy,
-        u32* __restrict__ ridx) {
+k1_poly(const int2* __restrict__ P, u32 n, u32 spin_limit, PolyTab* T, int2* rxy, u32* ridx) {
   extern __shared__ __align__(128) unsigned char k1p_smem[];
   K1PSmem& S = *reinterpret_cast<K1PSmem*>(k1p_smem);
   const int wid = threadIdx.x >> 5;

@@ -63,8 +63,7 @@ __device__ __forceinline__ int not_here(const PolyTab* T, u32 q, u32 n) {
 constexpr int KC_BLOCK = 512;
 
 __global__ void __launch_bounds__(KC_BLOCK)
-k_cand(const int2* __restrict__ P, u32 n, PolyTab* T, const int2* __restrict__ rxy, const u32* __restrict__ ridx,
-       int2* lxy, u32* lidx) {
+k_cand(const int2* __restrict__ P, u32 n, PolyTab* T, const int2* rxy, const u32* ridx, int2* lxy, u32* lidx) {
   __shared__ Cands S;
   const int lane = threadIdx.x & 31, t = threadIdx.x;
   if (t < kStarBins / 32) S.occ[t] = 0u;
@@ -116,8 +115,7 @@ k_cand(const int2* __restrict__ P, u32 n, PolyTab* T, const int2* __restrict__ r
 }
 
 __global__ void __launch_bounds__(KS_BLOCK)
-k_star(u32 n, PolyTab* T, const int2* __restrict__ lxy, const u32* __restrict__ lidx, Plan* plan, int* out,
-       long long cap) {
+k_star(u32 n, PolyTab* T, const int2* lxy, const u32* lidx, Plan* plan, int* out, long long cap) {
   extern __shared__ __align__(16) unsigned char ks_smem[];
   List& S = *reinterpret_cast<List*>(ks_smem);
   const int t = threadIdx.x;
