@@ -14,12 +14,18 @@
 //   the larger index.  (This takes c strictly inside the hull, which the
 //   verification below proves before any result is used.)
 // The drops of a round may use points that the same round drops: those are
-// input points too.  The rounds end with a polygon that is verified: every
-// consecutive cross product about c positive and every turn strictly left
-// means a convex polygon of input points with c strictly inside, in which
-// every other input point was shown to lie.  Anything else (a degenerate
-// set, a crowded bin, too many points or rounds) returns failure and the
-// caller takes the general path.
+// input points too.  The rounds end with a closed list that is verified: every
+// consecutive cross product about c positive and every turn strictly left.
+// That makes it a convex polygon of input points with c strictly inside, in
+// which every other input point was shown to lie, because the list goes round
+// c once.  The two local tests alone do not say so (a pentagram passes them);
+// the order does: the bins are one sweep of the whitened angle, whose error is
+// far below a right angle (frame_of bounds the map), inside a bin points stand
+// in exact order, and mend_order exchanges neighbours only.  Each step is
+// positive and below a half turn, and the angles follow one sweep, so the
+// steps add up to one turn.  A change of the order has to keep that.  Anything
+// else (a degenerate set, a crowded bin, too many points or rounds) returns
+// failure and the caller takes the general path.
 #pragma once
 
 #include "hull_internal.cuh"
@@ -95,10 +101,15 @@ __device__ __forceinline__ u32 block_scan(u32 v, u32* ws, u32& total) {
 
 // ---------------------------------------------------------------- frame
 // From strided points (V of every thread, relative to one point o of the
-// input): c, their mean rounded to integers, and the whitening map of their covariance (the inverse Cholesky factor,
-// determinant > 0).  Every block that calls it with the same P and n gets
+// input): c, their mean rounded to integers, and the whitening map of their
+// covariance (the inverse Cholesky factor, determinant > 0).  Every block that calls it with the same P and n gets
 // the same frame.  Nothing is assumed of c: a polygon of input points that
-// verifies about it proves that it lies inside.
+// verifies about it proves that it lies inside.  The map is bounded whatever
+// the sums lost to rounding (o far from a tight rest): |l21| <= sqrt(d) and
+// l22 >= 1e-4 sqrt(d) keep |m10| <= 1e4 m00, so a point's v is known to 3e4 x
+// 2^-24 |u| (two conversions and a product) and its angle to about 2^-9: a bin
+// spans far less than a half turn (bin_rank's order is total) and the bins are
+// one sweep of the angle.
 template <int BLOCK>
 struct FrameSmem {
   float sum[BLOCK / 32][5];
@@ -130,7 +141,8 @@ __device__ __forceinline__ StarFrame frame_of(const int2 (&p)[V], int2 o, FrameS
   }
   const float mx = s[0], my = s[1];
   const float a = fmaxf(s[2] - mx * mx, 1.0f), d = fmaxf(s[4] - my * my, 1.0f), b = s[3] - mx * my;
-  const float l11 = sqrtf(a), l21 = b / l11, l22 = sqrtf(fmaxf(d - l21 * l21, 1.0e-8f * d));
+  const float l11 = sqrtf(a), sd = sqrtf(d), l21 = fminf(fmaxf(b / l11, -sd), sd);
+  const float l22 = sqrtf(fmaxf(d - l21 * l21, 1.0e-8f * d));
   StarFrame F;
   F.m00 = 1.0f / l11;
   F.m11 = 1.0f / l22;
