@@ -119,6 +119,12 @@ struct PolyHead {
   int y0;
   u32 shy, nslab;
 };
+// No polygon because the sample lies on one line: its extremes a, b (equal
+// when it is one point), in range.
+struct PolyLine {
+  int ok;
+  int ax, ay, bx, by;
+};
 struct PolyTab {
   // cleared per call
   u64 best[kPolyDirs];   // per direction: (ordered projection << 32 | ~sample index), maximum
@@ -132,6 +138,7 @@ struct PolyTab {
   // written by k0
   StarFrame frame;
   PolyHead head;
+  PolyLine line;
   u32 tab[kPolySlabs];
   float2 nrm[kStarBins];  // directions of the bins' candidates
 };

@@ -76,6 +76,7 @@ k0_poly(const int2* __restrict__ P, u32 n, u32 ns, u32 slabs, PolyTab* __restric
   if (t == 0) {
     T->frame = F;
     T->head = H;
+    T->line = S.poly.line;
   }
 }
 

@@ -340,13 +340,13 @@ k1_poly(const int2* __restrict__ P, u32 n, u32 spin_limit, PolyTab* T, int2* rxy
   star::Ring<K1P_STAGES, K1P_CH> ring{&S.ring[wid][0][0], S.bar[wid], 0u, true};
   ring.init();
   // Consecutive chunks go to consecutive blocks.
-  star::stream_ring(ring, P, n, 0u, wid * gridDim.x + blockIdx.x, gridDim.x * K1P_WARPS, H, S.tab, sink, &T->error,
-                    spin_limit, [&] {
+  star::stream_ring(ring, P, n, 0u, wid * gridDim.x + blockIdx.x, gridDim.x * K1P_WARPS, H, &T->line, S.tab, sink,
+                    &T->error, spin_limit, [&] {
     pdl_wait();              // the first loads are under way while K0 finishes
     H = T->head;
     for (u32 q = threadIdx.x; q < H.nslab; q += K1P_BLOCK) S.tab[q] = T->tab[q];
     __syncthreads();
-  });
+  }, [&] { star::stream_line(P, n, 0u, wid * gridDim.x + blockIdx.x, gridDim.x * K1P_WARPS, &T->line, sink); });
   pdl_launch();
   if (sink.fill) sink.flush();
 }

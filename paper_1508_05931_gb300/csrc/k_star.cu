@@ -115,7 +115,8 @@ k_cand(const int2* __restrict__ P, u32 n, PolyTab* T, const int2* rxy, const u32
 }
 
 __global__ void __launch_bounds__(KS_BLOCK)
-k_star(u32 n, PolyTab* T, const int2* lxy, const u32* lidx, Plan* plan, int* out, long long cap) {
+k_star(u32 n, PolyTab* T, const int2* rxy, const u32* ridx, const int2* lxy, const u32* lidx, Plan* plan, int* out,
+       long long cap) {
   extern __shared__ __align__(16) unsigned char ks_smem[];
   List& S = *reinterpret_cast<List*>(ks_smem);
   const int t = threadIdx.x;
@@ -124,13 +125,15 @@ k_star(u32 n, PolyTab* T, const int2* lxy, const u32* lidx, Plan* plan, int* out
   const u32 id0 = lidx[t];
   const u32 q = min(T->raw_count, n), err = T->error;
   const int why = not_here(T, q, n);
-  if (why) {                          // s = 1 tells the degenerate case from too many points
-    if (t == 0) star_summary(plan, n, q, why == 1 ? 1u : 0u, -1, cap, err);
-    return;
-  }
-  const u32 m = T->list_count;
+  u32 m = T->list_count;
   int h = -1;
-  if (m <= kStarCap && !(err & ERR_RANGE)) {
+  if (why) {
+    // One line or one point, if the raw survivors say so; else s = 1 tells the
+    // degenerate case from too many points.
+    if (why == 1 && q >= 1u && q <= kStarCap && !(err & ERR_RANGE))
+      h = star::rest_of_list<KS_BLOCK>(S, rxy, ridx, q, out, cap);
+    m = why == 1 ? 1u : 0u;
+  } else if (m <= kStarCap && !(err & ERR_RANGE)) {
     for (u32 i = t; i < m; i += KS_BLOCK) {
       S.p[i] = i < (u32)KS_BLOCK ? p0 : lxy[i];
       S.id[i] = i < (u32)KS_BLOCK ? id0 : lidx[i];
@@ -214,7 +217,7 @@ k_small(const int2* __restrict__ P, u32 n, Plan* plan, int* out, long long cap) 
     h = star::list_hull<KS_BLOCK, KS_CAP, kStarBins>(S.list, m, F, out, cap);
   }
   if (h < 0 && !err && (flat || m0 <= (u32)KS_CAP)) {
-    h = star::rest_hull<KS_BLOCK>(S.list, P, n, out, cap);
+    h = star::rest_hull<KS_BLOCK>(S.list, P, nullptr, n, out, cap);
     m = 0u;                           // not undecided for being too many
   }
   if (t == 0) star_summary(plan, n, 0, m, h, cap, err);
@@ -237,7 +240,7 @@ cudaError_t launch_star(const int* xy, u32 n, PolyTab* T, const int2* rxy, const
   const cudaError_t e = launch_after(k_cand, dim3(want < most ? want : most), dim3(KC_BLOCK), 0, st,
                                      reinterpret_cast<const int2*>(xy), n, T, rxy, ridx, lxy, lidx);
   if (e != cudaSuccess) return e;
-  return launch_after(k_star, dim3(1), dim3(KS_BLOCK), sizeof(List), st, n, T, lxy, lidx, plan, out, cap);
+  return launch_after(k_star, dim3(1), dim3(KS_BLOCK), sizeof(List), st, n, T, rxy, ridx, lxy, lidx, plan, out, cap);
 }
 
 cudaError_t launch_small(const int* xy, u32 n, Plan* plan, int* out, long long cap, cudaStream_t st) {

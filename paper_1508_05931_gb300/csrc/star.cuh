@@ -64,6 +64,21 @@ __device__ __forceinline__ bool out_of_range(int x, int y) {
   return (u32)x + (u32)kCoordLimit > 2u * (u32)kCoordLimit || (u32)y + (u32)kCoordLimit > 2u * (u32)kCoordLimit;
 }
 
+// (x, y) as one word that orders points lexicographically, and back.
+__device__ __forceinline__ u64 lex_key(int2 p) {
+  return ((u64)((u32)p.x ^ 0x80000000u) << 32) | (u64)((u32)p.y ^ 0x80000000u);
+}
+__device__ __forceinline__ int2 lex_point(u64 v) {
+  return make_int2((int)((u32)(v >> 32) ^ 0x80000000u), (int)((u32)v ^ 0x80000000u));
+}
+
+// p in range and on the line through the extremes of L (their one point when they are equal).
+__device__ __forceinline__ bool on_line(const PolyLine& L, int2 p) {
+  if (out_of_range(p.x, p.y)) return false;
+  if (L.ax == L.bx && L.ay == L.by) return p.x == L.ax && p.y == L.ay;
+  return orient(L.ax, L.ay, L.bx, L.by, p.x, p.y) == 0;
+}
+
 // q dropped by the triangle (c, a, b); a, b, q relative to c.
 // orient(a, b, q) = cross(a, b) - cross(a, q) - cross(q, b): three products
 // (each below 2^61, the sum below 2^63).
@@ -185,6 +200,7 @@ struct PolySmem {
   float slope[kPolyDirs + 2];
   int k, ir, ymin, ymax;
   u64 alive;                            // sectors of the polygon's corners
+  PolyLine line;
 };
 
 // The polygon of the candidates (in angular order about c) and the table of
@@ -193,7 +209,8 @@ struct PolySmem {
 //
 // Warp 0 reduces the candidates to a convex polygon by rounds (the rule of
 // list_hull, the alive sectors in one 64-bit mask) and verifies it; a set
-// that does not verify gets no polygon (nothing is dropped).
+// that does not verify gets no polygon (nothing is dropped but, when all
+// candidates lie on one line, what lies between points of that line: S.line).
 //
 // Lower chain: corners 0 .. ir, x non-decreasing; upper chain: corners
 // ir .. k (corner k = corner 0), x non-increasing.  The lower chain is
@@ -210,6 +227,33 @@ struct PolySmem {
 // PAD: word s goes to tab[s + s / 32] (a thread's run of slabs then spreads
 // over the shared-memory banks).
 __device__ __forceinline__ u32 pad_slab(u32 s) { return s + (s >> 5); }
+
+// The line that all candidates lie on, if there is one (warp 0).
+static __device__ __noinline__ void line_of_sample(PolySmem& S) {
+  const int lane = threadIdx.x & 31;
+  const u64 has = ((u64)S.has[1] << 32) | S.has[0];
+  u64 mn = ~0ull, mx = 0ull;
+  #pragma unroll
+  for (int w = 0; w < 2; ++w)
+    if ((has >> (lane + 32 * w)) & 1ull) {
+      const u64 v = lex_key(S.p[lane + 32 * w]);
+      mn = v < mn ? v : mn; mx = v > mx ? v : mx;
+    }
+  #pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const u64 a = __shfl_xor_sync(0xFFFFFFFFu, mn, o), b = __shfl_xor_sync(0xFFFFFFFFu, mx, o);
+    mn = a < mn ? a : mn; mx = b > mx ? b : mx;
+  }
+  const int2 A = lex_point(mn), B = lex_point(mx);
+  PolyLine L{1, A.x, A.y, B.x, B.y};
+  bool on = has != 0ull && !out_of_range(A.x, A.y) && !out_of_range(B.x, B.y);
+  #pragma unroll
+  for (int w = 0; w < 2; ++w)
+    if ((has >> (lane + 32 * w)) & 1ull) on = on && on_line(L, S.p[lane + 32 * w]);
+  L.ok = __all_sync(0xFFFFFFFFu, on);
+  __syncwarp();
+  if (lane == 0) S.line = L;
+}
 
 template <int BLOCK, bool PAD = false>
 __device__ PolyHead build_poly(PolySmem& S, const StarFrame& F, u32* tab, u32 slabs) {
@@ -249,10 +293,7 @@ __device__ PolyHead build_poly(PolySmem& S, const StarFrame& F, u32* tab, u32 sl
     // Corners from the lexicographic minimum on.
     const int k = ok ? __popcll(alive) : 0;
     if (ok) {
-      auto lex = [&](int j) {
-        const int2 p = S.p[j];
-        return ((u64)((u32)p.x ^ 0x80000000u) << 32) | (u64)((u32)p.y ^ 0x80000000u);
-      };
+      auto lex = [&](int j) { return lex_key(S.p[j]); };
       u64 mn = ~0ull, mx = 0ull;
       int ylo = 0x7FFFFFFF, yhi = (int)0x80000000;
       #pragma unroll
@@ -299,7 +340,8 @@ __device__ PolyHead build_poly(PolySmem& S, const StarFrame& F, u32* tab, u32 sl
       }
       if (lane == 0) { S.ir = r1 >= r0 ? r1 - r0 : r1 - r0 + k; S.ymin = ylo; S.ymax = yhi; S.hx[k] = S.hx[0]; }
     }
-    if (lane == 0) { S.k = k; S.alive = alive; }
+    if (lane == 0) { S.k = k; S.alive = alive; S.line.ok = 0; }
+    if (!ok) line_of_sample(S);
   }
   __syncthreads();
   const int k = S.k;
@@ -572,10 +614,55 @@ struct Ring {
   }
 };
 
-template <int STAGES, int CH, class Sink, class Prep>
+// The points of a set whose sample lies on the line L: of those on it only
+// each warp's lexicographic extremes survive (what lies between two of them
+// is no vertex, an equal point with a larger index neither), every other
+// point does.  Without it all points of a line were raw survivors (20M points
+// 1,943 us a call, 1,655 before the star path).  Out of line, with a sink of
+// its own that it empties: the ring's loop keeps its registers.
+template <class Sink>
+__device__ __noinline__ void stream_line(const int2* Q, u32 cnt, u32 id0, u32 first, u32 step, const PolyLine* line,
+                                         Sink sink) {
+  const PolyLine L = *line;
+  constexpr u32 V = 4, R = 32u * V;
+  const int lane = threadIdx.x & 31;
+  u64 lo = ~0ull, hi = 0ull;
+  u32 ilo = 0xFFFFFFFFu, ihi = 0xFFFFFFFFu;       // a lane's indices increase: the first of equal points
+  for (u32 b = first; b < (cnt + R - 1u) / R; b += step) {
+    int2 p[V];
+    #pragma unroll
+    for (u32 r = 0; r < V; ++r) p[r] = b * R + 32u * r + lane < cnt ? Q[b * R + 32u * r + lane] : make_int2(0, 0);
+    #pragma unroll
+    for (u32 r = 0; r < V; ++r) {
+      const u32 i = b * R + 32u * r + lane;
+      const bool in = i < cnt, on = in && on_line(L, p[r]);
+      if (on) {
+        const u64 v = lex_key(p[r]);
+        if (v < lo) { lo = v; ilo = id0 + i; }
+        if (ihi == 0xFFFFFFFFu || v > hi) { hi = v; ihi = id0 + i; }
+      }
+      sink.push(in && !on, p[r].x, p[r].y, id0 + i);
+    }
+  }
+  #pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const u64 a = __shfl_xor_sync(0xFFFFFFFFu, lo, o), c = __shfl_xor_sync(0xFFFFFFFFu, hi, o);
+    const u32 ia = __shfl_xor_sync(0xFFFFFFFFu, ilo, o), ic = __shfl_xor_sync(0xFFFFFFFFu, ihi, o);
+    if (a < lo || (a == lo && ia < ilo)) { lo = a; ilo = ia; }
+    if (c > hi || (c == hi && ic < ihi)) { hi = c; ihi = ic; }
+  }
+  const bool any = ilo != 0xFFFFFFFFu;
+  const int2 w = lex_point(lane == 0 ? lo : hi);
+  sink.push(any && (lane == 0 || (lane == 1 && lo != hi)), w.x, w.y, lane == 0 ? ilo : ihi);
+  if (sink.fill) sink.flush();
+}
+
+// flat(): called by the warp instead of the stream when the sample lies on
+// one line (its copies have landed).
+template <int STAGES, int CH, class Sink, class Prep, class Flat>
 __device__ __forceinline__ void stream_ring(Ring<STAGES, CH>& ring, const int2* __restrict__ Q, u32 cnt, u32 id0,
-                                            u32 first, u32 step, const PolyHead& H, const u32* tab, Sink& sink,
-                                            u32* error, u32 spin, Prep prep) {
+                                            u32 first, u32 step, const PolyHead& H, const PolyLine* line,
+                                            const u32* tab, Sink& sink, u32* error, u32 spin, Prep prep, Flat flat) {
   static_assert(CH % 64 == 0 && CH <= 512, "whole pairs per lane, a mask bit per point below kLate");
   constexpr u32 R = CH / 2;                       // pairs per chunk
   const int lane = threadIdx.x & 31;
@@ -588,6 +675,19 @@ __device__ __forceinline__ void stream_ring(Ring<STAGES, CH>& ring, const int2* 
   if (lane == 0)
     for (u32 k = 0; k < min(mine, (u32)STAGES); ++k) ring.load(ring.it + k, p4 + (size_t)(first + k * step) * R, pol);
   prep();
+  if (!H.ok && line->ok) {            // the chunks under way are not needed
+    const u32 out = min(mine, (u32)STAGES);
+    bool got = true;
+    for (u32 j = 0; j < out; ++j)
+      got = mbar_wait(&ring.bar[(ring.it + j) % STAGES], ((ring.it + j) / STAGES) & 1u) && got;
+    ring.it += out;
+    if (!__all_sync(0xFFFFFFFFu, got)) {
+      if (lane == 0) atomicOr(error, ERR_TIMEOUT);
+      ring.ok = false;
+    }
+    flat();
+    return;
+  }
   for (u32 k = 0; k < mine; ++k, ++ring.it) {
     const u32 st = ring.it % STAGES;
     // A limit of one gives up on what is not there at once (a try suspends for
@@ -946,10 +1046,7 @@ __device__ int list_hull(ListSmem<BLOCK, CAP, NB>& S, u32 m, const StarFrame& F,
   m = drop_rounds<BLOCK, false>(S, m, F, S.tb, cur, true, done);
   if (!done) return -1;
   // The lexicographic minimum starts the output.
-  auto lex = [&](u32 i) {
-    const int2 p = S.p[cur[i]];
-    return ((u64)((u32)p.x ^ 0x80000000u) << 32) | (u64)((u32)p.y ^ 0x80000000u);
-  };
+  auto lex = [&](u32 i) { return lex_key(S.p[cur[i]]); };
   u64 mn = ~0ull;
   for (u32 i = t; i < m; i += BLOCK) { const u64 v = lex(i); mn = v < mn ? v : mn; }
   {
@@ -1021,22 +1118,24 @@ __device__ u32 filter_list(ListSmem<BLOCK, CAP, NB>& S, u32 m0, const StarFrame&
   return m;
 }
 
-// A degenerate or tiny input that the rounds did not decide (n >= 1 points in
-// range; the whole block): all points equal or on one line, found from the
-// lexicographic extremes; up to 64 points by Andrew's chain in one thread.
-// The number of vertices (in out when they fit) or -1.
+// A degenerate or tiny set that the rounds did not decide (n >= 1 points in
+// range with input indices ids, null: their positions; the whole block): all
+// points equal or on one line, found from the lexicographic extremes; up to 64
+// points by Andrew's chain in one thread.  The number of vertices (in out when
+// they fit) or -1.  Out of line: a rare call that shall not cost its callers
+// registers (inlined, kb_small took 112 us of a batch instead of 108).
 template <int BLOCK, class L>
-__device__ int rest_hull(L& S, const int2* __restrict__ P, u32 n, int* out, long long cap) {
+__device__ __noinline__ int rest_hull(L& S, const int2* P, const u32* ids, u32 n, int* out, long long cap) {
   __shared__ u64 s_lo, s_hi;
   __shared__ u32 s_il, s_ih;
   const int t = threadIdx.x;
-  auto lex = [](int2 p) { return ((u64)((u32)p.x ^ 0x80000000u) << 32) | (u64)((u32)p.y ^ 0x80000000u); };
+  auto id = [&](u32 i) { return ids ? ids[i] : i; };
   __syncthreads();
   if (t == 0) { s_lo = ~0ull; s_hi = 0ull; s_il = s_ih = 0xFFFFFFFFu; }
   __syncthreads();
   u64 lo = ~0ull, hi = 0ull;
   for (u32 i = t; i < n; i += BLOCK) {
-    const u64 v = lex(P[i]);
+    const u64 v = lex_key(P[i]);
     lo = v < lo ? v : lo; hi = v > hi ? v : hi;
   }
   #pragma unroll
@@ -1047,14 +1146,13 @@ __device__ int rest_hull(L& S, const int2* __restrict__ P, u32 n, int* out, long
   if ((t & 31) == 0) { atomicMin(&s_lo, lo); atomicMax(&s_hi, hi); }
   __syncthreads();
   lo = s_lo; hi = s_hi;
-  const int2 A = make_int2((int)((u32)(lo >> 32) ^ 0x80000000u), (int)((u32)lo ^ 0x80000000u));
-  const int2 B = make_int2((int)((u32)(hi >> 32) ^ 0x80000000u), (int)((u32)hi ^ 0x80000000u));
+  const int2 A = lex_point(lo), B = lex_point(hi);
   bool off = false;
   for (u32 i = t; i < n; i += BLOCK) {
     const int2 p = P[i];
-    const u64 v = lex(p);
-    if (v == lo) atomicMin(&s_il, i);
-    if (v == hi) atomicMin(&s_ih, i);
+    const u64 v = lex_key(p);
+    if (v == lo) atomicMin(&s_il, id(i));
+    if (v == hi) atomicMin(&s_ih, id(i));
     off = off || orient(A.x, A.y, B.x, B.y, p.x, p.y) != 0;
   }
   if (!__syncthreads_or(off)) {
@@ -1065,15 +1163,15 @@ __device__ int rest_hull(L& S, const int2* __restrict__ P, u32 n, int* out, long
   if (n > 64u) return -1;
   // Sorted by (x, y), the smallest index of equal points only.
   __shared__ u32 s_keep[2];
-  const u64 v = t < (int)n ? lex(P[t]) : 0ull;
+  const u64 v = t < (int)n ? lex_key(P[t]) : 0ull;
   bool keep = t < (int)n;
-  for (u32 j = 0; j < n && j < (u32)t && keep; ++j) keep = lex(P[j]) != v;
+  for (u32 j = 0; j < n && keep; ++j) keep = lex_key(P[j]) != v || id(j) >= id(t);
   const u32 km = __ballot_sync(0xFFFFFFFFu, keep);
   if (t < 64 && (t & 31) == 0) s_keep[t >> 5] = km;
   __syncthreads();
   u32 r = 0;
   if (keep)
-    for (u32 j = 0; j < n; ++j) r += ((s_keep[j >> 5] >> (j & 31u)) & 1u) && lex(P[j]) < v ? 1u : 0u;
+    for (u32 j = 0; j < n; ++j) r += ((s_keep[j >> 5] >> (j & 31u)) & 1u) && lex_key(P[j]) < v ? 1u : 0u;
   if (keep) S.ta[r] = (unsigned short)t;
   const int m = __syncthreads_count(keep);
   if (t == 0) {
@@ -1093,10 +1191,18 @@ __device__ int rest_hull(L& S, const int2* __restrict__ P, u32 n, int* out, long
     --k;                                 // the first point again
     S.flag = (u32)k;
     if (k <= cap)
-      for (int i = 0; i < k; ++i) out[i] = (int)S.tb[i];
+      for (int i = 0; i < k; ++i) out[i] = (int)id(S.tb[i]);
   }
   __syncthreads();
   return (int)S.flag;
+}
+
+// rest_hull of the q points of a list in global memory, out of line too.
+template <int BLOCK, class L>
+__device__ __noinline__ int rest_of_list(L& S, const int2* xy, const u32* idx, u32 q, int* out, long long cap) {
+  for (u32 i = threadIdx.x; i < q; i += BLOCK) { S.p[i] = xy[i]; S.id[i] = idx[i]; }
+  __syncthreads();
+  return rest_hull<BLOCK>(S, S.p, S.id, q, out, cap);
 }
 
 }  // namespace star
