@@ -441,8 +441,8 @@ hull_status run_front(hull_ctx* c, const int32_t* d_xy, u32 n, cudaStream_t st, 
     // chosen extremes and the quadrilateral's corners, unless the gate finds
     // the quadrilateral already discarding nearly all of a sample.  Not on
     // the single-read front: there the filter polygon only meets the raw
-    // survivors of the sample polygon (32 directions) after the witness
-    // test, and a larger polygon cannot pay for its features and inference.
+    // survivors of the sample polygon after the witness test, and a larger
+    // polygon cannot pay for its features and inference.
     e = launch_propose(d_xy, n, c->W16, c->feat, c->ext, c->ext_xy, c->plan, st);
     if (e != cudaSuccess) return cuda_fail(e);
   }

@@ -101,12 +101,13 @@ struct ExtPartial {
 // The single-read front's tables (k0_poly.cu builds the frame and the sample
 // polygon, k1_poly filters with them, k_star.cu finishes; star.cuh has the
 // device code).  The first part is cleared before every call.
-constexpr int kPolyDirs = 64;          // directions of the sample's extreme points
+constexpr int kPolyDirs = 64;          // angular sectors of the sample's candidates
 constexpr int kPolySlabs = 8192;       // most x slabs of the polygon's table
 constexpr int kStarBins = 2048;        // angular bins of the candidates
 constexpr u32 kStarCap = 8192;         // most points that one block finishes
-// An interior input point c and the whitening map u = m00 dx, v = m10 dx +
-// m11 dy of d = p - c.
+// A point c (the mean of a sample, rounded: not necessarily of the input, nor
+// known to lie inside the hull before the result verifies about it) and the
+// whitening map u = m00 dx, v = m10 dx + m11 dy of d = p - c.
 struct StarFrame {
   int cx, cy;
   float m00, m10, m11;
@@ -127,14 +128,12 @@ struct PolyLine {
 };
 struct PolyTab {
   // cleared per call
-  u64 best[kPolyDirs];   // per direction: (ordered projection << 32 | ~sample index), maximum
+  u64 best[kPolyDirs];   // per sector: the sample's candidate (star::cand_key: whitened radius, ~position), maximum
   u64 key[kStarBins];    // per angular bin: the raw survivors' candidate (star::cand_key), maximum
   u32 raw_count;         // K1's survivors: points on or outside the polygon
   u32 done;              // last-block counter of k0
   u32 list_count;        // points left by the candidates
-  u32 done2;             // last-block counter of k_star
-  u32 error;             // ERR_RANGE from K1
-  u32 pad[3];
+  u32 error;             // ERR_RANGE, ERR_TIMEOUT from K1
   // written by k0
   StarFrame frame;
   PolyHead head;

@@ -15,9 +15,10 @@
 // counts those: what the bucket sort and the chain merges did in eight
 // launches over the same few thousand points is one block's shared memory
 // here (k_star 22-27 us for 20M points under the profiler, 14-17 for 100k,
-// against 115-130 us of kernels before).  A list beyond kStarCap, a crowded
-// bin or a degenerate input sets ERR_RETRY: the call goes on with the sectors
-// (k_sector.cu) or the bucket sort.
+// against 115-130 us of kernels before).  An input on one line or on one point
+// is decided here too.  A list beyond kStarCap, a crowded bin or an input
+// without a polygon for another reason sets ERR_RETRY: the call goes on with
+// the sectors (k_sector.cu) or the bucket sort.
 #include "hull_internal.cuh"
 #include "kernels.h"
 #include "star.cuh"
@@ -54,8 +55,8 @@ struct SmallSmem {
   u32 count, error;
 };
 
-// No polygon: a degenerate input (1); too many raw survivors for one block
-// (2): the star path leaves both to others.
+// No polygon: a degenerate input (1; k_star tries the line); too many raw
+// survivors for one block (2).
 __device__ __forceinline__ int not_here(const PolyTab* T, u32 q, u32 n) {
   return !T->head.ok ? 1 : q > many_raw(n) ? 2 : 0;
 }
