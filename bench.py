@@ -403,11 +403,13 @@ def _time_hulls(ctx, sctx, t, out, stream, torch, k):
 
 
 def bench_radix_fallback(hull, torch, stream, k=10):
-    """The cost of the radix-pass rerun: 4M points drawn from 40 distinct
-    points (coordinates in [-1000, 1000), seed 9), whose duplicates fill a
-    bin the bucket sort cannot split, so the call is rerun on the radix
-    passes; beside it a 4M uniform disk (seed 12) that the bucket sort takes
-    itself.  ms per hull (one call per step) and whether the rerun ran."""
+    """Heavy duplicates: 4M points drawn from 40 distinct points (coordinates
+    in [-1000, 1000), seed 9), beside a 4M uniform disk (seed 12).  Per input
+    the call as it is (the star path, whose pass drops the copies) and the
+    paper's steps (a context with statistics), where the duplicates fill a bin
+    that the bucket sort cannot split and the call is rerun on the radix
+    passes: ms per hull (one call per step) and whether the rerun ran in the
+    timed calls."""
     from paper_1508_05931_gb300 import workloads as W
     rng = np.random.default_rng(9)
     few = rng.integers(-1000, 1000, size=(40, 2)).astype(np.int32)
@@ -417,13 +419,15 @@ def bench_radix_fallback(hull, torch, stream, k=10):
     for name, pts in cases:
         t = torch.as_tensor(np.ascontiguousarray(pts)).cuda()
         o = torch.empty(t.shape[0], dtype=torch.int32, device="cuda")
-        with hull.Context(torch.cuda.current_device()) as c:
-            ms = _ms_per_hull(c, t, o, stream, torch, k)
-        with hull.Context(torch.cuda.current_device(), collect_stats=True) as c:
-            c.compute_raw(t, o, stream)
-            fb = c.last_stats()["sort_fallback"]
-        res[name] = {"ms_per_hull": ms, "sort_fallback": int(fb), "n": int(len(pts))}
-    res["rerun_over_disk"] = res["duplicates_4M"]["ms_per_hull"] / res["disk_4M"]["ms_per_hull"]
+        res[name] = {"n": int(len(pts))}
+        for path, stats in (("call", False), ("paper_steps", True)):
+            with hull.Context(torch.cuda.current_device(), collect_stats=stats) as c:
+                ms = _ms_per_hull(c, t, o, stream, torch, k)
+                c.set_profiling(True)
+                c.compute_raw(t, o, stream)
+                res[name][path] = {"ms_per_hull": ms, "sort_fallback": int(c.profile()["radix_calls"] > 0)}
+    res["rerun_over_disk"] = (res["duplicates_4M"]["paper_steps"]["ms_per_hull"]
+                              / res["disk_4M"]["paper_steps"]["ms_per_hull"])
     return res
 
 
