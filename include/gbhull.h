@@ -256,7 +256,10 @@ typedef struct {
                                     (single-read front: the sample polygon; empty on the
                                     two-read front), extremes (single-read front: the
                                     pass that filters with the polygon; the star path's hull
-                                    is then in `final`, the slots between empty), witnesses (the
+                                    is then in `final`, the slots between empty; what goes on
+                                    from the raw survivors keeps these two, with the attempt's
+                                    time in `final` (sectors) or `witnesses` (the paper's
+                                    steps)), witnesses (the
                                     sample's best witness per bin), filter (the
                                     fused filter: witness test, filter polygon, compaction, bin
                                     scan), scatter (survivors into coarse bins), split (coarse bins

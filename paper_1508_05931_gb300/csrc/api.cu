@@ -426,9 +426,10 @@ hull_status run_front(hull_ctx* c, const int32_t* d_xy, u32 n, cudaStream_t st, 
   Workspace& w = c->ws;
   const size_t clear_bytes = (reinterpret_cast<char*>(w.wkey) - reinterpret_cast<char*>(w.bcnt)) +
                              (size_t)2 * kWitnessBins * sizeof(u64);
-  mark(c, 0, st);
+  // Behind the star path's front its stages stay as they were marked.
+  if (!single) mark(c, 0, st);
   cudaError_t e = cudaSuccess;
-  if (bucket) mark(c, 1, st);       // the sample polygon's slot: an empty stage
+  if (bucket && !single) mark(c, 1, st);       // the sample polygon's slot: an empty stage
   if (single)
     e = launch_k1_raw(w.h_xy[0], reinterpret_cast<const u32*>(w.h_idx[0]), n, c->cfg.spin_limit, c->plan, w.partials,
                       w.poly, c->num_sms, st);
@@ -446,7 +447,7 @@ hull_status run_front(hull_ctx* c, const int32_t* d_xy, u32 n, cudaStream_t st, 
     e = launch_propose(d_xy, n, c->W16, c->feat, c->ext, c->ext_xy, c->plan, st);
     if (e != cudaSuccess) return cuda_fail(e);
   }
-  mark(c, bucket ? 2 : 1, st);
+  if (!single) mark(c, bucket ? 2 : 1, st);
   const size_t t2 = (n + k2_tile() - 1) / k2_tile();
   if (bucket) {
     // The fused front: witnesses from a sample, then one pass that filters,
@@ -571,11 +572,13 @@ hull_status compute_from(hull_ctx* c, const int32_t* d_xy, u32 n, int32_t* d_out
       r = run_star(c, d_xy, n, d_out, cap, c->h_plan, st);
     } else if (from == FROM_FRONT || from == FROM_SECTORS) {
       // bound: the raw survivors' number where the host knows it.
-      mark(c, 0, st);
       cudaError_t e = cudaSuccess;
-      if (from == FROM_FRONT) { e = star_front(c, d_xy, n, st); bound = n; }
-      else mark(c, 1, st);
-      for (int p = 2; p <= 3 + kMaxPasses; ++p) mark(c, p, st);
+      if (from == FROM_FRONT) {
+        mark(c, 0, st);
+        e = star_front(c, d_xy, n, st);
+        bound = n;
+        for (int p = 2; p <= 3 + kMaxPasses; ++p) mark(c, p, st);
+      }
       if (e == cudaSuccess)
         e = launch_sectors(n, bound, w.poly, w.sect, w.h_xy[0], reinterpret_cast<u32*>(w.h_idx[0]), w.h_xy[1],
                            reinterpret_cast<u32*>(w.h_idx[1]), c->h_plan, d_out, (long long)cap, c->num_sms, st);
