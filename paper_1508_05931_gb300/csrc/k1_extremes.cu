@@ -310,10 +310,12 @@ k1_extremes(const int* __restrict__ xy, u32 n, u32 spin_limit, Plan* plan,
 // the polygon's columns, one 4-byte table word (8-byte words took two
 // shared-memory passes per warp).  Every warp streams its own ring of bulk
 // copies, tests eight points a lane and votes once; survivors are well below
-// one in a hundred of ordinary inputs.  20M square / disk, launch included:
-// 34 / 36 us with one block of 16 warps and rings of 256-point chunks; 41 with
-// two blocks on register double buffers; 37 with 32 warps, 38 / 41 with two
-// blocks of smaller rings; 43 for the eight-byte table with a scan per round.  An input that starts on an odd row
+// one in a hundred of ordinary inputs.  20M points take 30-33 us on the device
+// (gpu__time_duration of a launch; 160 MB, 4.9-5.3 TB/s).  Between two events,
+// launch included, square / disk: 34 / 36 us with one block of 16 warps and
+// rings of 256-point chunks; 41 with two blocks on register double buffers; 37
+// with 32 warps, 38 / 41 with two blocks of smaller rings; 43 for the
+// eight-byte table with a scan per round.  An input that starts on an odd row
 // (8-byte aligned) gives its first point to one lane and streams the rest.
 constexpr int K1P_BLOCK = 512;
 constexpr int K1P_WARPS = K1P_BLOCK / 32;
