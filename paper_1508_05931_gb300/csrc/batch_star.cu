@@ -129,7 +129,7 @@ kb_small(BatchStar a) {
       dirs = H.ok != 0;
       if (dirs) star::bin_normals<BS_BLOCK, BF_NB>(S.poly, F, S.list.dirs());
       __syncthreads();
-      star::ListSink<false, decltype(S.list)> sink{&S.list, &S.count, (u32)BF_CAP, false, nullptr, nullptr};
+      star::ListSink<decltype(S.list)> sink{&S.list, &S.count, (u32)BF_CAP, false};
       star::stream_points<4>(P, n, 0u, (u32)wid, (u32)(BS_BLOCK / 32), H, S.tab, sink, [] {});
       bad = sink.bad;
       flat = !H.ok;

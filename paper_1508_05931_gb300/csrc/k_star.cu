@@ -192,8 +192,7 @@ k_small(const int2* __restrict__ P, u32 n, Plan* plan, int* out, long long cap) 
     __syncthreads();
     if (t < kPolyDirs) {
       const u32 i = ~(u32)S.best[t];
-      S.poly.id[t] = i < NS ? (u32)star::sample_at(i, stride) : 0xFFFFFFFFu;
-      S.poly.p[t] = i < NS ? P[S.poly.id[t]] : make_int2(0, 0);
+      S.poly.p[t] = i < NS ? P[star::sample_at(i, stride)] : make_int2(0, 0);
       const u32 h = __ballot_sync(0xFFFFFFFFu, i < NS);
       if (lane == 0) S.poly.has[wid] = h;
     }
@@ -202,7 +201,7 @@ k_small(const int2* __restrict__ P, u32 n, Plan* plan, int* out, long long cap) 
     dirs = H.ok != 0;
     if (dirs) star::bin_normals<KS_BLOCK, kStarBins>(S.poly, F, S.list.dirs());
     __syncthreads();
-    star::ListSink<true, decltype(S.list)> sink{&S.list, &S.count, (u32)KS_CAP, false, &S.poly, &F};
+    star::ListSink<decltype(S.list)> sink{&S.list, &S.count, (u32)KS_CAP, false};
     star::stream_points<4>(P, n, 0u, (u32)wid, (u32)(KS_BLOCK / 32), H, S.tab, sink, [] {});
     bad = sink.bad;
     flat = !H.ok;

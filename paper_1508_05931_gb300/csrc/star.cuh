@@ -195,7 +195,6 @@ __device__ __forceinline__ void offer_sample(const StarFrame& F, int2 p, u32 pos
 
 struct PolySmem {
   int2 p[kPolyDirs];                    // candidates by sector
-  u32 id[kPolyDirs];                    // their input indices, for a ListSink (none: 0xFFFFFFFF)
   u32 has[2];                           // sectors with one
   int hx[kPolyDirs + 2], hy[kPolyDirs + 2];
   float slope[kPolyDirs + 2];
@@ -735,26 +734,13 @@ __device__ __forceinline__ void stream_ring(Ring<STAGES, CH>& ring, const int2* 
 }
 
 // The stream's sink of a block that finishes its points itself: its list.
-// DUPS: a duplicate of its sector's candidate with a larger index goes no
-// further, as in RawSink (60,000 points of 40 distinct ones overflowed k_small's
-// list and went on to the sectors and the bucket sort: 305 us, 77 with it).  Not
-// in the batch's blocks: there it took kb_small from 109 to 120 us of a batch.
-template <bool DUPS, class L>
+template <class L>
 struct ListSink {
   L* list;
   u32* count;
   u32 cap;
   bool bad;                 // a coordinate out of range
-  const PolySmem* poly;
-  const StarFrame* frame;
   __device__ __forceinline__ void push(bool out, int x, int y, u32 id) {
-    if (DUPS && out) {
-      float u, v;
-      to_uv(*frame, x - frame->cx, y - frame->cy, u, v);
-      const u32 s = bin_of<kPolyDirs>(u, v);
-      const int2 w = poly->p[s];
-      out = !(w.x == x && w.y == y && id > poly->id[s]);
-    }
     const u32 bal = __ballot_sync(0xFFFFFFFFu, out);
     if (bal) {
       const int lane = threadIdx.x & 31;
