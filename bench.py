@@ -272,12 +272,12 @@ def bench_batched(hull, torch, stream, plain_value, args):
             tuned = {k.split("|")[-1]: v_ for k, v_ in json.load(f).items()}
     except (OSError, ValueError):
         pass
-    seg_min = tuned.get("batched_seg_min")
-    paths = None
-    if seg_min:
-        seg = sizes >= seg_min
-        paths = {"segmented": {"instances": int(seg.sum()), "points": int(sizes[seg].sum())},
-                 "one_block": {"instances": int((~seg).sum()), "points": int(sizes[~seg].sum())}}
+    # How the star path divides the batch (hull_compute_batched): one block per
+    # small instance, the others through the pass.  `autotuned` is about the
+    # general path, for what the star path leaves undecided.
+    large = sizes > 16384
+    paths = {"pass": {"instances": int(large.sum()), "points": int(sizes[large].sum())},
+             "one_block": {"instances": int((~large).sum()), "points": int(sizes[~large].sum())}}
     return {"value": v, "unit": "Mpoints/s", "ms_per_batch": ms, "instances": len(offs) - 1,
             "points": int(len(pts)), "hull_vertices": int(oo[-1].item()), "steps": k,
             "vs_plain": v / plain_value, "autotuned": tuned, "paths": paths,
